@@ -128,7 +128,7 @@ void launch_fill_list(const Topo& t, const Phys& p, const Pool& pool, int cur, c
 // ---------------------------------------------------------------- RHS + RK (FP64)
 void launch_rhs_rk_f64(const Topo& t, const Phys& p, const Pool& pool, int cur, int stage, const double* dt,
                        double* rhs_out, cudaStream_t st, int level) {
-  launch_rhs_rk_impl<double>(t, p, pool, cur, stage, dt, rhs_out, st, level);
+  launch_rhs_rk_impl(t, p, pool, cur, stage, dt, rhs_out, st, level);
 }
 
 // ---------------------------------------------------------------- face fluxes of internal nodes
@@ -405,11 +405,12 @@ __global__ void __launch_bounds__(256) k_cfl(Topo t, Phys p, Pool pool, int cur,
       double Uc[5];
 #pragma unroll
       for (int v = 0; v < 5; ++v) Uc[v] = U[v * NCELL + s];
-      Prim<double> q = prim_of<double>(Uc, p.gamma, p.B);
-      if (!(q.rho > 0.0) || !(q.p + p.B > 0.0)) bad = true;
+      const Div64 rho = div64_prep(Uc[0]);
+      const Prim64 q = prim64(Uc, p.gamma, p.B, rho);
+      if (!pos64(Uc[0]) || !pos64(q.p + p.B)) bad = true;
 #pragma unroll
       for (int d = 0; d < 3; ++d) m[d] = fmax(m[d], fabs(q.vel[d]) + q.c);
-      if (p.mu > 0.0) m[3] = fmax(m[3], 1.0 / q.rho);
+      if (p.mu > 0.0) m[3] = fmax(m[3], div64(1.0, rho));
     }
     if (bad) atomicExch(status, (int)ST_NONPHYS);
     block_max<4>(m, sh);

@@ -1,184 +1,234 @@
-// Fused right-hand side + Runge-Kutta stage kernel of the FP64 path (Sec. 2.2
-// and Alg. ComputeLoop of arXiv:2012.04385, with the Shu-Osher TVD-RK3 or
-// TVD-RK2 stages); every reconstruction, flux scheme and the viscous terms
-// are run-time choices here.
+// Right-hand side and Runge-Kutta stage of the FP64 path (Sec. 2.2 and Alg.
+// ComputeLoop of arXiv:2012.04385, with the Shu-Osher TVD-RK3 or TVD-RK2
+// stages); every reconstruction, flux scheme and the viscous terms are run-time
+// choices here.
 //
-// One CTA works on one z-slab (16 x 16 x TZ internal cells) of one leaf block
-// at a time, looping over (leaf, slab) items.  For each direction it computes
-// every face flux of the slab (17 faces per pencil; threads walk the faces
-// linearly so neighbouring threads read neighbouring cells), keeps them in
-// shared memory, and each thread accumulates the flux differences of the
-// cells of its (i, j) column.  The stage update then reads u^(s) and u^n and
-// writes u^(s+1) into the other stage buffer.  Boundary-face fluxes go to the
-// block's face buffers for the jump correction.
+// Two kernels.  k_flux_f64 works on items of 32 pencils (rows of 16 cells of one
+// leaf along one direction, with three cells of halo at each end): the cell
+// quantities of the 22 x 32 cells go to shared memory, one warp computes the 32
+// fluxes of one face plane, and the flux differences of the 16 x 32 cells go to
+// global memory (boundary-face fluxes also to the block's face buffers for the
+// jump correction).  k_update_f64 adds the three directions' differences in the
+// order x, y, z and forms the stage.
+//
+// The path is bound by the FP64 pipe, at less than 1% of its memory traffic's
+// time, so the split follows the FP64 work: no face and no cell quantity of a
+// direction is computed twice (z-slabs shared 17 planes per 16 in x and y but
+// five per four in z, and formed every cell's primitives for each of the six
+// faces that read it), and 24 or 48 items per leaf occupy the GPU from eight
+// leaves on, where four slabs per leaf left 120 of 152 SMs idle.
+//
+// Uniform data.  A warp whose 32 stencils hold six equal cells takes the flat
+// form of the flux (one projection instead of six, constant WENO weights), and
+// in an item of constant pencils one face plane stands for all 17.  Both give
+// the same bits as the general form; cells are compared bit for bit.
+//
+// Measured (GB300; flux and update kernels together, before: one kernel per
+// z-slab with compiler divisions): shock-bubble on levels 0..2, 316 leaves,
+// 27.1 ms -> 7.6 ms per stage; TENO5 and LLF on 60 periodic leaves without
+// uniform data 5.34 ms -> 2.33 ms; Sod tube on 8 leaves 2.78 ms -> 0.25 ms.  The
+// FP64 pipe is 77% busy, with 14% of the issue slots used.
+//
+// Scratch.  The differences live in the stage buffer that the stage is about to
+// write: those of x at the cells themselves, those of y and z in its halo,
+// which the next halo fill rewrites.
 #pragma once
 
 #include "kernels.cuh"
 
 namespace mrb {
 
-constexpr int RHS_TZ = 4;
-constexpr int RHS_NSLAB = NB / RHS_TZ;
-constexpr int RHS_FMAX = NB * NB * (RHS_TZ + 1);   // >= 17 * 16 * RHS_TZ
-constexpr int RHS_THREADS = 256;
+constexpr int F64_P = 32;                     // pencils per item (16 on small trees)
+constexpr int F64_L = NB + 6;                 // cells per pencil
+constexpr int F64_WARPS = 8;                  // two CTAs and 128 registers a thread per SM
+constexpr int F64_THREADS = 32 * F64_WARPS;
+constexpr size_t F64_SMEM = sizeof(double) * (CQ_N * F64_L * F64_P + NV * (NB + 1) * F64_P);
 
-
-// Faces of one direction D of the slab starting at z0: fluxes into Fs, boundary
-// faces into the face buffers, then the flux differences into acc.
-template <class R, int D>
-__device__ __forceinline__ void rhs_dir(const double* __restrict__ u, double* __restrict__ fb, R* Fs, int z0, R g,
-                                        R B, int lin, int flux, double mu, double dx,
-                                        double (&acc)[RHS_TZ][NV]) {
-  const int ti = threadIdx.x & 15, tj = threadIdx.x >> 4;
-  constexpr int nf = (D == 2) ? NB * NB * (RHS_TZ + 1) : (NB + 1) * NB * RHS_TZ;
-  constexpr int stride = (D == 0) ? 1 : (D == 1 ? NS : NS * NS);
-  for (int f = threadIdx.x; f < nf; f += blockDim.x) {
-    int ci, cj, ck, fa;
-    if (D == 0) {
-      fa = f % 17;
-      int r = f / 17;
-      cj = r % 16;
-      ck = z0 + r / 16;
-      ci = fa - 3;
-    } else if (D == 1) {
-      ci = f % 16;
-      int r = f / 16;
-      fa = r % 17;
-      ck = z0 + r / 17;
-      cj = fa - 3;
-    } else {
-      ci = f % 16;
-      int r = f / 16;
-      cj = r % 16;
-      fa = r / 16;
-      ck = z0 + fa - 3;
-    }
-    const int base = sidx(ci, cj, ck);
-    R U6[6][5];
-#pragma unroll
-    for (int m = 0; m < 6; ++m)
-#pragma unroll
-      for (int v = 0; v < 5; ++v) U6[m][v] = R(u[v * NCELL + base + m * stride]);
-    R F[5];
-    face_flux<R>(U6, D, g, B, lin, flux, F);
-    if (mu > 0.0) {
-      // Navier-Stokes: F(U) - F_v at the face between stencil cells 2 and 3
-      double Fv[5];
-      viscous_flux(u, D, base + 2 * stride, mu, dx, Fv);
-#pragma unroll
-      for (int v = 0; v < 5; ++v) F[v] = R(double(F[v]) - Fv[v]);
-    }
-#pragma unroll
-    for (int v = 0; v < 5; ++v) Fs[v * RHS_FMAX + f] = F[v];
-    const int gface = (D == 2) ? z0 + fa : fa;
-    if (gface == 0 || gface == NB) {
-      const int side = 2 * D + (gface == NB ? 1 : 0);
-      int ta, tb;
-      if (D == 0) { ta = cj; tb = ck; }
-      else if (D == 1) { ta = ci; tb = ck; }
-      else { ta = ci; tb = cj; }
-#pragma unroll
-      for (int v = 0; v < 5; ++v) fb[((side * NV + v) * NB + tb) * NB + ta] = double(F[v]);
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int kz = 0; kz < RHS_TZ; ++kz) {
-    int lo, hi;
-    if (D == 0) { lo = (kz * 16 + tj) * 17 + ti; hi = lo + 1; }
-    else if (D == 1) { lo = (kz * 17 + tj) * 16 + ti; hi = lo + 16; }
-    else { lo = (kz * 16 + tj) * 16 + ti; hi = lo + 256; }
-#pragma unroll
-    for (int v = 0; v < 5; ++v) {
-      double diff = double(Fs[v * RHS_FMAX + lo]) - double(Fs[v * RHS_FMAX + hi]);
-      acc[kz][v] = (D == 0) ? diff : acc[kz][v] + diff;
-    }
-  }
-  __syncthreads();
+// Place of the differences of direction d at cell c (x fastest) in a stage
+// buffer, for every variable: x at the cell, y in the 8 x 576 cells of the z
+// halo planes, z in the x and y halo of the plane z (192 cells of the eight
+// y-halo rows and 64 of the x halo).
+__device__ __forceinline__ int diff_place(int d, int c) {
+  const int k = c >> 8, q = c & 255;
+  if (d == 0) return sidx(q & 15, q >> 4, k);
+  if (d == 1) return c < 2048 ? c : (NS - HW) * NS * NS + c - 2048;
+  const int in = q < 96 ? q : (q < 192 ? NS * (NS - HW) + q - 96 : (HW + ((q - 192) >> 2)) * NS + (q & 3));
+  return (k + HW) * NS * NS + in;
 }
 
-template <class R>
-__global__ void __launch_bounds__(RHS_THREADS) k_rhs_rk(Topo t, Phys p, Pool pool, int cur, int stage,
-                                                       const double* __restrict__ dt, double* __restrict__ rhs_out,
-                                                       int level) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  R* Fs = reinterpret_cast<R*>(smem_raw);
-  const int nitems = stage_nodes(t, level) * RHS_NSLAB;
+// Lane p of plane i along direction d, pencil number pp of the block.
+__device__ __forceinline__ void pencil_cell(int d, int pp, int i, int& x, int& y, int& z) {
+  const int a = pp & 15, b = pp >> 4;
+  x = d == 0 ? i : a;
+  y = d == 0 ? a : (d == 1 ? i : b);
+  z = d == 2 ? i : b;
+}
+
+// Items are (leaf, direction, P pencils); a warp takes 32/P face planes at a
+// time.  P = 32, or 16 while the items of 32 pencils would not give every SM
+// two (Sod tube of eight leaves: the 64 items along x carry nearly all of the
+// work).
+static __global__ void __launch_bounds__(F64_THREADS, 2)
+    k_flux_f64(Topo t, Phys p, Pool pool, int cur, int level) {
+  extern __shared__ __align__(16) double f64_smem[];
+  double* cq = f64_smem;
+  double* fl = cq + CQ_N * F64_L * F64_P;
+  __shared__ unsigned eqm[F64_L - 1];         // bit l: cells i and i + 1 of pencil l are equal
+  const int nodes = stage_nodes(t, level);
+  const int lp = (nodes * (3 * NFACE / F64_P) < (int)gridDim.x) ? 4 : 5;
+  const int P = 1 << lp, per_dir = NFACE >> lp, per_leaf = 3 * per_dir, QS = F64_L << lp;
   const double* __restrict__ src = pool.bufp(cur);
   double* __restrict__ dst = pool.bufp(cur ^ 1);
-  const R g = R(p.gamma), B = R(p.B);
-  const int lin = p.recon;   // reconstruction mode: 0 WENO5, 2 linear, 3 TENO5, 4 WENO-AO(5,3)
-  const int flux = p.flux;   // FLUX_ROE, FLUX_LLF or FLUX_HLLC
-  const int ti = threadIdx.x & 15, tj = threadIdx.x >> 4;
-  const ItemRange IR = item_range(nitems, p.blocked);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int pl = lane & (P - 1), sub = lane >> lp, nsub = 32 >> lp;      // pencil, and which of the warp's planes
+  const unsigned full = P == 32 ? 0xffffffffu : 0xffffu;
+  const ItemRange IR = item_range(nodes * per_leaf, p.blocked);
   for (int w = IR.first; w < IR.end; w += IR.step) {
-    const int li = w / RHS_NSLAB, z0 = (w % RHS_NSLAB) * RHS_TZ;
-    const int node = stage_node(t, level, li);
+    const int node = stage_node(t, level, w / per_leaf);
+    const int D = (w % per_leaf) / per_dir, pp = ((w % per_dir) << lp) + pl;
     const int slot = t.slot[node];
     const double* __restrict__ u = src + (size_t)slot * SLOT_U;
-    double* __restrict__ fb = pool.face + (size_t)slot * SLOT_F;
-    double acc[RHS_TZ][NV];
-    const double dxn = ldexp(p.dx0, -t.level[node]);
-    rhs_dir<R, 0>(u, fb, Fs, z0, g, B, lin, flux, p.mu, dxn, acc);
-    rhs_dir<R, 1>(u, fb, Fs, z0, g, B, lin, flux, p.mu, dxn, acc);
-    rhs_dir<R, 2>(u, fb, Fs, z0, g, B, lin, flux, p.mu, dxn, acc);
-    const int inst = t.inst[node];
-    const double dx = ldexp(p.dx0, -t.level[node]);
-    const double h = dt ? node_dt(t, p, dt, node, level) : 0.0;
-    (void)inst;
+    for (int i = warp * nsub + sub; i < F64_L; i += F64_WARPS * nsub) {
+      int x, y, z;
+      pencil_cell(D, pp, i - 3, x, y, z);
+      const int s = sidx(x, y, z);
 #pragma unroll
-    for (int kz = 0; kz < RHS_TZ; ++kz) {
-      const int k = z0 + kz;
-      const int s = sidx(ti, tj, k), ii = iidx(ti, tj, k);
-      double L[5];
-#pragma unroll
-      for (int v = 0; v < 5; ++v) L[v] = acc[kz][v] / dx;
-      if (p.has_grav) {
-        double rho = u[s], mx = u[NCELL + s], my = u[2 * NCELL + s], mz = u[3 * NCELL + s];
-        L[1] = L[1] + rho * p.grav[0];
-        L[2] = L[2] + rho * p.grav[1];
-        L[3] = L[3] + rho * p.grav[2];
-        L[4] = L[4] + ((mx * p.grav[0] + my * p.grav[1]) + mz * p.grav[2]);
+      for (int v = 0; v < NV; ++v) {
+        const int q = (v == 0 || v == 4) ? v : 1 + (v + 2 - D) % 3;      // lab component v - 1 in the direction frame
+        cq[q * QS + (i << lp) + pl] = u[v * NCELL + s];
       }
-      if (rhs_out) {
+    }
+    __syncthreads();
+    for (int i = warp; i < F64_L - 1; i += F64_WARPS) {
+      bool eq = true;
 #pragma unroll
-        for (int v = 0; v < 5; ++v) rhs_out[((size_t)li * NV + v) * NINT + ii] = L[v];
+      for (int v = 0; v < NV; ++v)
+        eq = eq && d2bits(cq[v * QS + (i << lp) + pl]) == d2bits(cq[v * QS + ((i + 1) << lp) + pl]);
+      const unsigned m = __ballot_sync(0xffffffffu, eq);
+      if (lane == 0) eqm[i] = m & full;
+    }
+    __syncthreads();
+    unsigned all = full;
+#pragma unroll
+    for (int i = 0; i < F64_L - 1; ++i) all &= eqm[i];
+    // every pencil constant: its first face stands for all (not with viscous
+    // terms, whose gradients read other pencils)
+    const bool uniform = all == full && !(p.mu > 0.0);
+    for (int i = warp * nsub + sub; i < (uniform ? 1 : F64_L); i += F64_WARPS * nsub)
+      flux64_cell(D, p.gamma, p.B, cq + (i << lp) + pl, QS);
+    __syncthreads();
+    const int nplane = uniform ? 1 : NB + 1;
+    for (int f0 = warp * nsub; f0 < nplane; f0 += F64_WARPS * nsub) {
+      const int fa = f0 + sub < nplane ? f0 + sub : f0;                  // (the last warp's spare lanes repeat its first plane)
+      const Row64 r{cq + (fa << lp) + pl, QS, P};
+      const unsigned m = eqm[fa] & eqm[fa + 1] & eqm[fa + 2] & eqm[fa + 3] & eqm[fa + 4];
+      double F[5];
+      if (__all_sync(0xffffffffu, (m >> pl) & 1u)) face_flux64<true>(r, p.gamma, p.B, p.recon, p.flux, F);
+      else face_flux64<false>(r, p.gamma, p.B, p.recon, p.flux, F);
+      if (p.mu > 0.0) {
+        // Navier-Stokes: F(U) - F_v at the face between stencil cells 2 and 3
+        int x, y, z;
+        pencil_cell(D, pp, fa - 1, x, y, z);
+        const double dx = ldexp(p.dx0, -t.level[node]);
+        double Fv[5];
+        viscous_flux(u, D, sidx(x, y, z), p.mu, div64_prep(dx), div64_prep(4.0 * dx), Fv);
+        F[0] = F[0] - Fv[0];
+        F[1] = F[1] - (D == 0 ? Fv[1] : (D == 1 ? Fv[2] : Fv[3]));
+        F[2] = F[2] - (D == 0 ? Fv[2] : (D == 1 ? Fv[3] : Fv[1]));
+        F[3] = F[3] - (D == 0 ? Fv[3] : (D == 1 ? Fv[1] : Fv[2]));
+        F[4] = F[4] - Fv[4];
+      }
+#pragma unroll
+      for (int v = 0; v < NV; ++v) fl[((v * (NB + 1) + fa) << lp) + pl] = F[v];
+    }
+    __syncthreads();
+    // flux differences and boundary-face fluxes, lab frame (component j of the
+    // direction frame is axis (D + j) mod 3)
+    double* __restrict__ o = dst + (size_t)slot * SLOT_U;
+    double* __restrict__ fb = pool.face + (size_t)slot * SLOT_F;
+    for (int e = warp * nsub + sub; e < NV * (NB + 2); e += F64_WARPS * nsub) {
+      const int v = e / (NB + 2), i = e % (NB + 2);
+      const int vl = (v == 0 || v == 4) ? v : 1 + (D + v - 1) % 3;
+      const double* f = fl + ((v * (NB + 1)) << lp) + pl;
+      if (i < NB) {
+        int x, y, z;
+        pencil_cell(D, pp, i, x, y, z);
+        o[vl * NCELL + diff_place(D, iidx(x, y, z))] = f[uniform ? 0 : i << lp] - f[uniform ? 0 : (i + 1) << lp];
       } else {
-        double* __restrict__ unb = pool.un + (size_t)slot * SLOT_N;
-        double* __restrict__ o = dst + (size_t)slot * SLOT_U;
+        const int hi = i - NB;
+        fb[((2 * D + hi) * NV + vl) * NFACE + pp] = f[(uniform || !hi) ? 0 : NB << lp];
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// L = ((dF_x + dF_y) + dF_z) / dx + S and the stage out = a u^n + b (u + dt L)
+// (or L itself), one CTA per four planes of a block.  Elementwise: it reads and
+// writes each cell of dst in the same thread, the halo only as scratch.
+static __global__ void __launch_bounds__(256) k_update_f64(Topo t, Phys p, Pool pool, int cur, int stage,
+                                                           const double* __restrict__ dt, double* __restrict__ rhs_out,
+                                                           int level) {
+  const int nitems = stage_nodes(t, level) * 4;
+  const double* __restrict__ src = pool.bufp(cur);
+  double* __restrict__ dst = pool.bufp(cur ^ 1);
+  const double ka = kRkA[rk_row(p)][stage], kb = kRkB[rk_row(p)][stage];
+  for (int w = blockIdx.x; w < nitems; w += gridDim.x) {
+    const int li = w >> 2, node = stage_node(t, level, li), slot = t.slot[node];
+    const double* __restrict__ u = src + (size_t)slot * SLOT_U;
+    double* __restrict__ unb = pool.un + (size_t)slot * SLOT_N;
+    double* __restrict__ o = dst + (size_t)slot * SLOT_U;
+    const Div64 dx = div64_prep(ldexp(p.dx0, -t.level[node]));
+    const double h = dt ? node_dt(t, p, dt, node, level) : 0.0;
+#pragma unroll 1
+    for (int q = 0; q < 4; ++q) {
+      const int c = (w & 3) * 1024 + q * 256 + threadIdx.x;
+      const int s = diff_place(0, c), s1 = diff_place(1, c), s2 = diff_place(2, c);
+      double us[NV], d0[NV], d1[NV], d2[NV], un[NV];
 #pragma unroll
-        for (int v = 0; v < 5; ++v) {
-          const double us = u[v * NCELL + s];
-          double un;
-          if (stage == 0) {
-            un = us;
-            unb[v * NINT + ii] = us;
-          } else {
-            un = unb[v * NINT + ii];
-          }
-          const double tt = us + h * L[v];
-          o[v * NCELL + s] = (stage == 0) ? tt : (kRkA[rk_row(p)][stage] * un + kRkB[rk_row(p)][stage] * tt);
+      for (int v = 0; v < NV; ++v) {
+        us[v] = u[v * NCELL + s];
+        d0[v] = o[v * NCELL + s];
+        d1[v] = o[v * NCELL + s1];
+        d2[v] = o[v * NCELL + s2];
+        un[v] = (stage != 0 && !rhs_out) ? unb[v * NINT + c] : us[v];
+      }
+      double L[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) L[v] = div64((d0[v] + d1[v]) + d2[v], dx);
+      if (p.has_grav) {
+        L[1] = L[1] + us[0] * p.grav[0];
+        L[2] = L[2] + us[0] * p.grav[1];
+        L[3] = L[3] + us[0] * p.grav[2];
+        L[4] = L[4] + ((us[1] * p.grav[0] + us[2] * p.grav[1]) + us[3] * p.grav[2]);
+      }
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        if (rhs_out) {
+          rhs_out[((size_t)li * NV + v) * NINT + c] = L[v];
+        } else {
+          if (stage == 0) unb[v * NINT + c] = us[v];
+          const double tt = us[v] + h * L[v];
+          o[v * NCELL + s] = (stage == 0) ? tt : ka * un[v] + kb * tt;
         }
       }
     }
   }
 }
 
-template <class R>
-void launch_rhs_rk_impl(const Topo& t, const Phys& p, const Pool& pool, int cur, int stage, const double* dt,
-                        double* rhs_out, cudaStream_t st, int level) {
-  const size_t smem = sizeof(R) * NV * RHS_FMAX;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_rhs_rk<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr = true;
+static void launch_rhs_rk_impl(const Topo& t, const Phys& p, const Pool& pool, int cur, int stage, const double* dt,
+                               double* rhs_out, cudaStream_t st, int level) {
+  static int resident = 0;
+  if (resident == 0) {
+    cudaFuncSetAttribute(k_flux_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F64_SMEM);
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_flux_f64, F64_THREADS, F64_SMEM);
+    resident = sm_count() * (per_sm < 1 ? 1 : per_sm);
   }
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rhs_rk<R>, RHS_THREADS, smem);
-  if (per_sm < 1) per_sm = 1;
-  const int grid = sm_count() * per_sm * (g_tune.stage_waves < 1 ? 1 : g_tune.stage_waves);
-  k_rhs_rk<R><<<grid, RHS_THREADS, smem, st>>>(t, p, pool, cur, stage, dt, rhs_out, level);
-  ++g_kernel_launches;
+  const int grid = resident * (g_tune.stage_waves < 1 ? 1 : g_tune.stage_waves);
+  k_flux_f64<<<grid, F64_THREADS, F64_SMEM, st>>>(t, p, pool, cur, level);
+  k_update_f64<<<sm_count() * 8, 256, 0, st>>>(t, p, pool, cur, stage, dt, rhs_out, level);
+  g_kernel_launches += 2;
 }
 
 }  // namespace mrb
