@@ -974,13 +974,136 @@ __device__ __forceinline__ void add_diff(int D, const float* __restrict__ Fs, in
   a[4] += d[4];
 }
 
+// ---- directions along which a slab does not vary
+// Where every pencil of a direction holds 22 (x, y) or 10 (z) bitwise equal
+// records, all its faces have the same flux: the flux differences are exactly
+// zero, and one face per pencil gives the block-boundary fluxes.  Adaptive
+// trees refine blocks, not directions: of the 5,776 leaves of the shock-bubble
+// (levels 0..4) 55% of the slabs are constant along x and 90% along y and z,
+// of the four-quadrant ensemble 70-73% (x, y) and all (z), of the explosion 73%,
+// so most of their face work was spent on zeros.  A few probes decide whether
+// the region is read once more, in 16-byte loads, for the exact test.
+// Measured (stage launch, before -> after): shock-bubble <3> 2.91 -> 2.25 ms and
+// <1> 4.46 -> 3.42 ms, ensemble of five 2.42 -> 1.84 ms, explosion (TENO5, HLLC)
+// 2.06 -> 1.39 ms; data that vary everywhere (210 blocks) 98.7 -> 100.0 us.
+//
+// flat_safe: values whose flux is finite with room to spare (then F - F = 0); a
+// slab with others takes the general path and keeps its infinities and NaN.
+__device__ __forceinline__ bool flat_safe(float r, float p, float E, float B) {
+  return r > 1e-6f && E < 1e12f && p + B > 1e-4f * E;
+}
+// The four records from slot `a` equal those from slot `b` (both multiples of
+// four).
+__device__ __forceinline__ bool same_chunk(const float* __restrict__ S, int a, int b) {
+#pragma unroll 1
+  for (int f = SF_NREC - 1; f >= 0; --f) {
+    const uint4 x = *reinterpret_cast<const uint4*>(S + f * SF_REG + a);
+    const uint4 y = *reinterpret_cast<const uint4*>(S + f * SF_REG + b);
+    if (((x.x ^ y.x) | (x.y ^ y.y) | (x.z ^ y.z) | (x.w ^ y.w)) != 0u) return false;
+  }
+  return true;
+}
+// The four cells from slot a (without the first, or the last) equal the record
+// at slot b.
+__device__ __forceinline__ bool same_cells(const float* __restrict__ S, int a, int b, bool skip_first, bool skip_last) {
+#pragma unroll 1
+  for (int f = SF_NREC - 1; f >= 0; --f) {
+    const uint4 x = *reinterpret_cast<const uint4*>(S + f * SF_REG + a);
+    const unsigned y = __float_as_uint(S[f * SF_REG + b]);
+    const unsigned d0 = skip_first ? 0u : x.x ^ y, d3 = skip_last ? 0u : x.w ^ y;
+    if ((d0 | (x.y ^ y) | (x.z ^ y) | d3) != 0u) return false;
+  }
+  return true;
+}
+__device__ __forceinline__ bool safe_chunk(const float* __restrict__ S, int a, float B) {
+  bool ok = true;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) ok = ok && flat_safe(S[a + c], S[4 * SF_REG + a + c], S[5 * SF_REG + a + c], B);
+  return ok;
+}
+
+// Directions worth testing: the pressure is the same at the ends and in the
+// middle of two rows.  Every thread reads the same few values, so data that
+// vary everywhere cost no vote and no barrier.
+__device__ __forceinline__ bool probe3(const float* __restrict__ p, int a, int b, int c) {
+  return __float_as_uint(p[a]) == __float_as_uint(p[b]) && __float_as_uint(p[a]) == __float_as_uint(p[c]);
+}
+__device__ __forceinline__ unsigned probe_xy(const float* __restrict__ S) {
+  const float* p = S + 4 * SF_REG;
+  const bool fx = probe3(p, xy_slot(-3, 0, 0), xy_slot(7, 0, 0), xy_slot(18, 0, 0)) &&
+                  probe3(p, xy_slot(-3, 11, 2), xy_slot(7, 11, 2), xy_slot(18, 11, 2));
+  const bool fy = probe3(p, xy_slot(0, -3, 0), xy_slot(0, 7, 0), xy_slot(0, 18, 0)) &&
+                  probe3(p, xy_slot(11, -3, 2), xy_slot(11, 7, 2), xy_slot(11, 18, 2));
+  return (fx ? 1u : 0u) | (fy ? 2u : 0u);
+}
+__device__ __forceinline__ unsigned probe_z(const float* __restrict__ S) {
+  const float* p = S + 4 * SF_REG;
+  return probe3(p, 0, 5 * 256, 9 * 256) && probe3(p, 187, 5 * 256 + 187, 9 * 256 + 187) ? 4u : 0u;
+}
+
+// This thread's share of the tests on the x-y region (bit 0: constant along x,
+// bit 1: along y) and on the z region (bit 2).
+__device__ __forceinline__ unsigned flat_xy(const float* __restrict__ S, float B, unsigned which) {
+  bool fx = which & 1u, fy = which & 2u;
+  for (int e = threadIdx.x; e < 16 * SF_TZ * 6 && fx; e += SF_THREADS) {   // rows y in [0, 16), x = -3 .. 18
+    const int r = e / 6, q = e % 6, row = xy_slot(0, r % 16, r / 16);
+    fx = same_cells(S, row + 4 * q - 4, row, q == 0, q == 5) &&
+         flat_safe(S[row], S[4 * SF_REG + row], S[5 * SF_REG + row], B);
+  }
+  for (int e = threadIdx.x; e < 22 * SF_TZ * 4 && fy; e += SF_THREADS) {   // x in [0, 16), y = -3 .. 18
+    const int q = e % 4, r = e / 4, ref = xy_slot(4 * q, 0, r / 22);
+    fy = same_chunk(S, xy_slot(4 * q, r % 22 - 3, r / 22), ref) && safe_chunk(S, ref, B);
+  }
+  return (fx ? 1u : 0u) | (fy ? 2u : 0u);
+}
+__device__ __forceinline__ unsigned flat_z(const float* __restrict__ S, float B) {
+  bool fz = true;
+  for (int e = threadIdx.x; e < (SF_TZ + 6) * 64 && fz; e += SF_THREADS) {
+    const int c = 4 * (e % 64);
+    fz = same_chunk(S, (e / 64) * 256 + c, 3 * 256 + c) && safe_chunk(S, 3 * 256 + c, B);
+  }
+  return fz ? 4u : 0u;
+}
+// The AND of every thread's bits (one barrier; sh: one word per warp).
+__device__ __forceinline__ unsigned block_and(unsigned bits, unsigned* sh) {
+  const unsigned m = __reduce_and_sync(0xffffffffu, bits);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
+  __syncthreads();
+  unsigned all = sh[0];
+#pragma unroll
+  for (int q = 1; q < SF_THREADS / 32; ++q) all &= sh[q];
+  return all;
+}
+// With stored decisions (MODE 3) the faces of a direction must share one.
+__device__ __forceinline__ bool one_decision(const uint32_t* __restrict__ selw, int first, int n) {
+  const uint32_t a = selw[first];
+  return (int)threadIdx.x >= n || ((a == 0u || a == 0xffffffffu) && selw[first + threadIdx.x] == a);
+}
+
+// Flux of a constant pencil on the block's two sides lo and hi of direction D
+// (each optional), lab frame, FP64.
+__device__ __forceinline__ void store_sides(int D, const float F[5], bool lo, bool hi, int ta, int tb,
+                                            double* __restrict__ fb) {
+  float Fl[5];
+  Fl[0] = F[0];
+  Fl[4] = F[4];
+  to_lab(D, F[1], F[2], F[3], Fl[1], Fl[2], Fl[3]);
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    const double x = f2d_fast(Fl[v]);
+    if (lo) fb[((2 * D * NV + v) * NB + tb) * NB + ta] = x;
+    if (hi) fb[(((2 * D + 1) * NV + v) * NB + tb) * NB + ta] = x;
+  }
+}
+
 // Per-direction sweep (the stage-0 selector variant, MODE 1): region of D,
 // faces with WENO5 fluxes and the selector's decisions, flux differences.
 template <int MODE>
 __device__ __forceinline__ void sweep_f32(int D, const Topo& t, const Pool& pool, int cur, int node, int slot,
                                           double* __restrict__ fb, float* __restrict__ S, float* __restrict__ Fs,
                                           int z0, float g, float B, float gm1, float (&acc)[SF_TZ][NV],
-                                          const LearnedCtx& L, unsigned (&cnt)[2]) {   // cnt: the warp's census
+                                          const LearnedCtx& L, unsigned (&cnt)[2],   // cnt: the warp's census
+                                          unsigned& flat, unsigned* flat_sh) {       // constant directions of the slab
   const int ti = threadIdx.x & 15, tj = threadIdx.x >> 4;
   // the x-y region serves the x and the y faces (loaded for D = 0 and kept
   // for D = 1), the z region the z faces
@@ -988,6 +1111,32 @@ __device__ __forceinline__ void sweep_f32(int D, const Topo& t, const Pool& pool
     if (D == 0) load_xy_f32(region_src(t, pool, cur, node, slot), S, z0, g, B, gm1);
     else load_region_f32(2, region_src(t, pool, cur, node, slot), S, z0, g, B, gm1);
     __syncthreads();
+    flat = D == 0 ? probe_xy(S) : probe_z(S);
+    if (flat) flat = block_and(D == 0 ? flat_xy(S, B, flat) : flat_z(S, B), flat_sh);
+  }
+  if ((flat >> D) & 1u) {
+    // constant pencils: every face has all-zero features and the logit z0; the
+    // block-boundary fluxes from one face per pencil, no differences
+    const int nw = region_faces(D) / 32;
+    const bool dl = L.z0 < L.tau;
+    if ((threadIdx.x & 31) == 0) {
+      uint32_t* word = L.bits + (z0 / SF_TZ) * 108 + D * 34;
+      for (int q = threadIdx.x >> 5; q < nw; q += SF_THREADS / 32) {
+        word[q] = dl ? 0xffffffffu : 0u;
+        cnt[0] += dl ? 32u : 0u;
+        cnt[1] += 32u;
+      }
+    }
+    const bool lo = D != 2 || z0 == 0, hi = D != 2 || z0 + SF_TZ == NB;
+    if ((lo || hi) && (D == 2 || threadIdx.x < 16 * SF_TZ)) {
+      const int a = ti, b = tj;      // x: (y, kz), y: (x, kz), z: (x, y)
+      const int c0 = D == 0 ? xy_slot(-3, a, b) : (D == 1 ? xy_slot(a, -3, b) : b * 16 + a);
+      float F[5];
+      face_flux_f32<MODE>(S, c0, sel3i(D, 1, 24, 256), rot_of(D), gm1, g, B, false, F);
+      store_sides(D, F, lo, hi, a, D == 2 ? b : z0 + b, fb);
+    }
+    if (D != 0) __syncthreads();     // the region is free for the next load
+    return;
   }
   const int nf = region_faces(D);
   const int st = sel3i(D, 1, 24, 256);
@@ -1056,29 +1205,43 @@ template <int MODE>
 __device__ __forceinline__ void sweep_xy(const double* __restrict__ u, const Topo& t, const Pool& pool, int cur,
                                          int node, int slot, double* __restrict__ fb, float* __restrict__ S,
                                          float* __restrict__ Fs, int z0, float g, float B, float gm1,
-                                         float (&acc)[SF_TZ][NV], const LearnedCtx& L) {
+                                         float (&acc)[SF_TZ][NV], const LearnedCtx& L, unsigned* flat_sh) {
   const int ti = threadIdx.x & 15, tj = threadIdx.x >> 4;
   load_xy_f32(region_src(t, pool, cur, node, slot), S, z0, g, B, gm1);
   __syncthreads();
-  for (int f = threadIdx.x; f < 2 * SF_NFX; f += blockDim.x) {
+  unsigned flat = 0u;
+  if (!(MODE & 32)) {                     // (viscous fluxes read other pencils)
+    flat = probe_xy(S);
+    if (flat) {
+      flat = flat_xy(S, B, flat);
+      if (MODE == 3) flat &= (one_decision(L.selw, 0, 34) ? 1u : 0u) | (one_decision(L.selw, 34, 34) ? 2u : 0u);
+      flat = block_and(flat, flat_sh);
+    }
+  }
+  // faces of each direction: all of them, or one per constant pencil
+  const bool flatx = flat & 1u, flaty = flat & 2u;
+  const int nx = flatx ? 16 * SF_TZ : SF_NFX, ny = flaty ? 16 * SF_TZ : SF_NFX;
+  for (int f = threadIdx.x; f < nx + ny; f += blockDim.x) {
     float F[5];
-    const bool isx = f < SF_NFX;          // warp-uniform (1088 = 34 warps)
+    const bool isx = f < nx;              // warp-uniform (64 or 1088 = 34 warps)
+    const bool one = isx ? flatx : flaty;
     int fa, c0, ta, tb, st, wi;
     if (isx) {
-      fa = f % 17;
-      const int r = f / 17;               // r = kz * 16 + j
+      fa = one ? 0 : f % 17;
+      const int r = one ? f : f / 17;     // r = kz * 16 + j
       c0 = xy_slot(fa - 3, r % 16, r / 16);
       ta = r % 16;
       tb = z0 + r / 16;
       st = 1;
       wi = f >> 5;
     } else {
-      const int fy = f - SF_NFX;
-      const int i = fy % 16, r = fy / 16; // r = kz * 17 + fa
-      fa = r % 17;
-      c0 = xy_slot(i, fa - 3, r / 17);
+      const int fy = f - nx;
+      const int i = fy % 16, r = fy / 16; // r = kz * 17 + fa, or kz
+      fa = one ? 0 : r % 17;
+      const int kz = one ? r : r / 17;
+      c0 = xy_slot(i, fa - 3, kz);
       ta = i;
-      tb = z0 + r / 17;
+      tb = z0 + kz;
       st = 24;
       wi = 34 + (fy >> 5);
     }
@@ -1088,16 +1251,17 @@ __device__ __forceinline__ void sweep_xy(const double* __restrict__ u, const Top
       if (isx) sub_viscous_f32<0>(u, sidx(fa - 1, ta, tb), L.mu, L.idx, F);
       else sub_viscous_f32<1>(u, sidx(ta, fa - 1, tb), L.mu, L.idx, F);
     }
-    store_face(isx ? 0 : 1, F, Fs, SF_FMAX, f, fa, ta, tb, fb);
+    if (one) store_sides(isx ? 0 : 1, F, true, true, ta, tb, fb);
+    else store_face(isx ? 0 : 1, F, Fs, SF_FMAX, f, fa, ta, tb, fb);
   }
   __syncthreads();
 #pragma unroll
   for (int kz = 0; kz < SF_TZ; ++kz) {
 #pragma unroll
     for (int v = 0; v < NV; ++v) acc[kz][v] = 0.f;
-    const int lx = (kz * 16 + tj) * 17 + ti, ly = SF_NFX + (kz * 17 + tj) * 16 + ti;
-    add_diff(0, Fs, SF_FMAX, lx, lx + 1, acc[kz]);
-    add_diff(1, Fs, SF_FMAX, ly, ly + 16, acc[kz]);
+    const int lx = (kz * 16 + tj) * 17 + ti, ly = nx + (kz * 17 + tj) * 16 + ti;
+    if (!flatx) add_diff(0, Fs, SF_FMAX, lx, lx + 1, acc[kz]);
+    if (!flaty) add_diff(1, Fs, SF_FMAX, ly, ly + 16, acc[kz]);
   }
   __syncthreads();
 }
@@ -1107,26 +1271,37 @@ template <int MODE>
 __device__ __forceinline__ void sweep_z(const double* __restrict__ u, const Topo& t, const Pool& pool, int cur,
                                         int node, int slot, double* __restrict__ fb, float* __restrict__ S,
                                         float* __restrict__ Fs, int z0, float g, float B, float gm1,
-                                        float (&acc)[SF_TZ][NV], const LearnedCtx& L) {
+                                        float (&acc)[SF_TZ][NV], const LearnedCtx& L, unsigned* flat_sh) {
   const int ti = threadIdx.x & 15, tj = threadIdx.x >> 4;
   load_region_f32(2, region_src(t, pool, cur, node, slot), S, z0, g, B, gm1);
   __syncthreads();
-  for (int f = threadIdx.x; f < SF_NFZ; f += blockDim.x) {
+  bool flat = false;
+  if (!(MODE & 32) && probe_z(S)) {
+    unsigned m = flat_z(S, B);
+    if (MODE == 3) m &= one_decision(L.selw, 68, 40) ? 4u : 0u;
+    flat = block_and(m, flat_sh) != 0u;
+  }
+  // constant pencils: no differences, and a flux only at the block's own sides
+  const bool lo = z0 == 0, hi = z0 + SF_TZ == NB;
+  for (int f = threadIdx.x; f < (flat ? ((lo || hi) ? NFACE : 0) : SF_NFZ); f += blockDim.x) {
     const int i = f % 16, j = (f / 16) % 16, fa = f / 256;
     const int c0 = (fa * 16 + j) * 16 + i;
     const bool lin = (MODE == 3) && ((L.selw[68 + (f >> 5)] >> (threadIdx.x & 31)) & 1u);
     float F[5];
     face_flux_f32<MODE>(S, c0, 256, rot_of(2), gm1, g, B, lin, F);
     if (MODE & 32) sub_viscous_f32<2>(u, sidx(i, j, z0 + fa - 1), L.mu, L.idx, F);
-    store_face(2, F, Fs, SF_FMAX, f, z0 + fa, i, j, fb);
+    if (flat) store_sides(2, F, lo, hi, i, j, fb);
+    else store_face(2, F, Fs, SF_FMAX, f, z0 + fa, i, j, fb);
   }
   __syncthreads();
+  if (!flat) {
 #pragma unroll
-  for (int kz = 0; kz < SF_TZ; ++kz) {
-    const int lo = (kz * 16 + tj) * 16 + ti;
-    add_diff(2, Fs, SF_FMAX, lo, lo + 256, acc[kz]);
+    for (int kz = 0; kz < SF_TZ; ++kz) {
+      const int lz = (kz * 16 + tj) * 16 + ti;
+      add_diff(2, Fs, SF_FMAX, lz, lz + 256, acc[kz]);
+    }
+    __syncthreads();
   }
-  __syncthreads();
 }
 
 template <int MODE>
@@ -1142,6 +1317,7 @@ __global__ void __launch_bounds__(SF_THREADS, 2)
   const float g = (float)p.gamma, B = (float)p.B, gm1 = (float)(p.gamma - 1.0);
   const int ti = threadIdx.x & 15, tj = threadIdx.x >> 4;
   __shared__ uint32_t sel_sh[108];
+  __shared__ unsigned flat_sh[SF_THREADS / 32];
   LearnedCtx L{nullptr, nullptr, nullptr, nullptr, 0.f, nullptr, nullptr, 0.f, sel_sh, (float)p.mu, 0.f};
   if (MODE == 1) {
     uint32_t* frag = reinterpret_cast<uint32_t*>(Fs + NV * SF_NFZ);   // after one direction's face fluxes
@@ -1197,11 +1373,12 @@ __global__ void __launch_bounds__(SF_THREADS, 2)
       for (int kz = 0; kz < SF_TZ; ++kz)
 #pragma unroll
         for (int v = 0; v < NV; ++v) acc[kz][v] = 0.f;
+      unsigned flat = 0u;
 #pragma unroll 1
-      for (int D = 0; D < 3; ++D) sweep_f32<MODE>(D, t, pool, cur, node, slot, fb, S, Fs, z0, g, B, gm1, acc, L, cnt);
+      for (int D = 0; D < 3; ++D) sweep_f32<MODE>(D, t, pool, cur, node, slot, fb, S, Fs, z0, g, B, gm1, acc, L, cnt, flat, flat_sh);
     } else {
-      sweep_xy<MODE>(u, t, pool, cur, node, slot, fb, S, Fs, z0, g, B, gm1, acc, L);
-      sweep_z<MODE>(u, t, pool, cur, node, slot, fb, S, Fs, z0, g, B, gm1, acc, L);
+      sweep_xy<MODE>(u, t, pool, cur, node, slot, fb, S, Fs, z0, g, B, gm1, acc, L, flat_sh);
+      sweep_z<MODE>(u, t, pool, cur, node, slot, fb, S, Fs, z0, g, B, gm1, acc, L, flat_sh);
     }
     if (MODE == 1) {
       lvl = t.level[node];
