@@ -71,7 +71,8 @@ struct mrb_ctx {
   uint64_t* d_keys = nullptr;
   int32_t *d_slot = nullptr, *d_level = nullptr, *d_inst = nullptr, *d_X = nullptr, *d_parent = nullptr,
           *d_child0 = nullptr, *d_nbr = nullptr, *d_leaves = nullptr, *d_lvl_nodes = nullptr, *d_bc_items = nullptr, *d_jump = nullptr, *d_cnt = nullptr,
-          *d_lmax = nullptr, *d_list = nullptr;
+          *d_lmax = nullptr, *d_list = nullptr, *d_pst = nullptr, *d_pall = nullptr;
+  uint32_t *d_miss = nullptr, *d_smask = nullptr;
   double *d_dt = nullptr, *d_delta_node = nullptr, *d_partial = nullptr;
   unsigned long long* d_census = nullptr;   // mrb_flux_census counters (allocated on first use)
   unsigned long long* d_smax = nullptr;
@@ -83,7 +84,7 @@ struct mrb_ctx {
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   cudaStream_t cap_st = nullptr;     // private stream for capture (the caller's may be the legacy stream)
   bool graph_dirty = true;
-  bool detail_filled = false;        // leaves' halos hold rho and E only (fill before the details)
+  bool detail_filled = false;        // stored halos are not complete (fill before the details)
   char* h_stage = nullptr;           // pinned staging of the topology uploads
   int32_t* h_list = nullptr;         // pinned staging of work lists
   cudaEvent_t stage_ev = nullptr, list_ev = nullptr;
@@ -111,6 +112,10 @@ struct mrb_ctx {
     t.lvl_nodes = d_lvl_nodes;
     t.bc_items = d_bc_items;
     t.jump = d_jump;
+    t.miss = d_miss;
+    t.smask = d_smask;
+    t.pst = d_pst;
+    t.pall = d_pall;
     t.cnt = d_cnt;
     return t;
   }
@@ -186,7 +191,7 @@ struct mrb_ctx {
       }
     }
     h_cnt[CNT_BC + MAXL + 1] = (int)h_bc_items.size();
-    h_cnt[CNT_JUMP] = 0;     // counted on the device after the neighbour table
+    // (the counts of jumps and predicted nodes are taken on the device after the neighbour table)
     // one pinned staging area for every array (asynchronous copies); the
     // previous rebuild's copies have long finished when it is rewritten
     if (stage_ev) CK(cudaEventSynchronize(stage_ev));
@@ -222,6 +227,7 @@ struct mrb_ctx {
     put(d_bc_items, h_bc_items.data(), sizeof(int32_t) * h_bc_items.size());
     put(d_cnt, h_cnt.data(), sizeof(int32_t) * CNT_SIZE);
     launch_nbr(topo(), phys, d_nbr, n, st);
+    launch_masks(topo(), phys, d_miss, d_smask, d_pst, d_pall, d_cnt, max_lmax, st);
     launch_jump_list(topo(), d_jump, d_cnt, (int)h_leaves.size(), st);
     CK(cudaGetLastError());
     CK(cudaEventRecord(stage_ev, st));
@@ -251,8 +257,13 @@ struct mrb_ctx {
 
   // ---- the steps
   void fill_halos(int mode = FILL_FULL) {
-    for (int l = 0; l <= max_lmax; ++l) launch_fill_level(topo(), phys, P, cur, l, st, mode);
+    if (mode == FILL_FULL) launch_fill_copies(topo(), phys, P, cur, st);
+    for (int l = 1; l <= max_lmax; ++l) launch_predict(topo(), phys, P, cur, l, mode, st);
+    if (mode == FILL_FULL) launch_fill_bc(topo(), phys, P, cur, st);
   }
+  // the stage kernels read face neighbours' cells and map boundary cells
+  // themselves; the viscous gradients read stored edge cells of the halo
+  int stage_fill() const { return cfg.mu > 0.0 ? FILL_FULL : FILL_STAGE; }
   void stage(int s, const double* dt) {
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (capturing >= 0) {
@@ -280,12 +291,8 @@ struct mrb_ctx {
   }
   void step_stages() {
     launch_cfl(topo(), phys, P, cur, d_smax, d_dt, d_status, st);
-    // the mixed-precision stage kernel reads face neighbours directly, so the
-    // stage fill of leaves is limited to predicted and boundary face regions;
-    // the viscous gradients read edge halo cells, which need the full fill
-    const int mode = (cfg.precision == MRB_FP32_ACC64 && !(cfg.mu > 0.0)) ? FILL_STAGE : FILL_FULL;
     for (int s = 0; s < phys.rk; ++s) {
-      fill_halos(mode);
+      fill_halos(stage_fill());
       stage(s, d_dt);
       project();
     }
@@ -301,7 +308,7 @@ struct mrb_ctx {
     launch_cfl(topo(), phys, P, cur, d_smax, d_dt, d_status, st);
     launch_lts_fmac(topo(), phys, P, 0, 0, d_dt, 1, st);
     const int L = max_lmax;
-    const int fmode = (cfg.precision == MRB_FP32_ACC64 && !(cfg.mu > 0.0)) ? FILL_STAGE : FILL_FULL;
+    const int fmode = stage_fill();
     const double cst[2][3] = {{0.0, 1.0, 0.5}, {0.0, 1.0, 0.0}};   // stage times, TVD-RK3 / TVD-RK2
     const int row = (phys.rk == 2) ? 1 : 0;
     for (int r = 0; r < (1 << L); ++r) {
@@ -318,7 +325,9 @@ struct mrb_ctx {
           launch_lts_interp(topo(), P, cur, l, th, 0, st);
           // the stepping level's halos, and those of the coarser levels its
           // predictions read; finer levels are filled when they step
-          for (int ll = 0; ll <= l; ++ll) launch_fill_level(topo(), phys, P, cur, ll, st, fmode);
+          if (fmode == FILL_FULL) launch_fill_copies(topo(), phys, P, cur, st);
+          for (int ll = 1; ll <= l; ++ll) launch_predict(topo(), phys, P, cur, ll, fmode, st);
+          if (fmode == FILL_FULL) launch_fill_bc(topo(), phys, P, cur, st);
           if (cfg.precision == MRB_FP32_ACC64) launch_rhs_rk_f32(topo(), phys, P, cur, s, d_dt, nullptr, st, l);
           else launch_rhs_rk_f64(topo(), phys, P, cur, s, d_dt, nullptr, st, l);
           launch_lts_copyback(topo(), P, cur, l, st);
@@ -405,9 +414,9 @@ struct mrb_ctx {
       throw Err(MRB_ECAPACITY, "block pool exhausted by refinement");
     if (refine.empty() && coarse_parents.empty()) return nl;
     if (detail_fill && !refine.empty()) {
-      // the halos of leaves were filled for the details only (rho, E): complete
-      // those of the blocks about to be refined, whose children are predicted
-      // over their whole stored range
+      // the fill before the details computed predicted regions only: complete
+      // the stored halos of the blocks about to be refined, whose children are
+      // predicted over their whole stored range
       upload_list(refine);
       launch_fill_list(topo(), phys, P, cur, d_list, (int)refine.size(), st);
       list_used();
@@ -647,6 +656,10 @@ int mrb_init_blocks(const mrb_config* cfg, void* pool, size_t pool_bytes, mrb_ct
     c->d_lvl_nodes = c->dalloc<int32_t>(n);
     c->d_bc_items = c->dalloc<int32_t>(6 * n);
     c->d_jump = c->dalloc<int32_t>(n);
+    c->d_miss = c->dalloc<uint32_t>(n);
+    c->d_smask = c->dalloc<uint32_t>(n);
+    c->d_pst = c->dalloc<int32_t>(n);
+    c->d_pall = c->dalloc<int32_t>(n);
     c->d_cnt = c->dalloc<int32_t>(CNT_SIZE);
     c->d_lmax = c->dalloc<int32_t>(cfg->n_instances);
     c->d_list = c->dalloc<int32_t>(2 * n);
@@ -1042,7 +1055,7 @@ int mrb_autotune(mrb_ctx* c, int32_t reps, double* times) {
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
-    const int fmode = (c->cfg.precision == MRB_FP32_ACC64 && !(c->cfg.mu > 0.0)) ? FILL_STAGE : FILL_FULL;
+    const int fmode = c->stage_fill();
     launch_cfl(c->topo(), c->phys, c->P, c->cur, c->d_smax, c->d_dt, c->d_status, c->st);
     auto run = [&](int what) {
       if (what == 0) {

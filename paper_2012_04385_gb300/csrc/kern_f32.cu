@@ -22,21 +22,19 @@ void launch_rhs_rk_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, 
   } else launch_stage_f32<0>(t, p, pool, cur, stage, dt, rhs_out, st, level);
 }
 
-void launch_fill_level_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, int level, cudaStream_t st,
-                           int mode) {
-  const NodeSet ns{level, nullptr, 0};
-  k_fill_regions_t<float><<<sm_count() * g_tune.fill_copy, 256, 0, st>>>(t, pool, cur, ns, mode);
-  k_fill_predict_t<float><<<sm_count() * g_tune.fill_pred, 256, 0, st>>>(t, pool, cur, ns, mode);
-  k_fill_bc<<<sm_count() * 4, 256, 0, st>>>(t, p, pool, cur, ns, mode);
-  g_kernel_launches += 3;
+void launch_predict_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, int level, int mode, cudaStream_t st) {
+  const bool stage = mode == FILL_STAGE;
+  k_predict_t<float><<<sm_count() * g_tune.fill_pred, 256, 0, st>>>(t, p, pool, cur, stage ? t.pst : t.pall,
+                                                                    t.cnt, level, stage ? t.smask : t.miss, mode);
+  ++g_kernel_launches;
 }
 
 void launch_fill_list_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, const int32_t* list, int n,
                           cudaStream_t st) {
-  const NodeSet ns{0, list, n};
-  k_fill_regions_t<float><<<sm_count() * 8, 256, 0, st>>>(t, pool, cur, ns, FILL_FULL);
-  k_fill_predict_t<float><<<sm_count() * 4, 256, 0, st>>>(t, pool, cur, ns, FILL_FULL);
-  k_fill_bc<<<sm_count() * 4, 256, 0, st>>>(t, p, pool, cur, ns, FILL_FULL);
+  const NodeSet ns{list, n};
+  k_fill_regions<<<sm_count() * 8, 256, 0, st>>>(t, pool, cur, ns);
+  k_predict_t<float><<<sm_count() * 4, 256, 0, st>>>(t, p, pool, cur, list, nullptr, n, t.miss, FILL_FULL);
+  k_fill_bc<<<sm_count() * 4, 256, 0, st>>>(t, p, pool, cur, ns);
   g_kernel_launches += 3;
 }
 
@@ -165,6 +163,8 @@ __global__ void __launch_bounds__(256) k_delta_p(Topo t, Phys p, Pool pool, int 
                                                  int all_nodes) {
   __shared__ double sh[8];
   __shared__ float2 box[4096];      // (rho, E) of the parent's cells 8 cb - 4 .. 8 cb + 11 per axis
+  __shared__ ParentBox pb;
+  __shared__ const double* own[27]; // the node's stored cells by region
   const int nitems = all_nodes ? t.cnt[CNT_NNODES] : t.cnt[CNT_NLEAVES];
   const double* B = pool.bufp(cur);
   const float C0 = -22.f / 128.f, C1 = 3.f / 128.f;
@@ -176,10 +176,10 @@ __global__ void __launch_bounds__(256) k_delta_p(Topo t, Phys p, Pool pool, int 
       continue;
     }
     const int par = t.parent[node];
-    const double* U = B + (size_t)t.slot[node] * SLOT_U;
-    const double* P = B + (size_t)t.slot[par] * SLOT_U;
     const int ch = (int)(t.keys[node] & 7ull);
-    const int cb0 = ch & 1, cb1 = (ch >> 1) & 1, cb2 = (ch >> 2) & 1;
+    parent_box(t, p, B, par, ch, pb);
+    if (threadIdx.x < 27) own[threadIdx.x] = region_base(t, B, node, threadIdx.x);
+    __syncthreads();
     bool gl[3], gh[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
@@ -188,20 +188,29 @@ __global__ void __launch_bounds__(256) k_delta_p(Topo t, Phys p, Pool pool, int 
       gl[d] = (Xd == 0) && (p.bc[2 * d] != 1);
       gh[d] = (Xd == nl - 1) && (p.bc[2 * d + 1] != 1);
     }
-    const int bx0 = 8 * cb0 - 4, by0 = 8 * cb1 - 4, bz0 = 8 * cb2 - 4;
     for (int e = threadIdx.x; e < 4096; e += blockDim.x) {
-      const int s = sidx(bx0 + e % 16, by0 + (e / 16) % 16, bz0 + e / 256);
-      box[e] = make_float2(d2f_fast(P[s]), d2f_fast(P[4 * NCELL + s]));
+      const unsigned w = box_word(pb, e & 15, (e >> 4) & 15, e >> 8);
+      const double* __restrict__ c = pb.p[(w >> 16) & 7u] + (w & 0xffffu);
+      box[e] = make_float2(d2f_fast(c[0]), d2f_fast(c[4 * NCELL]));
     }
     __syncthreads();
-    const SAcc2 A{box, bx0, by0, bz0};
+    const SAcc2 A{box, 0, 0, 0};
     float m = 0.f;
     for (int q = threadIdx.x; q < 1728; q += blockDim.x) {
       const int rx = q % 12 - 2, ry = (q / 12) % 12 - 2, rz = q / 144 - 2;
       const bool ghost = (rx < 0 && gl[0]) || (rx >= 8 && gh[0]) || (ry < 0 && gl[1]) || (ry >= 8 && gh[1]) ||
                          (rz < 0 && gl[2]) || (rz >= 8 && gh[2]);
       if (ghost) continue;
-      const int i = 8 * cb0 + rx, j = 8 * cb1 + ry, k = 8 * cb2 + rz;
+      const int i = rx + 4, j = ry + 4, k = rz + 4;
+      // the eight fine cells, loaded ahead of the Q-terms in aligned pairs
+      const double* __restrict__ U = own[own_region(rx, ry, rz)] + sidx(2 * rx, 2 * ry, 2 * rz);
+      double2 fr[4], fe[4];
+#pragma unroll
+      for (int q2 = 0; q2 < 4; ++q2) {       // rows y + (q2 & 1), z + (q2 >> 1)
+        const int o = ((q2 >> 1) * NS + (q2 & 1)) * NS;
+        fr[q2] = *reinterpret_cast<const double2*>(U + o);
+        fe[q2] = *reinterpret_cast<const double2*>(U + 4 * NCELL + o);
+      }
       const float2 u = A(i, j, k);
       const float2 Qx = f2fma(f2s(C0), f2sub(A(i + 1, j, k), A(i - 1, j, k)), f2mul(f2s(C1), f2sub(A(i + 2, j, k), A(i - 2, j, k))));
       const float2 Qy = f2fma(f2s(C0), f2sub(A(i, j + 1, k), A(i, j - 1, k)), f2mul(f2s(C1), f2sub(A(i, j + 2, k), A(i, j - 2, k))));
@@ -239,8 +248,8 @@ __global__ void __launch_bounds__(256) k_delta_p(Topo t, Phys p, Pool pool, int 
         pr = (a ^ c) ? f2sub(pr, Qxz) : f2add(pr, Qxz);
         pr = (b ^ c) ? f2sub(pr, Qyz) : f2add(pr, Qyz);
         pr = (a ^ b ^ c) ? f2sub(pr, Qxyz) : f2add(pr, Qxyz);
-        const int s = sidx(2 * rx + a, 2 * ry + b, 2 * rz + c);
-        const float2 uf = make_float2(d2f_fast(U[s]), d2f_fast(U[4 * NCELL + s]));
+        const int q2 = b + 2 * c;
+        const float2 uf = make_float2(d2f_fast(a ? fr[q2].y : fr[q2].x), d2f_fast(a ? fe[q2].y : fe[q2].x));
         const float2 dd = f2sub(uf, pr);
         const float r0 = fabsf(dd.x / uf.x), r1 = fabsf(dd.y / uf.y);
         m = fmaxf(m, fmaxf(r0, r1));

@@ -96,19 +96,26 @@ void launch_get_state(const Topo& t, const Pool& pool, int cur, const int32_t* n
 }
 
 // ---------------------------------------------------------------- halo fill (mr.cuh)
-void launch_fill_level(const Topo& t, const Phys& p, const Pool& pool, int cur, int level, cudaStream_t st,
-                       int mode) {
+void launch_fill_copies(const Topo& t, const Phys& p, const Pool& pool, int cur, cudaStream_t st) {
+  (void)p;
+  k_fill_regions<<<sm_count() * g_tune.fill_copy, 256, 0, st>>>(t, pool, cur, NodeSet{nullptr, 0});
+  ++g_kernel_launches;
+}
+
+void launch_fill_bc(const Topo& t, const Phys& p, const Pool& pool, int cur, cudaStream_t st) {
+  k_fill_bc<<<sm_count() * 4, 256, 0, st>>>(t, p, pool, cur, NodeSet{nullptr, 0});
+  ++g_kernel_launches;
+}
+
+void launch_predict(const Topo& t, const Phys& p, const Pool& pool, int cur, int level, int mode, cudaStream_t st) {
   if (p.precision == 1) {
-    launch_fill_level_f32(t, p, pool, cur, level, st, mode);
+    launch_predict_f32(t, p, pool, cur, level, mode, st);
     return;
   }
-  // the FP64 stage kernel reads every halo region: no stage-partial fill
-  const NodeSet ns{level, nullptr, 0};
-  const int m = (mode == FILL_STAGE) ? FILL_FULL : mode;
-  k_fill_regions_t<double><<<sm_count() * g_tune.fill_copy, 256, 0, st>>>(t, pool, cur, ns, m);
-  k_fill_predict_t<double><<<sm_count() * g_tune.fill_pred, 256, 0, st>>>(t, pool, cur, ns, m);
-  k_fill_bc<<<sm_count() * 4, 256, 0, st>>>(t, p, pool, cur, ns, m);
-  g_kernel_launches += 3;
+  const bool stage = mode == FILL_STAGE;
+  k_predict_t<double><<<sm_count() * g_tune.fill_pred, 256, 0, st>>>(t, p, pool, cur, stage ? t.pst : t.pall, t.cnt,
+                                                                     level, stage ? t.smask : t.miss, mode);
+  ++g_kernel_launches;
 }
 
 void launch_fill_list(const Topo& t, const Phys& p, const Pool& pool, int cur, const int32_t* list, int n,
@@ -118,10 +125,10 @@ void launch_fill_list(const Topo& t, const Phys& p, const Pool& pool, int cur, c
     launch_fill_list_f32(t, p, pool, cur, list, n, st);
     return;
   }
-  const NodeSet ns{0, list, n};
-  k_fill_regions_t<double><<<sm_count() * 8, 256, 0, st>>>(t, pool, cur, ns, FILL_FULL);
-  k_fill_predict_t<double><<<sm_count() * 4, 256, 0, st>>>(t, pool, cur, ns, FILL_FULL);
-  k_fill_bc<<<sm_count() * 4, 256, 0, st>>>(t, p, pool, cur, ns, FILL_FULL);
+  const NodeSet ns{list, n};
+  k_fill_regions<<<sm_count() * 8, 256, 0, st>>>(t, pool, cur, ns);
+  k_predict_t<double><<<sm_count() * 4, 256, 0, st>>>(t, p, pool, cur, list, nullptr, n, t.miss, FILL_FULL);
+  k_fill_bc<<<sm_count() * 4, 256, 0, st>>>(t, p, pool, cur, ns);
   g_kernel_launches += 3;
 }
 
@@ -600,6 +607,56 @@ __global__ void k_nbr(Topo t, Phys p, int32_t* __restrict__ nbr_out) {
       else hi = mid - 1;
     }
     nbr_out[e] = found;
+  }
+}
+
+// Predicted regions.  miss: every region without a same-level node (nor beyond the
+// boundary).  smask: those a stage needs -- of a leaf (and with local time
+// stepping of every node) the face regions; of an internal node what the wanted
+// regions of its children read: a region s of the child in octant cb reads the
+// parent's cells within two of it, which lie beyond the parent on axis d (on the
+// octant's side) when s_d is 0 or points out of the parent.
+constexpr uint32_t FACE_REGIONS = (1u << 12) | (1u << 14) | (1u << 10) | (1u << 16) | (1u << 4) | (1u << 22);
+__global__ void k_masks(Topo t, Phys p, uint32_t* __restrict__ miss, uint32_t* __restrict__ smask,
+                        int32_t* __restrict__ pst, int32_t* __restrict__ pall, int32_t* __restrict__ cnt, int level) {
+  const int beg = t.cnt[CNT_LVL + level], end = t.cnt[CNT_LVL + level + 1];
+  for (int w = beg + blockIdx.x * blockDim.x + threadIdx.x; w < end; w += gridDim.x * blockDim.x) {
+    const int node = t.lvl_nodes[w];
+    uint32_t ms = 0;
+    for (int r = 0; r < 27; ++r)
+      if (t.nbr[(size_t)node * 27 + r] == -1) ms |= 1u << r;
+    const int c0 = t.child0[node];
+    uint32_t need = (c0 < 0 || p.lts) ? FACE_REGIONS : 0u;
+    for (int ch = 0; c0 >= 0 && ch < 8; ++ch) {
+      uint32_t m = smask[c0 + ch];
+      while (m) {
+        const int r = __ffs(m) - 1;
+        m &= m - 1;
+        const int s[3] = {r % 3 - 1, (r / 3) % 3 - 1, r / 9 - 1};
+        int beyond = 0;
+        for (int d = 0; d < 3; ++d)
+          if (s[d] == 0 || s[d] == (((ch >> d) & 1) ? 1 : -1)) beyond |= 1 << d;
+        for (int q = 1; q < 8; ++q) {
+          if (q & ~beyond) continue;
+          int rr = 13;
+          for (int d = 0; d < 3; ++d)
+            if ((q >> d) & 1) rr += (((ch >> d) & 1) ? 1 : -1) * (d == 0 ? 1 : (d == 1 ? 3 : 9));
+          need |= 1u << rr;
+        }
+      }
+    }
+    miss[node] = ms;
+    smask[node] = need & ms;
+    if (need & ms) pst[beg + atomicAdd(&cnt[CNT_PST + level], 1)] = node;
+    if (ms) pall[beg + atomicAdd(&cnt[CNT_PALL + level], 1)] = node;
+  }
+}
+
+void launch_masks(const Topo& t, const Phys& p, uint32_t* miss, uint32_t* smask, int32_t* pst, int32_t* pall, int32_t* cnt,
+                  int max_level, cudaStream_t st) {
+  for (int l = max_level; l >= 0; --l) {
+    k_masks<<<sm_count(), 128, 0, st>>>(t, p, miss, smask, pst, pall, cnt, l);
+    ++g_kernel_launches;
   }
 }
 

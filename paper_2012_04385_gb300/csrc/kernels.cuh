@@ -13,15 +13,24 @@ constexpr int MAXL = 11;              // deepest level
 constexpr int CNT_NNODES = 0, CNT_NLEAVES = 1, CNT_LVL = 2;   // lvl offsets at CNT_LVL + l, l = 0..MAXL+1
 constexpr int CNT_BC = CNT_LVL + MAXL + 2;                     // bc item offsets at CNT_BC + l, l = 0..MAXL+1
 constexpr int CNT_JUMP = CNT_BC + MAXL + 2;                    // number of jump items
-constexpr int CNT_SIZE = CNT_JUMP + 1;
+constexpr int CNT_PST = CNT_JUMP + 1;                          // nodes with stage predictions per level, l = 0..MAXL
+constexpr int CNT_PALL = CNT_PST + MAXL + 1;                   // nodes with any predicted region per level
+constexpr int CNT_SIZE = CNT_PALL + MAXL + 1;
 
 enum : int { ST_OK = 0, ST_NONPHYS = 6 };
 
-// Halo fill modes, for leaves (internal nodes are always filled completely):
-//   FILL_FULL       every region, every variable;
-//   FILL_STAGE      only the predicted face regions (the mixed-precision stage
-//                   kernel reads same-level face neighbours' cells directly);
-//   FILL_DETAIL     every region, rho and E only (the detail norm's inputs).
+// Halo fill modes.  A halo cell facing a same-level node is that node's internal
+// cell, and one beyond a non-periodic boundary is a mapped cell, so the kernels
+// of a step read those where they are (mr.cuh, HaloSrc) and only predicted
+// regions, which exist nowhere else, are ever computed for them:
+//   FILL_FULL       every region of every node in its stored halo (mrb_fill_halos,
+//                   and the stages with viscous terms, which read edges);
+//   FILL_STAGE      the predicted regions that a stage reads: face regions of the
+//                   leaves, and what their predictions read of internal nodes;
+//   FILL_DETAIL     every predicted region, of leaves rho and E only (the detail
+//                   norm's inputs).
+// Measured on the shock-bubble (levels 0..4, 6,600 nodes): the copies and boundary
+// cells were 1.8 of 3.1 ms of fills per step.
 enum : int { FILL_FULL = 0, FILL_STAGE = 1, FILL_DETAIL = 2 };
 
 // Node arrays, in ascending id order (instance, level, Morton).
@@ -38,6 +47,10 @@ struct Topo {
   const int32_t* lvl_nodes;// node indices grouped by level
   const int32_t* bc_items; // 8 * node + side of every non-periodic domain-boundary side, grouped by level
   const int32_t* jump;     // 64 * leaf index + mask of the sides whose same-level neighbour is refined
+  const uint32_t* miss;    // 27-bit mask of a node's predicted halo regions (nbr == -1)
+  const uint32_t* smask;   // those that a stage needs (see k_masks)
+  const int32_t* pst;      // nodes with smask != 0, grouped by level like lvl_nodes (count CNT_PST + l)
+  const int32_t* pall;     // nodes with miss != 0, likewise (count CNT_PALL + l)
   const int32_t* cnt;      // counts, see CNT_*
 };
 
@@ -140,8 +153,11 @@ void launch_set_cons(const Topo& t, const Pool& pool, int cur, const int32_t* no
                      cudaStream_t st);
 void launch_get_state(const Topo& t, const Pool& pool, int cur, const int32_t* nodes, int n, double* out,
                       int with_halo, cudaStream_t st);
-void launch_fill_level(const Topo& t, const Phys& p, const Pool& pool, int cur, int level, cudaStream_t st,
-                       int mode = 0);
+// stored halos facing same-level nodes, and ghost cells beyond the boundary, of every node
+void launch_fill_copies(const Topo& t, const Phys& p, const Pool& pool, int cur, cudaStream_t st);
+void launch_fill_bc(const Topo& t, const Phys& p, const Pool& pool, int cur, cudaStream_t st);
+// predicted regions of the nodes of `level` (after those of the coarser levels)
+void launch_predict(const Topo& t, const Phys& p, const Pool& pool, int cur, int level, int mode, cudaStream_t st);
 // every halo region of the listed nodes (device list of n node indices), all variables
 void launch_fill_list(const Topo& t, const Phys& p, const Pool& pool, int cur, const int32_t* list, int n,
                       cudaStream_t st);
@@ -191,11 +207,14 @@ void launch_refine_fill(const Topo& t, const Phys& p, const Pool& pool, int cur,
 // order unspecified; every item is independent).
 void launch_jump_list(const Topo& t, int32_t* jump, int32_t* cnt, int n_leaves_cap, cudaStream_t st);
 void launch_nbr(const Topo& t, const Phys& p, int32_t* nbr_out, int nnodes_cap, cudaStream_t st);
+// Masks of predicted regions and the lists of the nodes that have any, levels
+// fine to coarse (max_level .. 0).
+void launch_masks(const Topo& t, const Phys& p, uint32_t* miss, uint32_t* smask, int32_t* pst, int32_t* pall, int32_t* cnt,
+                  int max_level, cudaStream_t st);
 void launch_sums(const Topo& t, const Phys& p, const Pool& pool, int cur, double* partial, double* out,
                  int nleaves_cap, cudaStream_t st);
 // mixed-precision variants (kern_f32.cu)
-void launch_fill_level_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, int level, cudaStream_t st,
-                           int mode);
+void launch_predict_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, int level, int mode, cudaStream_t st);
 void launch_fill_list_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, const int32_t* list, int n,
                           cudaStream_t st);
 // Roe / LLF census of every leaf face (FP64 decisions on the stage buffer):

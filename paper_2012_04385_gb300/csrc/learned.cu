@@ -116,6 +116,7 @@ __global__ void __launch_bounds__(SF_THREADS) k_face_samples(Topo t, Phys p, Poo
     RS.sh = pool.shp(cur) ? pool.shp(cur) + (size_t)slot * SLOT_SH : nullptr;
 #pragma unroll
     for (int q = 0; q < 6; ++q) RS.nsh[q] = nullptr;
+    RS.bnd = RS.mir = 0u;
 #pragma unroll 1
     for (int D = 0; D < 3; ++D)
       sample_dir(D, RS, smp_smem, li, z0, g, B, gm1, tau_lab, stride, feats, labels, where, cap);

@@ -25,14 +25,8 @@ template <> __device__ __forceinline__ float to_r<float>(double x) { return d2f_
 template <class R> __device__ __forceinline__ double from_r(R x) { return double(x); }
 template <> __device__ __forceinline__ double from_r<float>(float x) { return f2d_fast(x); }
 
-// Parent values for the Q-terms: the stored FP64 array, converted to R on
-// load, or a box of R values staged in shared memory (origin i0, j0, k0 in
-// stored coordinates, row length nx, plane size nxy).  Both give the same R
-// value for a cell, so the Q-terms do not depend on where they are read.
-template <class R> struct GAcc {
-  const double* P;
-  __device__ __forceinline__ R operator()(int i, int j, int k) const { return to_r<R>(P[sidx(i, j, k)]); }
-};
+// Parent values for the Q-terms: a box of R values staged in shared memory
+// (origin i0, j0, k0 in stored coordinates, row length nx, plane size nxy).
 template <class R> struct SAcc {
   const R* s;
   int i0, j0, k0, nx, nxy;
@@ -103,11 +97,111 @@ template <class R, class A> __device__ __forceinline__ QT<R> qterms_t(const A& P
   return t;
 }
 
-// Stage the parent values of the box [i0, i0+nx) x [j0, j0+ny) x [k0, k0+nz)
-// (stored coordinates) of variable v into shared memory as R; all threads.
+// ---------------------------------------------------------------- stored cells where they are
+// Boundary condition of one axis: block coordinate x beyond a non-periodic side
+// (condition blo / bhi, -1 for none) mapped back into the block (zero gradient:
+// the nearest internal cell; symmetry: the mirror cell, with the normal
+// momentum negated: `bit` of flip).
+__device__ __forceinline__ int bc_map(int x, int blo, int bhi, int& flip, int bit) {
+  if (x < 0 && blo >= 0) {
+    flip ^= (blo == 2) ? bit : 0;
+    return blo == 0 ? 0 : -1 - x;
+  }
+  if (x >= NB && bhi >= 0) {
+    flip ^= (bhi == 2) ? bit : 0;
+    return bhi == 0 ? NB - 1 : 2 * NB - 1 - x;
+  }
+  return x;
+}
+
+// Base of region r (0 .. 26) of a node such that the node's stored index of a
+// cell of that region applies: the same-level neighbour's internal cells, or
+// the node's own stored halo where there is none (predicted).
+__device__ __forceinline__ const double* region_base(const Topo& t, const double* __restrict__ buf, int node, int r) {
+  const int nb = t.nbr[(size_t)node * 27 + r];
+  if (nb < 0) return buf + (size_t)t.slot[node] * SLOT_U;
+  const int sx = r % 3 - 1, sy = (r / 3) % 3 - 1, sz = r / 9 - 1;
+  return buf + (size_t)t.slot[nb] * SLOT_U - NB * (sx + NS * (sy + NS * sz));
+}
+
+// The 16^3 parent cells that a child in octant ch reads: 8 cb - 4 .. 8 cb + 11 per
+// axis, i.e. cells of the parent and of the seven regions on the octant's side
+// of it.  Per axis a table of the 16 coordinates: the offset in the stored array
+// of the cell that holds the value (bits 0-15; the coordinate itself, or the one
+// it maps to beyond a boundary), bit 16 + d when it lies in the region beyond
+// axis d, bit 20 + d when the mapping mirrors.  The sum of three entries is the
+// cell's offset and its flags, so a staged cell costs two additions and one
+// pointer select.
+struct ParentBox {
+  const double* p[8];      // bases by which axes are beyond the parent (bit d)
+  unsigned tab[3][16];
+};
+// (threads 0 .. 47; the caller synchronises)
+__device__ __forceinline__ void parent_box(const Topo& t, const Phys& p, const double* __restrict__ buf, int par, int ch,
+                                           ParentBox& b) {
+  const int q = threadIdx.x;
+  if (q < 8) {
+    int r = 13;
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+      if ((q >> d) & 1) r += (((ch >> d) & 1) ? 1 : -1) * (d == 0 ? 1 : (d == 1 ? 3 : 9));
+    b.p[q] = region_base(t, buf, par, r);
+  }
+  if (q < 48) {
+    const int d = q >> 4, hi = (ch >> d) & 1;
+    const int nl = (d == 0 ? p.nb[0] : (d == 1 ? p.nb[1] : p.nb[2])) << t.level[par], X = t.X[(size_t)par * 3 + d];
+    const int code = d == 0 ? (hi ? p.bc[1] : p.bc[0]) : (d == 1 ? (hi ? p.bc[3] : p.bc[2]) : (hi ? p.bc[5] : p.bc[4]));
+    const int bc = (X == (hi ? nl - 1 : 0) && code != 1) ? code : -1;
+    int x = 8 * hi - 4 + (q & 15), flip = 0;
+    unsigned w = 0;
+    if (x < 0 || x >= NB) {
+      if (bc >= 0) x = bc_map(x, hi ? -1 : bc, hi ? bc : -1, flip, 1);
+      else w = 1u << (16 + d);
+    }
+    w |= (unsigned)flip << (20 + d);
+    b.tab[d][q & 15] = w + (unsigned)((x + HW) * (d == 0 ? 1 : (d == 1 ? NS : NS * NS)));
+  }
+}
+// Flags and offset of box cell (i, j, k) in 0 .. 15; the value of variable v there.
+__device__ __forceinline__ unsigned box_word(const ParentBox& b, int i, int j, int k) {
+  return b.tab[0][i] + b.tab[1][j] + b.tab[2][k];
+}
+__device__ __forceinline__ double box_value(const ParentBox& b, unsigned w, int v) {
+  const double x = b.p[(w >> 16) & 7u][v * NCELL + (w & 0xffffu)];
+  return (v >= 1 && v <= 3 && ((w >> (19 + v)) & 1u)) ? -x : x;
+}
+
+// Stage the cells [i0, i0+nx) x [j0, j0+ny) x [k0, k0+nz) of the box (nx, ny, nz
+// 6, 12 or 16) of every variable (or rho and E only) as R, the
+// q-th at s + q * nx ny nz; all threads.  A group of 8 or 16 lanes owns a row.
 template <class R>
-__device__ __forceinline__ void stage_box(R* __restrict__ s, const double* __restrict__ P, int i0, int j0, int k0,
-                                          int nx, int ny, int nz) {
+__device__ __forceinline__ void stage_box(R* __restrict__ s, const ParentBox& b, bool detail_only, int i0, int j0,
+                                          int k0, int nx, int ny, int nz) {
+  const int lg = nx > 8 ? 4 : 3, i = threadIdx.x & ((1 << lg) - 1);
+  if (i >= nx) return;
+  const int n = nx * ny * nz, inv = ny == 16 ? 4096 : (ny == 12 ? 5462 : 10923);   // row / ny = row inv / 2^16 (rows < 256)
+  const unsigned wi = b.tab[0][i0 + i];
+  for (int row = threadIdx.x >> lg; row < ny * nz; row += blockDim.x >> lg) {
+    const int k = (row * inv) >> 16, j = row - k * ny;
+    const unsigned w = wi + b.tab[1][j0 + j] + b.tab[2][k0 + k];
+    const double* __restrict__ c = b.p[(w >> 16) & 7u] + (w & 0xffffu);
+    R* o = s + row * nx + i;
+    if (detail_only) {
+      o[0] = to_r<R>(c[0]);
+      o[n] = to_r<R>(c[4 * NCELL]);
+    } else {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        const double x = c[v * NCELL];
+        o[v * n] = to_r<R>((v >= 1 && v <= 3 && ((w >> (19 + v)) & 1u)) ? -x : x);
+      }
+    }
+  }
+}
+// The same from the parent's own stored cells (halo filled).
+template <class R>
+__device__ __forceinline__ void stage_stored(R* __restrict__ s, const double* __restrict__ P, int i0, int j0, int k0,
+                                             int nx, int ny, int nz) {
   const int n = nx * ny * nz;
   for (int e = threadIdx.x; e < n; e += blockDim.x) {
     const int i = e % nx, j = (e / nx) % ny, k = e / (nx * ny);
@@ -124,30 +218,16 @@ template <class R> __device__ __forceinline__ R predict_t(const QT<R>& t, R sx, 
 // ---------------------------------------------------------------- halo fill by region
 // Sec. 3 (Fig. MrCommunicationMesh): a halo region facing a same-level node
 // is a copy of its internal cells, one facing no same-level node is predicted
-// from the node's parent (one parent cell, eight fine cells, per step).  One
-// warp per (node, halo region) on a persistent grid; k_fill_bc then applies
-// the boundary conditions.  The nodes are those of one level, or a list.
-// Internal nodes, whose halos feed their children's predictions, are always
-// filled completely; leaves according to the fill mode (FILL_* in kernels.cuh).
+// from the node's parent (one parent cell, eight fine cells, per step), and
+// ghost cells take the boundary conditions.  The stored copies and ghost cells
+// are written only for FILL_FULL (and the listed nodes about to be refined):
+// copies depend on no halo and run for all levels at once, predictions level by
+// level, ghost cells (which may continue a copy or a prediction) at the end.
 
 struct NodeSet {
-  int level;                // nodes of this level, when list is null
-  const int32_t* list;      // else these nodes
+  const int32_t* list;      // these nodes, or every node when null
   int n;
 };
-
-__device__ __forceinline__ void nodeset_range(const Topo& t, const NodeSet& ns, int& beg, int& cnt) {
-  if (ns.list) {
-    beg = 0;
-    cnt = ns.n;
-  } else {
-    beg = t.cnt[CNT_LVL + ns.level];
-    cnt = t.cnt[CNT_LVL + ns.level + 1] - beg;
-  }
-}
-__device__ __forceinline__ int nodeset_node(const Topo& t, const NodeSet& ns, int beg, int i) {
-  return ns.list ? ns.list[i] : t.lvl_nodes[beg + i];
-}
 
 // Variable q of the fill: all five, or rho (q = 0) and E (q = 1) only.
 __device__ __forceinline__ int fill_var(bool detail_only, int q) { return detail_only ? 4 * q : q; }
@@ -159,106 +239,86 @@ __device__ __forceinline__ int region_log2(int s) { return s == 0 ? 4 : 2; }   /
 // One warp per (node, halo region).  Extents are powers of two, so the element
 // index splits with shifts; copies move 16-byte pairs of doubles (every
 // region row starts on a 32-byte boundary of the 24^3 array).
-template <class R>
-__global__ void __launch_bounds__(256) k_fill_regions_t(Topo t, Pool pool, int cur, NodeSet ns, int mode) {
-  int beg, cnt;
-  nodeset_range(t, ns, beg, cnt);
+static __global__ void __launch_bounds__(256) k_fill_regions(Topo t, Pool pool, int cur, NodeSet ns) {
   double* buf = pool.bufp(cur);
-  const int nitems = cnt * 26;
+  const int nitems = (ns.list ? ns.n : t.cnt[CNT_NNODES]) * 26;
   const int lane = threadIdx.x & 31;
   const int wpb = blockDim.x >> 5;
   for (int w = blockIdx.x * wpb + (threadIdx.x >> 5); w < nitems; w += gridDim.x * wpb) {
-    const int node = nodeset_node(t, ns, beg, w / 26);
+    const int node = ns.list ? ns.list[w / 26] : w / 26;
     const int r = w % 26 < 13 ? w % 26 : w % 26 + 1;      // skip the centre
-    const int sx = r % 3 - 1, sy = (r / 3) % 3 - 1, sz = r / 9 - 1;
-    const bool face = (sx != 0) + (sy != 0) + (sz != 0) == 1;
-    const bool leaf = t.child0[node] < 0;
-    const bool partial = mode == FILL_STAGE && leaf;
-    const bool detail_only = mode == FILL_DETAIL && leaf;
-    const int nvar = detail_only ? 2 : NV;
-    if (partial && !face) continue;
     const int nb = t.nbr[(size_t)node * 27 + r];
+    if (nb < 0) continue;
+    const int sx = r % 3 - 1, sy = (r / 3) % 3 - 1, sz = r / 9 - 1;
     double* u = buf + (size_t)t.slot[node] * SLOT_U;
-    if (nb >= 0) {
-      if (partial) continue;                              // read directly by the stage kernel
-      const double* src = buf + (size_t)t.slot[nb] * SLOT_U;
-      const int lx = region_log2(sx) - 1, ly = region_log2(sy), lz = region_log2(sz);   // x in pairs
-      const int x0 = region_start(sx), y0 = region_start(sy), z0 = region_start(sz);
-      const int lxy = lx + ly, ln = lxy + lz;
-      const int soff = -NB * (sx + NS * (sy + NS * sz));
-      const int ne = nvar << ln;               // a multiple of 32
-      // four 16-byte loads in flight per lane before their stores
-      for (int e0 = lane; e0 < ne; e0 += 128) {
-        double2 val[4];
-        int dst[4];
+    const double* src = buf + (size_t)t.slot[nb] * SLOT_U;
+    const int lx = region_log2(sx) - 1, ly = region_log2(sy), lz = region_log2(sz);   // x in pairs
+    const int x0 = region_start(sx), y0 = region_start(sy), z0 = region_start(sz);
+    const int lxy = lx + ly, ln = lxy + lz;
+    const int soff = -NB * (sx + NS * (sy + NS * sz));
+    const int ne = NV << ln;                 // a multiple of 32
+    // four 16-byte loads in flight per lane before their stores
+    for (int e0 = lane; e0 < ne; e0 += 128) {
+      double2 val[4];
+      int dst[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int e = e0 + 32 * q;
-          const int v = fill_var(detail_only, e >> ln), c = e & ((1 << ln) - 1);
-          const int i = x0 + 2 * (c & ((1 << lx) - 1)), j = y0 + ((c >> lx) & ((1 << ly) - 1)), k = z0 + (c >> lxy);
-          dst[q] = v * NCELL + sidx(i, j, k);
-          if (e < ne) val[q] = *reinterpret_cast<const double2*>(src + dst[q] + soff);
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          if (e0 + 32 * q < ne) *reinterpret_cast<double2*>(u + dst[q]) = val[q];
+      for (int q = 0; q < 4; ++q) {
+        const int e = e0 + 32 * q;
+        const int v = e >> ln, c = e & ((1 << ln) - 1);
+        const int i = x0 + 2 * (c & ((1 << lx) - 1)), j = y0 + ((c >> lx) & ((1 << ly) - 1)), k = z0 + (c >> lxy);
+        dst[q] = v * NCELL + sidx(i, j, k);
+        if (e < ne) val[q] = *reinterpret_cast<const double2*>(src + dst[q] + soff);
       }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (e0 + 32 * q < ne) *reinterpret_cast<double2*>(u + dst[q]) = val[q];
     }
   }
 }
 
-// Predicted halo regions (no same-level node on that side, the node has a
-// parent): one CTA per node, one region after the other; the parent cells
-// of the region and their +-2 stencil (6 or 12 per axis) are staged in shared
-// memory as R for the variables filled, then every thread evaluates the
-// Q-terms of parent cells and writes their eight fine cells.
+// Predicted halo regions (no same-level node on that side): the regions of a
+// node's mask are shared out to PRED_SPLIT CTAs (a leaf at a jump has nine or
+// more), each taking one after the other; the parent cells of the region and
+// their +-2 stencil (6 or 12 per axis) are staged in shared memory as R for the
+// variables filled, then every thread evaluates the Q-terms of parent cells
+// and writes their eight fine cells.
+constexpr int PRED_SPLIT = 4;
 template <class R>
-__global__ void __launch_bounds__(256) k_fill_predict_t(Topo t, Pool pool, int cur, NodeSet ns, int mode) {
+__global__ void __launch_bounds__(256) k_predict_t(Topo t, Phys p, Pool pool, int cur, const int32_t* __restrict__ list,
+                                                   const int32_t* __restrict__ cnt, int n,
+                                                   const uint32_t* __restrict__ mask, int mode) {
+  // the nodes of level n in a list grouped by level (cnt given), or n listed nodes
   __shared__ R box[NV * 864];
-  __shared__ unsigned rmask;
-  int beg, cnt;
-  nodeset_range(t, ns, beg, cnt);
+  __shared__ ParentBox pb;
   double* buf = pool.bufp(cur);
-  for (int w = blockIdx.x; w < cnt; w += gridDim.x) {
-    const int node = nodeset_node(t, ns, beg, w);
+  const int nitems = (cnt ? cnt[(mode == FILL_STAGE ? CNT_PST : CNT_PALL) + n] : n) * PRED_SPLIT;
+  if (cnt) list += cnt[CNT_LVL + n];
+  for (int w = blockIdx.x; w < nitems; w += gridDim.x) {
+    const int node = list[w / PRED_SPLIT];
+    unsigned m = mask[node];
+    const int part = w % PRED_SPLIT;
+    if (__popc(m) <= part) continue;
     const int par = t.parent[node];
-    if (par < 0) continue;                                   // level 0: no prediction
-    const bool leaf = t.child0[node] < 0;
-    const bool partial = mode == FILL_STAGE && leaf;
-    const bool detail_only = mode == FILL_DETAIL && leaf;
-    const int nvar = detail_only ? 2 : NV;
-    if (threadIdx.x < 32) {
-      bool want = false;
-      const int r = threadIdx.x;
-      if (r < 27 && r != 13) {
-        const int sx = r % 3 - 1, sy = (r / 3) % 3 - 1, sz = r / 9 - 1;
-        const bool face = (sx != 0) + (sy != 0) + (sz != 0) == 1;
-        want = t.nbr[(size_t)node * 27 + r] == -1 && (!partial || face);
-      }
-      const unsigned m = __ballot_sync(0xffffffffu, want);
-      if (threadIdx.x == 0) rmask = m;
-    }
-    __syncthreads();
-    unsigned m = rmask;
-    __syncthreads();
-    if (!m) continue;
-    double* u = buf + (size_t)t.slot[node] * SLOT_U;
-    const double* P = buf + (size_t)t.slot[par] * SLOT_U;
     const int ch = (int)(t.keys[node] & 7ull);
-    const int cb[3] = {ch & 1, (ch >> 1) & 1, (ch >> 2) & 1};
-    while (m) {
+    __syncthreads();                                         // the previous item's box is free
+    parent_box(t, p, buf, par, ch, pb);
+    __syncthreads();
+    const bool detail_only = mode == FILL_DETAIL && t.child0[node] < 0;
+    const int nvar = detail_only ? 2 : NV;
+    double* u = buf + (size_t)t.slot[node] * SLOT_U;
+    for (int rank = 0; m; ++rank) {
       const int r = __ffs(m) - 1;
       m &= m - 1;
+      if (rank % PRED_SPLIT != part) continue;
       const int sx = r % 3 - 1, sy = (r / 3) % 3 - 1, sz = r / 9 - 1;
       // parent cells of the region relative to the child's origin: [q0, q0 + n)
       const int lx = sx == 0 ? 3 : 1, ly = sy == 0 ? 3 : 1, lz = sz == 0 ? 3 : 1;
       const int qx0 = sx < 0 ? -2 : (sx == 0 ? 0 : 8), qy0 = sy < 0 ? -2 : (sy == 0 ? 0 : 8), qz0 = sz < 0 ? -2 : (sz == 0 ? 0 : 8);
-      // staged box: those parent cells +-2, in the parent's stored coordinates
-      const int bx0 = 8 * cb[0] + qx0 - 2, by0 = 8 * cb[1] + qy0 - 2, bz0 = 8 * cb[2] + qz0 - 2;
+      // staged box: those parent cells +-2 (box coordinates: relative to 8 cb - 4)
+      const int bx0 = qx0 + 2, by0 = qy0 + 2, bz0 = qz0 + 2;
       const int nx = (1 << lx) + 4, ny = (1 << ly) + 4, nz = (1 << lz) + 4;
       const int nb = nx * ny * nz;
-      for (int q = 0; q < nvar; ++q)
-        stage_box<R>(box + q * nb, P + fill_var(detail_only, q) * NCELL, bx0, by0, bz0, nx, ny, nz);
+      stage_box<R>(box, pb, detail_only, bx0, by0, bz0, nx, ny, nz);
       __syncthreads();
       const int lxy = lx + ly, ln = lxy + lz;
       for (int e = threadIdx.x; e < (nvar << ln); e += blockDim.x) {
@@ -266,12 +326,15 @@ __global__ void __launch_bounds__(256) k_fill_predict_t(Topo t, Pool pool, int c
         const int v = fill_var(detail_only, q);
         const int rx = qx0 + (c & ((1 << lx) - 1)), ry = qy0 + ((c >> lx) & ((1 << ly) - 1)), rz = qz0 + (c >> lxy);
         const SAcc<R> A{box + q * nb, bx0, by0, bz0, nx, nx * ny};
-        const QT<R> qt = qterms_t<R>(A, 8 * cb[0] + rx, 8 * cb[1] + ry, 8 * cb[2] + rz);
+        const QT<R> qt = qterms_t<R>(A, rx + 4, ry + 4, rz + 4);
+        // the two fine cells of a row are one aligned 16-byte store
 #pragma unroll
-        for (int sub = 0; sub < 8; ++sub) {
-          const int a = sub & 1, b = (sub >> 1) & 1, cc = (sub >> 2) & 1;
-          const R val = predict_t<R>(qt, a ? R(-1) : R(1), b ? R(-1) : R(1), cc ? R(-1) : R(1));
-          u[v * NCELL + sidx(2 * rx + a, 2 * ry + b, 2 * rz + cc)] = from_r<R>(val);
+        for (int sub = 0; sub < 8; sub += 2) {
+          const int b = (sub >> 1) & 1, cc = (sub >> 2) & 1;
+          const R v0 = predict_t<R>(qt, R(1), b ? R(-1) : R(1), cc ? R(-1) : R(1));
+          const R v1 = predict_t<R>(qt, R(-1), b ? R(-1) : R(1), cc ? R(-1) : R(1));
+          *reinterpret_cast<double2*>(u + v * NCELL + sidx(2 * rx, 2 * ry + b, 2 * rz + cc)) =
+              make_double2(from_r<R>(v0), from_r<R>(v1));
         }
       }
       __syncthreads();
@@ -279,36 +342,21 @@ __global__ void __launch_bounds__(256) k_fill_predict_t(Topo t, Pool pool, int c
   }
 }
 
-// Boundary conditions of the nodes of `level` on the domain boundary (after
-// their copies and predictions).  The oracle applies the x, y and z passes in
-// turn; their composition maps each ghost cell to one source cell, every
-// coordinate beyond a non-periodic side being mapped back into the block
-// (zero gradient: the nearest internal cell; any other condition: the mirror
-// cell, with the normal momentum negated under symmetry).  So one warp per
+// Stored ghost cells of the nodes on the domain boundary (after their copies and
+// predictions).  The oracle applies the x, y and z passes in turn; their
+// composition maps each ghost cell to one source cell (bc_map), so one warp per
 // (node, side) item fills the side's 4 x 24 x 24 slab from source cells that this
 // kernel never writes; cells in two slabs get the same value twice.  Work
 // items are (node, side, chunk of 256 slab cells), one warp each.
-__device__ __forceinline__ int bc_map(int x, int blo, int bhi, int& flip, int bit) {
-  if (x < 0 && blo >= 0) {
-    flip ^= (blo == 2) ? bit : 0;
-    return blo == 0 ? 0 : -1 - x;
-  }
-  if (x >= NB && bhi >= 0) {
-    flip ^= (bhi == 2) ? bit : 0;
-    return bhi == 0 ? NB - 1 : 2 * NB - 1 - x;
-  }
-  return x;
-}
-
-static __global__ void __launch_bounds__(256) k_fill_bc(Topo t, Phys p, Pool pool, int cur, NodeSet ns, int mode) {
-  // sides: the level's boundary items, or every side of the listed nodes
+static __global__ void __launch_bounds__(256) k_fill_bc(Topo t, Phys p, Pool pool, int cur, NodeSet ns) {
+  // sides: every boundary item, or every side of the listed nodes
   int beg, cnt;
   if (ns.list) {
     beg = 0;
     cnt = 6 * ns.n;
   } else {
-    beg = t.cnt[CNT_BC + ns.level];
-    cnt = t.cnt[CNT_BC + ns.level + 1] - beg;
+    beg = t.cnt[CNT_BC];
+    cnt = t.cnt[CNT_BC + MAXL + 1] - beg;
   }
   double* buf = pool.bufp(cur);
   constexpr int NCHUNK = 9;                  // 2304 slab cells = 9 chunks of 256
@@ -327,7 +375,6 @@ static __global__ void __launch_bounds__(256) k_fill_bc(Topo t, Phys p, Pool poo
     }
     const int d = side >> 1, chunk = w % NCHUNK;
     const int level = t.level[node];
-    const bool detail_only = mode == FILL_DETAIL && t.child0[node] < 0;
     int blo[3], bhi[3];   // condition of each boundary side of this node, -1 if none (or periodic)
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
@@ -360,7 +407,6 @@ static __global__ void __launch_bounds__(256) k_fill_bc(Topo t, Phys p, Pool poo
         if (e < n) {
 #pragma unroll
           for (int v = 0; v < NV; ++v) {
-            if (detail_only && v >= 1 && v <= 3) continue;
             const double s = u[v * NCELL + si];
             val[q][v] = (v >= 1 && v <= 3 && ((flip >> (v - 1)) & 1)) ? -s : s;
           }
@@ -371,7 +417,7 @@ static __global__ void __launch_bounds__(256) k_fill_bc(Topo t, Phys p, Pool poo
         if (e0 + 32 * q < n) {
 #pragma unroll
           for (int v = 0; v < NV; ++v)
-            if (!(detail_only && v >= 1 && v <= 3)) u[v * NCELL + di[q]] = val[q][v];
+            u[v * NCELL + di[q]] = val[q][v];
         }
     }
   }
@@ -382,11 +428,18 @@ static __global__ void __launch_bounds__(256) k_fill_bc(Topo t, Phys p, Pool poo
 // cells and over rho, E of |u - P(u_parent)| / |u|.  Every leaf, and with
 // `all_nodes` every node (the tags then also read the details of the parents
 // of leaf groups).
+// Region of the fine cells of parent cell (rx, ry, rz) (-2 .. 9 relative to the child's origin).
+__device__ __forceinline__ int own_region(int rx, int ry, int rz) {
+  return (rx < 0 ? 0 : (rx < 8 ? 1 : 2)) + 3 * (ry < 0 ? 0 : (ry < 8 ? 1 : 2)) + 9 * (rz < 0 ? 0 : (rz < 8 ? 1 : 2));
+}
 template <class R>
 __global__ void __launch_bounds__(256) k_delta_t(Topo t, Phys p, Pool pool, int cur, double* __restrict__ delta_node,
                                                  int all_nodes) {
   __shared__ double sh[8];
   __shared__ R box[4096];           // the parent's cells 8 cb - 4 .. 8 cb + 11 per axis, one variable
+  __shared__ ParentBox pb;
+  __shared__ const double* own[27]; // the node's stored cells by region
+
   const int nitems = all_nodes ? t.cnt[CNT_NNODES] : t.cnt[CNT_NLEAVES];
   const double* B = pool.bufp(cur);
   for (int li = blockIdx.x; li < nitems; li += gridDim.x) {
@@ -397,10 +450,10 @@ __global__ void __launch_bounds__(256) k_delta_t(Topo t, Phys p, Pool pool, int 
       continue;
     }
     const int par = t.parent[node];
-    const double* U = B + (size_t)t.slot[node] * SLOT_U;
-    const double* P = B + (size_t)t.slot[par] * SLOT_U;
     const int ch = (int)(t.keys[node] & 7ull);
-    const int cb[3] = {ch & 1, (ch >> 1) & 1, (ch >> 2) & 1};
+    parent_box(t, p, B, par, ch, pb);
+    if (threadIdx.x < 27) own[threadIdx.x] = region_base(t, B, node, threadIdx.x);
+    __syncthreads();
     bool gl[3], gh[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
@@ -409,26 +462,31 @@ __global__ void __launch_bounds__(256) k_delta_t(Topo t, Phys p, Pool pool, int 
       gl[d] = (Xd == 0) && (p.bc[2 * d] != 1);
       gh[d] = (Xd == nl - 1) && (p.bc[2 * d + 1] != 1);
     }
-    const int bx0 = 8 * cb[0] - 4, by0 = 8 * cb[1] - 4, bz0 = 8 * cb[2] - 4;
     R m = R(0);
     for (int vi = 0; vi < 2; ++vi) {
       const int v = vi == 0 ? 0 : 4;
-      stage_box<R>(box, P + v * NCELL, bx0, by0, bz0, 16, 16, 16);
+      for (int e = threadIdx.x; e < 4096; e += blockDim.x)
+        box[e] = to_r<R>(box_value(pb, box_word(pb, e & 15, (e >> 4) & 15, e >> 8), v));
       __syncthreads();
-      const SAcc<R> A{box, bx0, by0, bz0, 16, 256};
+      const SAcc<R> A{box, 0, 0, 0, 16, 256};
       for (int q = threadIdx.x; q < 1728; q += blockDim.x) {
         const int rx = q % 12 - 2, ry = (q / 12) % 12 - 2, rz = q / 144 - 2;
         // all eight fine cells of this parent cell share the ghost status
         const bool ghost = (rx < 0 && gl[0]) || (rx >= 8 && gh[0]) || (ry < 0 && gl[1]) || (ry >= 8 && gh[1]) ||
                            (rz < 0 && gl[2]) || (rz >= 8 && gh[2]);
         if (ghost) continue;
-        const QT<R> qt = qterms_t<R>(A, 8 * cb[0] + rx, 8 * cb[1] + ry, 8 * cb[2] + rz);
+        const double* U = own[own_region(rx, ry, rz)] + v * NCELL + sidx(2 * rx, 2 * ry, 2 * rz);
+        double2 uf[4];
+#pragma unroll
+        for (int q2 = 0; q2 < 4; ++q2)
+          uf[q2] = *reinterpret_cast<const double2*>(U + ((q2 >> 1) * NS + (q2 & 1)) * NS);   // rows y + (q2 & 1), z + (q2 >> 1)
+        const QT<R> qt = qterms_t<R>(A, rx + 4, ry + 4, rz + 4);
 #pragma unroll
         for (int sub = 0; sub < 8; ++sub) {
           const int a = sub & 1, b = (sub >> 1) & 1, c = (sub >> 2) & 1;
           const R pr = predict_t<R>(qt, a ? R(-1) : R(1), b ? R(-1) : R(1), c ? R(-1) : R(1));
-          const R uf = to_r<R>(U[v * NCELL + sidx(2 * rx + a, 2 * ry + b, 2 * rz + c)]);
-          const R r = (uf - pr) / uf;
+          const R u0 = to_r<R>(a ? uf[b + 2 * c].y : uf[b + 2 * c].x);
+          const R r = (u0 - pr) / u0;
           m = (r < R(0) ? -r : r) > m ? (r < R(0) ? -r : r) : m;
         }
       }
@@ -470,7 +528,7 @@ __global__ void __launch_bounds__(256) k_refine_fill_t(Topo t, Pool pool, int cu
     const int ch = (int)(t.keys[child] & 7ull);
     const int cb[3] = {ch & 1, (ch >> 1) & 1, (ch >> 2) & 1};
     const int bx0 = 8 * cb[0] - 4, by0 = 8 * cb[1] - 4, bz0 = 8 * cb[2] - 4;
-    stage_box<R>(box, P, bx0, by0, bz0, 16, 16, 16);
+    stage_stored<R>(box, P, bx0, by0, bz0, 16, 16, 16);
     __syncthreads();
     const SAcc<R> A{box, bx0, by0, bz0, 16, 256};
     for (int r = threadIdx.x; r < 1728; r += blockDim.x) {

@@ -89,13 +89,30 @@ static __global__ void __launch_bounds__(F64_THREADS, 2)
     const int slot = t.slot[node];
     const double* __restrict__ u = src + (size_t)slot * SLOT_U;
     for (int i = warp * nsub + sub; i < F64_L; i += F64_WARPS * nsub) {
+      // beyond the block: the face neighbour's internal cells, the block's own
+      // cells mapped back at a boundary, or its stored (predicted) halo
+      int c = i - 3;
+      const double* __restrict__ cells = u;
+      bool flip = false;
+      if (c < 0 || c >= NB) {
+        const int hi = c >= NB, nb = t.nbr[(size_t)node * 27 + 13 + (hi ? 1 : -1) * (D == 0 ? 1 : (D == 1 ? 3 : 9))];
+        if (nb >= 0) {
+          cells = src + (size_t)t.slot[nb] * SLOT_U;
+          c += hi ? -NB : NB;
+        } else if (nb == -2) {
+          const bool mirror = p.bc[2 * D + hi] == 2;
+          c = mirror ? (hi ? 2 * NB - 1 - c : -1 - c) : (hi ? NB - 1 : 0);
+          flip = mirror;
+        }
+      }
       int x, y, z;
-      pencil_cell(D, pp, i - 3, x, y, z);
+      pencil_cell(D, pp, c, x, y, z);
       const int s = sidx(x, y, z);
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         const int q = (v == 0 || v == 4) ? v : 1 + (v + 2 - D) % 3;      // lab component v - 1 in the direction frame
-        cq[q * QS + (i << lp) + pl] = u[v * NCELL + s];
+        const double a = cells[v * NCELL + s];
+        cq[q * QS + (i << lp) + pl] = (flip && q == 1) ? neg64(a) : a;
       }
     }
     __syncthreads();

@@ -11,7 +11,8 @@
 // of its internal cells beside its FP64 state, written by the previous
 // stage's update; the kernel copies the records of a region into shared
 // memory with 16-byte asynchronous copies (the block's own stored halo,
-// converted from FP64, where a face has no same-level neighbour): for the x
+// converted from FP64, where a face is predicted from the parent, and its own
+// records mapped back beyond a domain boundary): for the x
 // and y directions one region holds the slab with 3 cells on each side in x
 // and in y, for z the slab with 3 planes below and above.  One thread per
 // face then computes the face flux from six records (velocity read in the
@@ -264,7 +265,10 @@ __device__ __forceinline__ RoeF roe_f32(const float* __restrict__ S, int cl, int
 }
 
 // Left eigenvector k (rotated frame): rows 0 and 4 the acoustic fields, 1 the
-// entropy field, 2 and 3 the shear fields.
+// entropy field, 2 and 3 the shear fields.  FORM: rounding of the entropy row's
+// 1 - b2 (b2 = hb1 q2), which the compiler may or may not contract depending on
+// the code around it: 0 as it likes, 1 two roundings, 2 one.
+template <int FORM = 0>
 __device__ __forceinline__ void lrow_f32(const RoeF& e, int k, float l[5]) {
   if (k == 0 || k == 4) {
     const float sg = (k == 0) ? 1.f : -1.f;
@@ -274,7 +278,7 @@ __device__ __forceinline__ void lrow_f32(const RoeF& e, int k, float l[5]) {
     l[3] = -e.hb1 * e.ut2;
     l[4] = e.hb1;
   } else if (k == 1) {
-    l[0] = 1.f - e.b2;
+    l[0] = FORM == 1 ? __fsub_rn(1.f, e.b2) : (FORM == 2 ? fmaf(-e.hb1, e.q2, 1.f) : 1.f - e.b2);
     l[1] = e.b1 * e.un;
     l[2] = e.b1 * e.ut1;
     l[3] = e.b1 * e.ut2;
@@ -482,10 +486,14 @@ __device__ __forceinline__ bool same_record(const float* __restrict__ S, int c, 
 // tells whether the six records are identical, in which case every selector
 // feature of the face is exactly zero (tested on the flux's own loads: a
 // separate test that read the 36 values again cost the selector stage 12%).
-template <int MODE, bool FLAT = false>
+// XY: the call of the x-y loop, whose linear and TENO5 variants with the Roe flux
+// round 1 - b2 twice (the others once, the LLF variants twice); fixed here so
+// that results do not depend on the compiler's choice.
+template <int MODE, bool FLAT = false, bool XY = false>
 __device__ __forceinline__ void face_flux_f32(const float* __restrict__ S, int c0, int st, Rot R, float gm1, float g,
                                               float B, bool lin, float F[5], bool* flat = nullptr) {
   constexpr int FLUX = (MODE >> 3) & 3;
+  constexpr int FORM = (FLUX == 1 || (XY && (MODE == 2 || MODE == 4))) ? 1 : 2;
   float Ur[6][5], Fr[6][5];
 #pragma unroll
   for (int m = 0; m < 6; m += 2) cell_uf2(S, c0 + m * st, c0 + (m + 1) * st, R, Ur[m], Ur[m + 1], Fr[m], Fr[m + 1]);
@@ -576,7 +584,7 @@ __device__ __forceinline__ void face_flux_f32(const float* __restrict__ S, int c
       gh = rec5<MODE>(use_lin, G[5], G[4], G[3], G[2], G[1]);
     } else {
       float l[5], V[6];
-      lrow_f32(e, k, l);
+      lrow_f32<FORM>(e, k, l);
       if (k == 2 || k == 3) {
         const int j = (k == 2) ? 2 : 3;
 #pragma unroll
@@ -766,24 +774,52 @@ __device__ __forceinline__ void cp_async_wait_all() {
 }
 
 // Sources of a slab's region: the block's FP64 stage buffer (stored cells,
-// for its predicted and boundary halo regions) and the FP32 records of the
-// internal cells of the block and of its same-level face neighbours (x-, x+,
-// y-, y+, z-, z+; null where there is none, and then the block's own halo
-// is read).  sh is null when the context keeps no records: everything is
+// for its predicted halo regions), the FP32 records of the internal cells of the
+// block and of its same-level face neighbours (x-, x+, y-, y+, z-, z+; null where
+// there is none), and the sides beyond a non-periodic boundary, whose ghost
+// cells are the block's own records mapped back (bit q of bnd; symmetric sides
+// also in mir).  Without a neighbour and a boundary bit the block's own stored
+// halo is read.  sh is null when the context keeps no records: everything is
 // then converted from the block's own stored cells.
 struct RegionSrc {
   const double* u;
   const float* sh;
   const float* nsh[6];
+  unsigned bnd, mir;
 };
+
+// Four ghost records from the block's own (x0 a multiple of four, one coordinate
+// beyond boundary side `side`) -> slots slot .. slot + 3: zero gradient takes the
+// nearest internal cell, symmetry the mirror cell with the normal velocity
+// negated -- bit for bit the records of the mapped FP64 cells.
+__device__ __forceinline__ void ghost_chunk(const RegionSrc& R, int side, int x0, int y, int z, float* __restrict__ S,
+                                            int slot) {
+  const bool mirror = (R.mir >> side) & 1u;
+  const int d = side >> 1;
+  if (d == 1) y = mirror ? ((side & 1) ? 2 * NB - 1 - y : -1 - y) : ((side & 1) ? NB - 1 : 0);
+  if (d == 2) z = mirror ? ((side & 1) ? 2 * NB - 1 - z : -1 - z) : ((side & 1) ? NB - 1 : 0);
+  const int x = d == 0 ? ((side & 1) ? NB - 4 : 0) : x0;
+  const float* src = R.sh + (z * NB + y) * NB + x;
+#pragma unroll
+  for (int f = 0; f < SF_NREC; ++f) {
+    float4 q = *reinterpret_cast<const float4*>(src + f * NINT);
+    if (d == 0) {
+      const float e = (side & 1) ? q.w : q.x;
+      q = mirror ? make_float4(q.w, q.z, q.y, q.x) : make_float4(e, e, e, e);
+    }
+    if (mirror && f == 1 + d) q = make_float4(-q.x, -q.y, -q.z, -q.w);
+    *reinterpret_cast<float4*>(S + f * SF_REG + slot) = q;
+  }
+}
 
 // Source of the chunk of four cells along x from x0 at (y, z) in block
 // coordinates (x0 a multiple of 4, at most one coordinate outside the block):
 // the FP32 records of the block or of the same-level face neighbour on that
-// side, or null (the block's own stored halo, converted from FP64).
-__device__ __forceinline__ const float* chunk_src(const RegionSrc& R, int x0, int y, int z) {
+// side, or null (ghost cells, or the block's own stored halo converted from
+// FP64); the side beyond the block (or -1) in `side`.
+__device__ __forceinline__ const float* chunk_src(const RegionSrc& R, int x0, int y, int z, int& side) {
+  side = -1;
   if (!R.sh) return nullptr;
-  int side = -1;
   if (x0 < 0) side = 0;
   else if (x0 >= NB) side = 1;
   else if (y < 0) side = 2;
@@ -807,16 +843,20 @@ __device__ __forceinline__ const float* chunk_src(const RegionSrc& R, int x0, in
 
 // The chunk at (x0, y, z) and the same chunk on the next nk - 1 planes (z + k,
 // same source block) -> slots slot + k * slot_step of S: one 16-byte
-// asynchronous copy per field and plane, or (own halo) four records
-// converted from FP64.
+// asynchronous copy per field and plane, or four ghost records, or (own halo)
+// four records converted from FP64.
 __device__ __forceinline__ void chunk_planes(const RegionSrc& R, int x0, int y, int z, int nk, float* __restrict__ S,
                                              int slot, int slot_step, float g, float B, float gm1) {
-  const float* src = chunk_src(R, x0, y, z);
+  int side;
+  const float* src = chunk_src(R, x0, y, z, side);
+  const bool ghost = !src && side >= 0 && ((R.bnd >> side) & 1u);
   for (int k = 0; k < nk; ++k) {
     if (src) {
 #pragma unroll
       for (int f = 0; f < SF_NREC; ++f)
         cp_async16(S + f * SF_REG + slot + k * slot_step, src + f * NINT + k * NB * NB);
+    } else if (ghost) {
+      ghost_chunk(R, side, x0, y, z + k, S, slot + k * slot_step);
     } else {
 #pragma unroll
       for (int c = 0; c < 4; ++c) put_record(R.u, sidx(x0 + c, y, z + k), S, slot + k * slot_step + c, g, B, gm1);
@@ -877,14 +917,20 @@ __device__ __forceinline__ void load_xy_f32(const RegionSrc& R, float* __restric
 
 // Sources of the block at `slot` with its same-level face neighbours (stage
 // buffer `cur`).
-__device__ __forceinline__ RegionSrc region_src(const Topo& t, const Pool& pool, int cur, int node, int slot) {
+__device__ __forceinline__ RegionSrc region_src(const Topo& t, const Phys& p, const Pool& pool, int cur, int node,
+                                                int slot) {
   RegionSrc R;
   R.u = pool.bufp(cur) + (size_t)slot * SLOT_U;
   R.sh = pool.shp(cur) ? pool.shp(cur) + (size_t)slot * SLOT_SH : nullptr;
+  R.bnd = R.mir = 0u;
   const int rn[6] = {12, 14, 10, 16, 4, 22};
 #pragma unroll
   for (int q = 0; q < 6; ++q) {
     const int nb = R.sh ? t.nbr[(size_t)node * 27 + rn[q]] : -1;
+    if (nb == -2) {
+      R.bnd |= 1u << q;
+      if (p.bc[q] == 2) R.mir |= 1u << q;
+    }
     R.nsh[q] = (nb >= 0) ? pool.shp(cur) + (size_t)t.slot[nb] * SLOT_SH : nullptr;
   }
   return R;
@@ -1099,7 +1145,7 @@ __device__ __forceinline__ void store_sides(int D, const float F[5], bool lo, bo
 // Per-direction sweep (the stage-0 selector variant, MODE 1): region of D,
 // faces with WENO5 fluxes and the selector's decisions, flux differences.
 template <int MODE>
-__device__ __forceinline__ void sweep_f32(int D, const Topo& t, const Pool& pool, int cur, int node, int slot,
+__device__ __forceinline__ void sweep_f32(int D, const Topo& t, const Phys& p, const Pool& pool, int cur, int node, int slot,
                                           double* __restrict__ fb, float* __restrict__ S, float* __restrict__ Fs,
                                           int z0, float g, float B, float gm1, float (&acc)[SF_TZ][NV],
                                           const LearnedCtx& L, unsigned (&cnt)[2],   // cnt: the warp's census
@@ -1108,8 +1154,8 @@ __device__ __forceinline__ void sweep_f32(int D, const Topo& t, const Pool& pool
   // the x-y region serves the x and the y faces (loaded for D = 0 and kept
   // for D = 1), the z region the z faces
   if (D != 1) {
-    if (D == 0) load_xy_f32(region_src(t, pool, cur, node, slot), S, z0, g, B, gm1);
-    else load_region_f32(2, region_src(t, pool, cur, node, slot), S, z0, g, B, gm1);
+    if (D == 0) load_xy_f32(region_src(t, p, pool, cur, node, slot), S, z0, g, B, gm1);
+    else load_region_f32(2, region_src(t, p, pool, cur, node, slot), S, z0, g, B, gm1);
     __syncthreads();
     flat = D == 0 ? probe_xy(S) : probe_z(S);
     if (flat) flat = block_and(D == 0 ? flat_xy(S, B, flat) : flat_z(S, B), flat_sh);
@@ -1202,12 +1248,12 @@ __device__ __forceinline__ void sweep_f32(int D, const Topo& t, const Pool& pool
 // stride and the rotation's offsets, so one inlined copy serves both; 1.5%
 // faster than one copy per direction).
 template <int MODE>
-__device__ __forceinline__ void sweep_xy(const double* __restrict__ u, const Topo& t, const Pool& pool, int cur,
+__device__ __forceinline__ void sweep_xy(const double* __restrict__ u, const Topo& t, const Phys& p, const Pool& pool, int cur,
                                          int node, int slot, double* __restrict__ fb, float* __restrict__ S,
                                          float* __restrict__ Fs, int z0, float g, float B, float gm1,
                                          float (&acc)[SF_TZ][NV], const LearnedCtx& L, unsigned* flat_sh) {
   const int ti = threadIdx.x & 15, tj = threadIdx.x >> 4;
-  load_xy_f32(region_src(t, pool, cur, node, slot), S, z0, g, B, gm1);
+  load_xy_f32(region_src(t, p, pool, cur, node, slot), S, z0, g, B, gm1);
   __syncthreads();
   unsigned flat = 0u;
   if (!(MODE & 32)) {                     // (viscous fluxes read other pencils)
@@ -1246,7 +1292,7 @@ __device__ __forceinline__ void sweep_xy(const double* __restrict__ u, const Top
       wi = 34 + (fy >> 5);
     }
     const bool lin = (MODE == 3) && ((L.selw[wi] >> (threadIdx.x & 31)) & 1u);
-    face_flux_f32<MODE>(S, c0, st, isx ? rot_of(0) : rot_of(1), gm1, g, B, lin, F);
+    face_flux_f32<MODE, false, true>(S, c0, st, isx ? rot_of(0) : rot_of(1), gm1, g, B, lin, F);
     if (MODE & 32) {
       if (isx) sub_viscous_f32<0>(u, sidx(fa - 1, ta, tb), L.mu, L.idx, F);
       else sub_viscous_f32<1>(u, sidx(ta, fa - 1, tb), L.mu, L.idx, F);
@@ -1268,12 +1314,12 @@ __device__ __forceinline__ void sweep_xy(const double* __restrict__ u, const Top
 
 // z direction of the slab (MODES 0, 2, 3).
 template <int MODE>
-__device__ __forceinline__ void sweep_z(const double* __restrict__ u, const Topo& t, const Pool& pool, int cur,
+__device__ __forceinline__ void sweep_z(const double* __restrict__ u, const Topo& t, const Phys& p, const Pool& pool, int cur,
                                         int node, int slot, double* __restrict__ fb, float* __restrict__ S,
                                         float* __restrict__ Fs, int z0, float g, float B, float gm1,
                                         float (&acc)[SF_TZ][NV], const LearnedCtx& L, unsigned* flat_sh) {
   const int ti = threadIdx.x & 15, tj = threadIdx.x >> 4;
-  load_region_f32(2, region_src(t, pool, cur, node, slot), S, z0, g, B, gm1);
+  load_region_f32(2, region_src(t, p, pool, cur, node, slot), S, z0, g, B, gm1);
   __syncthreads();
   bool flat = false;
   if (!(MODE & 32) && probe_z(S)) {
@@ -1375,10 +1421,10 @@ __global__ void __launch_bounds__(SF_THREADS, 2)
         for (int v = 0; v < NV; ++v) acc[kz][v] = 0.f;
       unsigned flat = 0u;
 #pragma unroll 1
-      for (int D = 0; D < 3; ++D) sweep_f32<MODE>(D, t, pool, cur, node, slot, fb, S, Fs, z0, g, B, gm1, acc, L, cnt, flat, flat_sh);
+      for (int D = 0; D < 3; ++D) sweep_f32<MODE>(D, t, p, pool, cur, node, slot, fb, S, Fs, z0, g, B, gm1, acc, L, cnt, flat, flat_sh);
     } else {
-      sweep_xy<MODE>(u, t, pool, cur, node, slot, fb, S, Fs, z0, g, B, gm1, acc, L, flat_sh);
-      sweep_z<MODE>(u, t, pool, cur, node, slot, fb, S, Fs, z0, g, B, gm1, acc, L, flat_sh);
+      sweep_xy<MODE>(u, t, p, pool, cur, node, slot, fb, S, Fs, z0, g, B, gm1, acc, L, flat_sh);
+      sweep_z<MODE>(u, t, p, pool, cur, node, slot, fb, S, Fs, z0, g, B, gm1, acc, L, flat_sh);
     }
     if (MODE == 1) {
       lvl = t.level[node];
