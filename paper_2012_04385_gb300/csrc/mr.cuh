@@ -171,32 +171,58 @@ __device__ __forceinline__ double box_value(const ParentBox& b, unsigned w, int 
   return (v >= 1 && v <= 3 && ((w >> (19 + v)) & 1u)) ? -x : x;
 }
 
+// A value c whose box of equal values predicts c: every difference and mixed
+// difference is +0, every Q-term +0, and c + (+-0) is c unless c is -0; c + c stays
+// finite.
+__device__ __forceinline__ bool const_safe(float c) {
+  return fabsf(c) < 1e30f && __float_as_uint(c) != 0x80000000u;
+}
+__device__ __forceinline__ bool const_safe(double c) {
+  return fabs(c) < 1e300 && (unsigned long long)__double_as_longlong(c) != 0x8000000000000000ull;
+}
+__device__ __forceinline__ bool same_bits(float a, float b) { return __float_as_uint(a) == __float_as_uint(b); }
+__device__ __forceinline__ bool same_bits(double a, double b) { return __double_as_longlong(a) == __double_as_longlong(b); }
+
 // Stage the cells [i0, i0+nx) x [j0, j0+ny) x [k0, k0+nz) of the box (nx, ny, nz
 // 6, 12 or 16) of every variable (or rho and E only) as R, the
 // q-th at s + q * nx ny nz; all threads.  A group of 8 or 16 lanes owns a row.
+// Returns the variables (bit q) whose cells staged by this thread all equal the
+// box's first cell.
 template <class R>
-__device__ __forceinline__ void stage_box(R* __restrict__ s, const ParentBox& b, bool detail_only, int i0, int j0,
+__device__ __forceinline__ unsigned stage_box(R* __restrict__ s, const ParentBox& b, bool detail_only, int i0, int j0,
                                           int k0, int nx, int ny, int nz) {
   const int lg = nx > 8 ? 4 : 3, i = threadIdx.x & ((1 << lg) - 1);
-  if (i >= nx) return;
+  unsigned eq = 31u;
+  if (i >= nx) return eq;
   const int n = nx * ny * nz, inv = ny == 16 ? 4096 : (ny == 12 ? 5462 : 10923);   // row / ny = row inv / 2^16 (rows < 256)
-  const unsigned wi = b.tab[0][i0 + i];
+  const unsigned wi = b.tab[0][i0 + i], w0 = box_word(b, i0, j0, k0);
+  R first[NV];
+#pragma unroll
+  for (int q = 0; q < NV; ++q)
+    if (!detail_only || q < 2) first[q] = to_r<R>(box_value(b, w0, detail_only ? 4 * q : q));
   for (int row = threadIdx.x >> lg; row < ny * nz; row += blockDim.x >> lg) {
     const int k = (row * inv) >> 16, j = row - k * ny;
     const unsigned w = wi + b.tab[1][j0 + j] + b.tab[2][k0 + k];
     const double* __restrict__ c = b.p[(w >> 16) & 7u] + (w & 0xffffu);
     R* o = s + row * nx + i;
     if (detail_only) {
-      o[0] = to_r<R>(c[0]);
-      o[n] = to_r<R>(c[4 * NCELL]);
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const R x = to_r<R>(c[4 * q * NCELL]);
+        if (!same_bits(x, first[q])) eq &= ~(1u << q);
+        o[q * n] = x;
+      }
     } else {
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        const double x = c[v * NCELL];
-        o[v * n] = to_r<R>((v >= 1 && v <= 3 && ((w >> (19 + v)) & 1u)) ? -x : x);
+        const double y = c[v * NCELL];
+        const R x = to_r<R>((v >= 1 && v <= 3 && ((w >> (19 + v)) & 1u)) ? -y : y);
+        if (!same_bits(x, first[v])) eq &= ~(1u << v);
+        o[v * n] = x;
       }
     }
   }
+  return eq;
 }
 // The same from the parent's own stored cells (halo filled).
 template <class R>
@@ -281,7 +307,9 @@ static __global__ void __launch_bounds__(256) k_fill_regions(Topo t, Pool pool, 
 // more), each taking one after the other; the parent cells of the region and
 // their +-2 stencil (6 or 12 per axis) are staged in shared memory as R for the
 // variables filled, then every thread evaluates the Q-terms of parent cells
-// and writes their eight fine cells.
+// and writes their eight fine cells.  Jumps lie where the solution is smooth, so
+// most boxes hold one value: it predicts itself (const_safe), without the 125
+// shared-memory loads of the Q-terms.
 constexpr int PRED_SPLIT = 4;
 template <class R>
 __global__ void __launch_bounds__(256) k_predict_t(Topo t, Phys p, Pool pool, int cur, const int32_t* __restrict__ list,
@@ -290,13 +318,16 @@ __global__ void __launch_bounds__(256) k_predict_t(Topo t, Phys p, Pool pool, in
   // the nodes of level n in a list grouped by level (cnt given), or n listed nodes
   __shared__ R box[NV * 864];
   __shared__ ParentBox pb;
+  __shared__ unsigned eqs[8];
   double* buf = pool.bufp(cur);
-  const int nitems = (cnt ? cnt[(mode == FILL_STAGE ? CNT_PST : CNT_PALL) + n] : n) * PRED_SPLIT;
+  const int nnode = cnt ? cnt[(mode == FILL_STAGE ? CNT_PST : CNT_PALL) + n] : n, nitems = nnode * PRED_SPLIT;
   if (cnt) list += cnt[CNT_LVL + n];
+  // (the parts of all nodes one after the other: the first holds most of the
+  // work, and must not fall to every fourth CTA only)
   for (int w = blockIdx.x; w < nitems; w += gridDim.x) {
-    const int node = list[w / PRED_SPLIT];
+    const int node = list[w % nnode];
     unsigned m = mask[node];
-    const int part = w % PRED_SPLIT;
+    const int part = w / nnode;
     if (__popc(m) <= part) continue;
     const int par = t.parent[node];
     const int ch = (int)(t.keys[node] & 7ull);
@@ -318,13 +349,24 @@ __global__ void __launch_bounds__(256) k_predict_t(Topo t, Phys p, Pool pool, in
       const int bx0 = qx0 + 2, by0 = qy0 + 2, bz0 = qz0 + 2;
       const int nx = (1 << lx) + 4, ny = (1 << ly) + 4, nz = (1 << lz) + 4;
       const int nb = nx * ny * nz;
-      stage_box<R>(box, pb, detail_only, bx0, by0, bz0, nx, ny, nz);
+      const unsigned eq = __reduce_and_sync(0xffffffffu, stage_box<R>(box, pb, detail_only, bx0, by0, bz0, nx, ny, nz));
+      if ((threadIdx.x & 31) == 0) eqs[threadIdx.x >> 5] = eq;
       __syncthreads();
+      unsigned constant = eqs[0];
+#pragma unroll
+      for (int q = 1; q < 8; ++q) constant &= eqs[q];
       const int lxy = lx + ly, ln = lxy + lz;
       for (int e = threadIdx.x; e < (nvar << ln); e += blockDim.x) {
         const int q = e >> ln, c = e & ((1 << ln) - 1);
         const int v = fill_var(detail_only, q);
         const int rx = qx0 + (c & ((1 << lx) - 1)), ry = qy0 + ((c >> lx) & ((1 << ly) - 1)), rz = qz0 + (c >> lxy);
+        if (((constant >> q) & 1u) && const_safe(box[q * nb])) {
+          const double x = from_r<R>(box[q * nb]);
+#pragma unroll
+          for (int sub = 0; sub < 4; ++sub)
+            *reinterpret_cast<double2*>(u + v * NCELL + sidx(2 * rx, 2 * ry + (sub & 1), 2 * rz + (sub >> 1))) = make_double2(x, x);
+          continue;
+        }
         const SAcc<R> A{box + q * nb, bx0, by0, bz0, nx, nx * ny};
         const QT<R> qt = qterms_t<R>(A, rx + 4, ry + 4, rz + 4);
         // the two fine cells of a row are one aligned 16-byte store
@@ -465,9 +507,14 @@ __global__ void __launch_bounds__(256) k_delta_t(Topo t, Phys p, Pool pool, int 
     R m = R(0);
     for (int vi = 0; vi < 2; ++vi) {
       const int v = vi == 0 ? 0 : 4;
-      for (int e = threadIdx.x; e < 4096; e += blockDim.x)
-        box[e] = to_r<R>(box_value(pb, box_word(pb, e & 15, (e >> 4) & 15, e >> 8), v));
-      __syncthreads();
+      const R first = to_r<R>(box_value(pb, box_word(pb, 0, 0, 0), v));
+      bool eq = const_safe(first);
+      for (int e = threadIdx.x; e < 4096; e += blockDim.x) {
+        const R x = to_r<R>(box_value(pb, box_word(pb, e & 15, (e >> 4) & 15, e >> 8), v));
+        box[e] = x;
+        eq = eq && same_bits(x, first);
+      }
+      const bool constant = __syncthreads_and(eq);       // (a box of one value predicts it)
       const SAcc<R> A{box, 0, 0, 0, 16, 256};
       for (int q = threadIdx.x; q < 1728; q += blockDim.x) {
         const int rx = q % 12 - 2, ry = (q / 12) % 12 - 2, rz = q / 144 - 2;
@@ -480,11 +527,12 @@ __global__ void __launch_bounds__(256) k_delta_t(Topo t, Phys p, Pool pool, int 
 #pragma unroll
         for (int q2 = 0; q2 < 4; ++q2)
           uf[q2] = *reinterpret_cast<const double2*>(U + ((q2 >> 1) * NS + (q2 & 1)) * NS);   // rows y + (q2 & 1), z + (q2 >> 1)
-        const QT<R> qt = qterms_t<R>(A, rx + 4, ry + 4, rz + 4);
+        QT<R> qt;
+        if (!constant) qt = qterms_t<R>(A, rx + 4, ry + 4, rz + 4);
 #pragma unroll
         for (int sub = 0; sub < 8; ++sub) {
           const int a = sub & 1, b = (sub >> 1) & 1, c = (sub >> 2) & 1;
-          const R pr = predict_t<R>(qt, a ? R(-1) : R(1), b ? R(-1) : R(1), c ? R(-1) : R(1));
+          const R pr = constant ? first : predict_t<R>(qt, a ? R(-1) : R(1), b ? R(-1) : R(1), c ? R(-1) : R(1));
           const R u0 = to_r<R>(a ? uf[b + 2 * c].y : uf[b + 2 * c].x);
           const R r = (u0 - pr) / u0;
           m = (r < R(0) ? -r : r) > m ? (r < R(0) ? -r : r) : m;
