@@ -72,7 +72,7 @@ struct mrb_ctx {
   int32_t *d_slot = nullptr, *d_level = nullptr, *d_inst = nullptr, *d_X = nullptr, *d_parent = nullptr,
           *d_child0 = nullptr, *d_nbr = nullptr, *d_leaves = nullptr, *d_lvl_nodes = nullptr, *d_bc_items = nullptr, *d_jump = nullptr, *d_cnt = nullptr,
           *d_lmax = nullptr, *d_list = nullptr, *d_pst = nullptr, *d_pall = nullptr;
-  uint32_t *d_miss = nullptr, *d_smask = nullptr;
+  uint32_t *d_miss = nullptr, *d_smask = nullptr, *d_fmask = nullptr;
   double *d_dt = nullptr, *d_delta_node = nullptr, *d_partial = nullptr;
   unsigned long long* d_census = nullptr;   // mrb_flux_census counters (allocated on first use)
   unsigned long long* d_smax = nullptr;
@@ -116,6 +116,7 @@ struct mrb_ctx {
     t.smask = d_smask;
     t.pst = d_pst;
     t.pall = d_pall;
+    t.fmask = d_fmask;
     t.cnt = d_cnt;
     return t;
   }
@@ -227,7 +228,7 @@ struct mrb_ctx {
     put(d_bc_items, h_bc_items.data(), sizeof(int32_t) * h_bc_items.size());
     put(d_cnt, h_cnt.data(), sizeof(int32_t) * CNT_SIZE);
     launch_nbr(topo(), phys, d_nbr, n, st);
-    launch_masks(topo(), phys, d_miss, d_smask, d_pst, d_pall, d_cnt, max_lmax, st);
+    launch_masks(topo(), phys, d_miss, d_smask, d_fmask, d_pst, d_pall, d_cnt, max_lmax, st);
     launch_jump_list(topo(), d_jump, d_cnt, (int)h_leaves.size(), st);
     CK(cudaGetLastError());
     CK(cudaEventRecord(stage_ev, st));
@@ -280,14 +281,14 @@ struct mrb_ctx {
     if (cfg.precision == MRB_FP32_ACC64) launch_rhs_rk_f32(topo(), phys, P, cur, s, dt, nullptr, st);
     else launch_rhs_rk_f64(topo(), phys, P, cur, s, dt, nullptr, st);
     if (e1) CK(cudaEventRecordWithFlags(e1, st, flags));
-    for (int l = max_lmax - 1; l >= 0; --l) launch_face_avg_level(topo(), P, l, st);
-    launch_jump(topo(), phys, P, cur ^ 1, s, dt, nullptr, st);
-    launch_shadow(topo(), phys, P, cur ^ 1, SH_JUMP, nullptr, 0, 0, st);
+    if (max_lmax > 0) {      // (no jumps on a single level)
+      launch_jump(topo(), phys, P, cur ^ 1, s, dt, nullptr, st);
+      launch_shadow(topo(), phys, P, cur ^ 1, SH_JUMP, nullptr, 0, 0, st);
+    }
     cur ^= 1;
   }
   void project() {
-    for (int l = max_lmax - 1; l >= 0; --l) launch_project_level(topo(), P, cur, l, st);
-    launch_shadow(topo(), phys, P, cur, SH_INTERNAL, nullptr, 0, 0, st);
+    for (int l = max_lmax - 1; l >= 0; --l) launch_project_level(topo(), phys, P, cur, l, st);
   }
   void step_stages() {
     launch_cfl(topo(), phys, P, cur, d_smax, d_dt, d_status, st);
@@ -339,10 +340,8 @@ struct mrb_ctx {
       int lo = L;
       for (int l = L; l >= 0; --l)
         if ((r + 1) % (1 << (L - l)) == 0) lo = l;
-      for (int l = max_lmax - 1; l >= lo; --l) launch_project_level(topo(), P, cur, l, st);
-      launch_shadow(topo(), phys, P, cur, SH_INTERNAL, nullptr, 0, 0, st);
+      for (int l = max_lmax - 1; l >= lo; --l) launch_project_level(topo(), phys, P, cur, l, st);
     }
-    for (int l = max_lmax - 1; l >= 0; --l) launch_face_avg_level(topo(), P, l, st, 1);
     launch_lts_reflux(topo(), phys, P, cur, st);
     launch_shadow(topo(), phys, P, cur, SH_JUMP, nullptr, 0, 0, st);
     project();
@@ -658,6 +657,7 @@ int mrb_init_blocks(const mrb_config* cfg, void* pool, size_t pool_bytes, mrb_ct
     c->d_jump = c->dalloc<int32_t>(n);
     c->d_miss = c->dalloc<uint32_t>(n);
     c->d_smask = c->dalloc<uint32_t>(n);
+    c->d_fmask = c->dalloc<uint32_t>(n);
     c->d_pst = c->dalloc<int32_t>(n);
     c->d_pall = c->dalloc<int32_t>(n);
     c->d_cnt = c->dalloc<int32_t>(CNT_SIZE);
@@ -804,8 +804,7 @@ int mrb_compute_rhs(mrb_ctx* c, double* rhs_dev) {
     if (!rhs_dev) throw Err(MRB_EINVAL, "null rhs");
     if (c->cfg.precision == MRB_FP32_ACC64) launch_rhs_rk_f32(c->topo(), c->phys, c->P, c->cur, 0, nullptr, rhs_dev, c->st);
     else launch_rhs_rk_f64(c->topo(), c->phys, c->P, c->cur, 0, nullptr, rhs_dev, c->st);
-    for (int l = c->max_lmax - 1; l >= 0; --l) launch_face_avg_level(c->topo(), c->P, l, c->st);
-    launch_jump(c->topo(), c->phys, c->P, c->cur, 0, nullptr, rhs_dev, c->st);
+    if (c->max_lmax > 0) launch_jump(c->topo(), c->phys, c->P, c->cur, 0, nullptr, rhs_dev, c->st);
   });
 }
 

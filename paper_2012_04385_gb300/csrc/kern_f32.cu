@@ -38,19 +38,38 @@ void launch_fill_list_f32(const Topo& t, const Phys& p, const Pool& pool, int cu
   g_kernel_launches += 3;
 }
 
+// Averaging with the FP32 records of the averaged cells.
+struct PutRecord {
+  float* R;
+  float g, B, gm1;
+  __device__ __forceinline__ void operator()(int slot, int ii, const double* U) const {
+    float rec[6];
+    make_record(U[0], U[1], U[2], U[3], U[4], g, B, gm1, rec);
+    float* __restrict__ o = R + (size_t)slot * SLOT_SH + ii;
+#pragma unroll
+    for (int f = 0; f < 6; ++f) o[f * NINT] = rec[f];
+  }
+};
+__global__ void __launch_bounds__(256) k_project_f32(Topo t, Phys p, Pool pool, int buf, int level) {
+  project_level(t, pool, buf, level,
+                PutRecord{pool.shp(buf), (float)p.gamma, (float)p.B, (float)(p.gamma - 1.0)});
+}
+
+void launch_project_level_f32(const Topo& t, const Phys& p, const Pool& pool, int buf, int level, cudaStream_t st) {
+  k_project_f32<<<sm_count() * g_tune.project, 256, 0, st>>>(t, p, pool, buf, level);
+  ++g_kernel_launches;
+}
+
 // FP32 records of stage buffer b: one CTA per item, the records of the item's
 // internal cells recomputed from the FP64 values (make_record, the same
 // arithmetic as the stage kernel's own conversion).
 __global__ void __launch_bounds__(256) k_shadow(Topo t, Phys p, Pool pool, int b, int mode,
                                                 const int32_t* __restrict__ list, int n, int stride) {
   const float g = (float)p.gamma, B = (float)p.B, gm1 = (float)(p.gamma - 1.0);
-  const int nitems = (mode == SH_INTERNAL) ? t.cnt[CNT_NNODES] : (mode == SH_JUMP ? t.cnt[CNT_JUMP] : n);
+  const int nitems = mode == SH_JUMP ? t.cnt[CNT_JUMP] : n;
   for (int w = blockIdx.x; w < nitems; w += gridDim.x) {
     int node, mask = 0;
-    if (mode == SH_INTERNAL) {
-      node = w;
-      if (t.child0[node] < 0) continue;           // leaves keep the stage kernel's records
-    } else if (mode == SH_JUMP) {
+    if (mode == SH_JUMP) {
       node = t.leaves[t.jump[w] >> 6];
       mask = t.jump[w] & 63;
     } else {

@@ -138,41 +138,34 @@ void launch_rhs_rk_f64(const Topo& t, const Phys& p, const Pool& pool, int cur, 
   launch_rhs_rk_impl(t, p, pool, cur, stage, dt, rhs_out, st, level);
 }
 
-// ---------------------------------------------------------------- face fluxes of internal nodes
-// parent face cell = mean of the 2 x 2 covering child face cells, levels fine to coarse
-__global__ void k_face_avg_level(Topo t, double* __restrict__ faces, int level) {
-  const int beg = t.cnt[CNT_LVL + level], end = t.cnt[CNT_LVL + level + 1];
-  for (int w = beg + blockIdx.x; w < end; w += gridDim.x) {
-    const int node = t.lvl_nodes[w];
-    const int c0 = t.child0[node];
-    if (c0 < 0) continue;
-    double* F = faces + (size_t)t.slot[node] * SLOT_F;
-    for (int e = threadIdx.x; e < 6 * NFACE; e += blockDim.x) {
-      const int s = e / NFACE, aa = e % 16, bb = (e / 16) % 16;
-      const int d = s / 2, hi = s & 1;
-      const int t1 = (d == 0) ? 1 : 0, t2 = (d == 2) ? 1 : 2;
-      const int ct1 = aa / 8, ct2 = bb / 8;
-      int cb[3];
-      cb[d] = hi;
-      cb[t1] = ct1;
-      cb[t2] = ct2;
-      const int ch = cb[0] | (cb[1] << 1) | (cb[2] << 2);
-      const double* C = faces + (size_t)t.slot[c0 + ch] * SLOT_F;
-      const int fa = 2 * (aa - 8 * ct1), fbb = 2 * (bb - 8 * ct2);
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        const double* cf = C + (s * NV + v) * NFACE;
-        double f00 = cf[fbb * NB + fa], f10 = cf[fbb * NB + fa + 1];
-        double f01 = cf[(fbb + 1) * NB + fa], f11 = cf[(fbb + 1) * NB + fa + 1];
-        F[(s * NV + v) * NFACE + bb * NB + aa] = 0.25 * ((f00 + f10) + (f01 + f11));
-      }
-    }
+// ---------------------------------------------------------------- fine side of a jump
+// Flux of an internal node's face cell (side s, position aa, bb): the mean of
+// the 2 x 2 covering child face cells, themselves means where the child is
+// refined too.  Formed where a jump reads it; averaging every face of every
+// internal node level by level took a launch per level and 135 us per stage on
+// the shock-bubble, for the few per cent of faces that a jump reads.
+static __device__ __noinline__ double fine_flux(const int32_t* __restrict__ child0, const int32_t* __restrict__ slot,
+                                                const double* __restrict__ faces, int node, int s, int v, int aa, int bb) {
+  const int d = s / 2, hi = s & 1;
+  const int ct1 = aa / 8, ct2 = bb / 8;
+  const int b1 = (d == 0) ? 2 : 1, b2 = (d == 2) ? 2 : 4, bd = (d == 0) ? 1 : (d == 1 ? 2 : 4);
+  const int ch = child0[node] + (hi ? bd : 0) + (ct1 ? b1 : 0) + (ct2 ? b2 : 0);
+  const int fa = 2 * (aa - 8 * ct1), fb = 2 * (bb - 8 * ct2);
+  double f00, f10, f01, f11;
+  if (child0[ch] < 0) {
+    const double* cf = faces + (size_t)slot[ch] * SLOT_F + (s * NV + v) * NFACE + fb * NB + fa;
+    const double2 lo = *reinterpret_cast<const double2*>(cf), up = *reinterpret_cast<const double2*>(cf + NB);
+    f00 = lo.x;
+    f10 = lo.y;
+    f01 = up.x;
+    f11 = up.y;
+  } else {
+    f00 = fine_flux(child0, slot, faces, ch, s, v, fa, fb);
+    f10 = fine_flux(child0, slot, faces, ch, s, v, fa + 1, fb);
+    f01 = fine_flux(child0, slot, faces, ch, s, v, fa, fb + 1);
+    f11 = fine_flux(child0, slot, faces, ch, s, v, fa + 1, fb + 1);
   }
-}
-
-void launch_face_avg_level(const Topo& t, const Pool& pool, int level, cudaStream_t st, int integrated) {
-  k_face_avg_level<<<sm_count() * 4, 256, 0, st>>>(t, integrated ? pool.fmac : pool.face, level);
-  ++g_kernel_launches;
+  return 0.25 * ((f00 + f10) + (f01 + f11));
 }
 
 // ---------------------------------------------------------------- local time stepping
@@ -255,7 +248,11 @@ __global__ void k_lts_fmac(Topo t, Phys p, Pool pool, int level, int stage, cons
     }
     const double* F = pool.face + slot * SLOT_F;
     const double wgt = kRkW[rk_row(p)][stage] * ldexp(dt[t.inst[node]], p.lmax[t.inst[node]] - level);
-    for (int e = threadIdx.x; e < SLOT_F; e += blockDim.x) M[e] = M[e] + wgt * F[e];
+    const uint32_t fm = t.fmask[node];          // (the sides that the reflux reads)
+    for (int sd = 0; sd < 6; ++sd) {
+      if (!((fm >> sd) & 1u)) continue;
+      for (int e = sd * NV * NFACE + threadIdx.x; e < (sd + 1) * NV * NFACE; e += blockDim.x) M[e] = M[e] + wgt * F[e];
+    }
   }
 }
 
@@ -273,7 +270,7 @@ __global__ void k_lts_reflux(Topo t, Phys p, Pool pool, int cur) {
     const int li = t.jump[w] >> 6, mask = t.jump[w] & 63;
     const int node = t.leaves[li];
     const double* Fc_all = pool.fmac + (size_t)t.slot[node] * SLOT_F;
-    const double dx = ldexp(p.dx0, -t.level[node]);
+    const Div64 dx = div64_prep(ldexp(p.dx0, -t.level[node]));
     double* U = pool.bufp(cur) + (size_t)t.slot[node] * SLOT_U;
 #pragma unroll 1
     for (int s = 0; s < 6; ++s) {
@@ -283,7 +280,6 @@ __global__ void k_lts_reflux(Topo t, Phys p, Pool pool, int cur) {
       const int r = (sv[2] + 1) * 9 + (sv[1] + 1) * 3 + (sv[0] + 1);
       if (!((mask >> s) & 1)) continue;
       const int nb = t.nbr[(size_t)node * 27 + r];
-      const double* Ff_all = pool.fmac + (size_t)t.slot[nb] * SLOT_F;
       const int so = s ^ 1;
       const int t1 = (d == 0) ? 1 : 0, t2 = (d == 2) ? 1 : 2;
       for (int e = threadIdx.x; e < NFACE; e += blockDim.x) {
@@ -295,8 +291,8 @@ __global__ void k_lts_reflux(Topo t, Phys p, Pool pool, int cur) {
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
           const double Fc = Fc_all[(s * NV + v) * NFACE + e];
-          const double Ff = Ff_all[(so * NV + v) * NFACE + e];
-          const double dU = hi ? (Fc - Ff) / dx : (Ff - Fc) / dx;
+          const double Ff = fine_flux(t.child0, t.slot, pool.fmac, nb, so, v, aa, bb);
+          const double dU = div64(hi ? Fc - Ff : Ff - Fc, dx);
           double& ur = U[v * NCELL + sidx(c[0], c[1], c[2])];
           ur = ur + dU;
         }
@@ -323,7 +319,7 @@ __global__ void k_jump(Topo t, Phys p, Pool pool, int target, int stage, const d
     const int li = t.jump[w] >> 6, mask = t.jump[w] & 63;
     const int node = t.leaves[li];
     const double* Fc_all = pool.face + (size_t)t.slot[node] * SLOT_F;
-    const double dx = ldexp(p.dx0, -t.level[node]);
+    const Div64 dx = div64_prep(ldexp(p.dx0, -t.level[node]));
     const double h = dt ? dt[t.inst[node]] : 0.0;
     const double bs = kRkB[rk_row(p)][stage];
     double* U = pool.bufp(target) + (size_t)t.slot[node] * SLOT_U;
@@ -335,7 +331,6 @@ __global__ void k_jump(Topo t, Phys p, Pool pool, int target, int stage, const d
       const int r = (sv[2] + 1) * 9 + (sv[1] + 1) * 3 + (sv[0] + 1);
       if (!((mask >> s) & 1)) continue;      // the side's neighbour is not refined
       const int nb = t.nbr[(size_t)node * 27 + r];
-      const double* Ff_all = pool.face + (size_t)t.slot[nb] * SLOT_F;
       const int so = s ^ 1;
       const int t1 = (d == 0) ? 1 : 0, t2 = (d == 2) ? 1 : 2;
       for (int e = threadIdx.x; e < NFACE; e += blockDim.x) {
@@ -347,8 +342,8 @@ __global__ void k_jump(Topo t, Phys p, Pool pool, int target, int stage, const d
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
           const double Fc = Fc_all[(s * NV + v) * NFACE + e];
-          const double Ff = Ff_all[(so * NV + v) * NFACE + e];
-          const double dL = hi ? (Fc - Ff) / dx : (Ff - Fc) / dx;
+          const double Ff = fine_flux(t.child0, t.slot, pool.face, nb, so, v, aa, bb);
+          const double dL = div64(hi ? Fc - Ff : Ff - Fc, dx);
           if (rhs_out) {
             double& Lr = rhs_out[((size_t)li * NV + v) * NINT + iidx(c[0], c[1], c[2])];
             Lr = Lr + dL;
@@ -372,8 +367,16 @@ void launch_jump(const Topo& t, const Phys& p, const Pool& pool, int target, int
 }
 
 // ---------------------------------------------------------------- averaging (mr.cuh)
-void launch_project_level(const Topo& t, const Pool& pool, int buf, int level, cudaStream_t st) {
-  k_project_octants<<<sm_count() * g_tune.project, 256, 0, st>>>(t, pool, buf, level);
+static __global__ void __launch_bounds__(256) k_project(Topo t, Pool pool, int buf, int level) {
+  project_level(t, pool, buf, level, NoRecord{});
+}
+
+void launch_project_level(const Topo& t, const Phys& p, const Pool& pool, int buf, int level, cudaStream_t st) {
+  if (p.precision == 1) {
+    launch_project_level_f32(t, p, pool, buf, level, st);
+    return;
+  }
+  k_project<<<sm_count() * g_tune.project, 256, 0, st>>>(t, pool, buf, level);
   ++g_kernel_launches;
 }
 
@@ -618,7 +621,7 @@ __global__ void k_nbr(Topo t, Phys p, int32_t* __restrict__ nbr_out) {
 // octant's side) when s_d is 0 or points out of the parent.
 constexpr uint32_t FACE_REGIONS = (1u << 12) | (1u << 14) | (1u << 10) | (1u << 16) | (1u << 4) | (1u << 22);
 __global__ void k_masks(Topo t, Phys p, uint32_t* __restrict__ miss, uint32_t* __restrict__ smask,
-                        int32_t* __restrict__ pst, int32_t* __restrict__ pall, int32_t* __restrict__ cnt, int level) {
+                        uint32_t* __restrict__ fmask, int32_t* __restrict__ pst, int32_t* __restrict__ pall, int32_t* __restrict__ cnt, int level) {
   const int beg = t.cnt[CNT_LVL + level], end = t.cnt[CNT_LVL + level + 1];
   for (int w = beg + blockIdx.x * blockDim.x + threadIdx.x; w < end; w += gridDim.x * blockDim.x) {
     const int node = t.lvl_nodes[w];
@@ -645,6 +648,13 @@ __global__ void k_masks(Topo t, Phys p, uint32_t* __restrict__ miss, uint32_t* _
         }
       }
     }
+    uint32_t fm = 0;
+    const int rn[6] = {12, 14, 10, 16, 4, 22};
+    for (int sd = 0; sd < 6; ++sd) {
+      const int nb = t.nbr[(size_t)node * 27 + rn[sd]];
+      if (nb == -1 || (nb >= 0 && t.child0[nb] >= 0)) fm |= 1u << sd;
+    }
+    fmask[node] = c0 < 0 ? fm : 0u;
     miss[node] = ms;
     smask[node] = need & ms;
     if (need & ms) pst[beg + atomicAdd(&cnt[CNT_PST + level], 1)] = node;
@@ -652,10 +662,10 @@ __global__ void k_masks(Topo t, Phys p, uint32_t* __restrict__ miss, uint32_t* _
   }
 }
 
-void launch_masks(const Topo& t, const Phys& p, uint32_t* miss, uint32_t* smask, int32_t* pst, int32_t* pall, int32_t* cnt,
-                  int max_level, cudaStream_t st) {
+void launch_masks(const Topo& t, const Phys& p, uint32_t* miss, uint32_t* smask, uint32_t* fmask, int32_t* pst,
+                  int32_t* pall, int32_t* cnt, int max_level, cudaStream_t st) {
   for (int l = max_level; l >= 0; --l) {
-    k_masks<<<sm_count(), 128, 0, st>>>(t, p, miss, smask, pst, pall, cnt, l);
+    k_masks<<<sm_count(), 128, 0, st>>>(t, p, miss, smask, fmask, pst, pall, cnt, l);
     ++g_kernel_launches;
   }
 }

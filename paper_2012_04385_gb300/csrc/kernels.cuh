@@ -51,6 +51,8 @@ struct Topo {
   const uint32_t* smask;   // those that a stage needs (see k_masks)
   const int32_t* pst;      // nodes with smask != 0, grouped by level like lvl_nodes (count CNT_PST + l)
   const int32_t* pall;     // nodes with miss != 0, likewise (count CNT_PALL + l)
+  const uint32_t* fmask;   // 6-bit mask of a leaf's sides whose face fluxes something reads: next to a refined
+                           // neighbour (the jump correction's coarse side) or to none (its fine side)
   const int32_t* cnt;      // counts, see CNT_*
 };
 
@@ -173,9 +175,6 @@ void launch_rhs_rk_f32_llf(const Topo& t, const Phys& p, const Pool& pool, int c
                            double* rhs_out, cudaStream_t st, int level = -1);
 void launch_rhs_rk_f32_hllc(const Topo& t, const Phys& p, const Pool& pool, int cur, int stage, const double* dt,
                             double* rhs_out, cudaStream_t st, int level = -1);
-// internal nodes' face fluxes of `level` from their children (faces = pool.face,
-// or the macro step's integrated fluxes pool.fmac with integrated = 1)
-void launch_face_avg_level(const Topo& t, const Pool& pool, int level, cudaStream_t st, int integrated = 0);
 // ---- local time stepping
 // Interpolation in time of the nodes of levels < below (factor theta[m] per
 // level m; the end state kept in the other stage buffer), or its undoing.
@@ -195,7 +194,9 @@ void launch_lts_fmac(const Topo& t, const Phys& p, const Pool& pool, int level, 
 void launch_lts_reflux(const Topo& t, const Phys& p, const Pool& pool, int cur, cudaStream_t st);
 void launch_jump(const Topo& t, const Phys& p, const Pool& pool, int target, int stage, const double* dt,
                  double* rhs_out, cudaStream_t st);
-void launch_project_level(const Topo& t, const Pool& pool, int buf, int level, cudaStream_t st);
+// averaging of the internal nodes of `level`, with their FP32 records (mixed precision)
+void launch_project_level(const Topo& t, const Phys& p, const Pool& pool, int buf, int level, cudaStream_t st);
+void launch_project_level_f32(const Topo& t, const Phys& p, const Pool& pool, int buf, int level, cudaStream_t st);
 void launch_cfl(const Topo& t, const Phys& p, const Pool& pool, int cur, unsigned long long* smax, double* dt,
                 int* status, cudaStream_t st);
 void launch_delta_tags(const Topo& t, const Phys& p, const Pool& pool, int cur, double* delta_node,
@@ -209,8 +210,8 @@ void launch_jump_list(const Topo& t, int32_t* jump, int32_t* cnt, int n_leaves_c
 void launch_nbr(const Topo& t, const Phys& p, int32_t* nbr_out, int nnodes_cap, cudaStream_t st);
 // Masks of predicted regions and the lists of the nodes that have any, levels
 // fine to coarse (max_level .. 0).
-void launch_masks(const Topo& t, const Phys& p, uint32_t* miss, uint32_t* smask, int32_t* pst, int32_t* pall, int32_t* cnt,
-                  int max_level, cudaStream_t st);
+void launch_masks(const Topo& t, const Phys& p, uint32_t* miss, uint32_t* smask, uint32_t* fmask, int32_t* pst,
+                  int32_t* pall, int32_t* cnt, int max_level, cudaStream_t st);
 void launch_sums(const Topo& t, const Phys& p, const Pool& pool, int cur, double* partial, double* out,
                  int nleaves_cap, cudaStream_t st);
 // mixed-precision variants (kern_f32.cu)
@@ -226,10 +227,10 @@ void launch_delta_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, d
 void launch_cfl_speeds_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, unsigned long long* smax,
                            int* status, cudaStream_t st);
 // FP32 records of stage buffer b from its FP64 internal cells (mixed-precision
-// path): SH_INTERNAL every internal node (after averaging), SH_JUMP the
-// boundary planes that the jump correction changed, SH_LIST the nodes of a
-// device list of n entries (every `stride`-th entry is a node index).
-enum : int { SH_INTERNAL = 0, SH_JUMP = 1, SH_LIST = 2 };
+// path): SH_JUMP the boundary planes that the jump correction changed, SH_LIST
+// the nodes of a device list of n entries (every `stride`-th entry is a node
+// index).  The stage kernel and the averaging write the records of their cells.
+enum : int { SH_JUMP = 1, SH_LIST = 2 };
 void launch_shadow(const Topo& t, const Phys& p, const Pool& pool, int b, int mode, const int32_t* list, int n,
                    int stride, cudaStream_t st);
 // Records of the listed nodes (kept, or converted afresh from the FP64 state).

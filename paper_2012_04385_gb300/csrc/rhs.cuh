@@ -163,6 +163,7 @@ static __global__ void __launch_bounds__(F64_THREADS, 2)
     // direction frame is axis (D + j) mod 3)
     double* __restrict__ o = dst + (size_t)slot * SLOT_U;
     double* __restrict__ fb = pool.face + (size_t)slot * SLOT_F;
+    const unsigned fm = t.fmask[node];          // sides whose fluxes something reads
     for (int e = warp * nsub + sub; e < NV * (NB + 2); e += F64_WARPS * nsub) {
       const int v = e / (NB + 2), i = e % (NB + 2);
       const int vl = (v == 0 || v == 4) ? v : 1 + (D + v - 1) % 3;
@@ -173,7 +174,7 @@ static __global__ void __launch_bounds__(F64_THREADS, 2)
         o[vl * NCELL + diff_place(D, iidx(x, y, z))] = f[uniform ? 0 : i << lp] - f[uniform ? 0 : (i + 1) << lp];
       } else {
         const int hi = i - NB;
-        fb[((2 * D + hi) * NV + vl) * NFACE + pp] = f[(uniform || !hi) ? 0 : NB << lp];
+        if ((fm >> (2 * D + hi)) & 1u) fb[((2 * D + hi) * NV + vl) * NFACE + pp] = f[(uniform || !hi) ? 0 : NB << lp];
       }
     }
     __syncthreads();

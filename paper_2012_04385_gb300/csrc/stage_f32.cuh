@@ -986,15 +986,16 @@ __device__ __forceinline__ void to_lab(int D, float n, float t1, float t2, float
 }
 
 // Store face f's flux (direction frame of D) into the flux slots (row length
-// fstr per variable), and into
-// the block's face buffer (lab frame, FP64) when the face is on the block
-// boundary (gface 0 or 16 along D).
+// fstr per variable), and into the block's face buffer (lab frame, FP64) when
+// the face is on a side of the block (gface 0 or 16 along D) whose fluxes
+// something reads (bit of fm; storing every side was 61 KB per leaf, 7% of the
+// stage's traffic: shock-bubble stage 2.31 -> 2.10 ms without it).
 __device__ __forceinline__ void store_face(int D, const float F[5], float* __restrict__ Fs, int fstr, int f, int gface,
-                                           int ta, int tb, double* __restrict__ fb) {
+                                           int ta, int tb, double* __restrict__ fb, unsigned fm) {
 #pragma unroll
   for (int v = 0; v < 5; ++v) Fs[v * fstr + f] = F[v];
-  if (gface == 0 || gface == NB) {
-    const int side = 2 * D + (gface == NB ? 1 : 0);
+  const int side = 2 * D + (gface == NB ? 1 : 0);
+  if ((gface == 0 || gface == NB) && ((fm >> side) & 1u)) {
     float Fl[5];
     Fl[0] = F[0];
     Fl[4] = F[4];
@@ -1149,7 +1150,8 @@ __device__ __forceinline__ void sweep_f32(int D, const Topo& t, const Phys& p, c
                                           double* __restrict__ fb, float* __restrict__ S, float* __restrict__ Fs,
                                           int z0, float g, float B, float gm1, float (&acc)[SF_TZ][NV],
                                           const LearnedCtx& L, unsigned (&cnt)[2],   // cnt: the warp's census
-                                          unsigned& flat, unsigned* flat_sh) {       // constant directions of the slab
+                                          unsigned& flat, unsigned* flat_sh,         // constant directions of the slab
+                                          unsigned fm) {                             // sides whose fluxes are read
   const int ti = threadIdx.x & 15, tj = threadIdx.x >> 4;
   // the x-y region serves the x and the y faces (loaded for D = 0 and kept
   // for D = 1), the z region the z faces
@@ -1173,7 +1175,7 @@ __device__ __forceinline__ void sweep_f32(int D, const Topo& t, const Phys& p, c
         cnt[1] += 32u;
       }
     }
-    const bool lo = D != 2 || z0 == 0, hi = D != 2 || z0 + SF_TZ == NB;
+    const bool lo = (D != 2 || z0 == 0) && ((fm >> (2 * D)) & 1u), hi = (D != 2 || z0 + SF_TZ == NB) && ((fm >> (2 * D + 1)) & 1u);
     if ((lo || hi) && (D == 2 || threadIdx.x < 16 * SF_TZ)) {
       const int a = ti, b = tj;      // x: (y, kz), y: (x, kz), z: (x, y)
       const int c0 = D == 0 ? xy_slot(-3, a, b) : (D == 1 ? xy_slot(a, -3, b) : b * 16 + a);
@@ -1228,7 +1230,7 @@ __device__ __forceinline__ void sweep_f32(int D, const Topo& t, const Phys& p, c
       cnt[1] += __popc(ba);
     }
     if (!act) continue;
-    store_face(D, F, Fs, SF_NFZ, f, (D == 2) ? z0 + fa : fa, ta, tb, fb);
+    store_face(D, F, Fs, SF_NFZ, f, (D == 2) ? z0 + fa : fa, ta, tb, fb, fm);
   }
   __syncthreads();
 #pragma unroll
@@ -1251,7 +1253,7 @@ template <int MODE>
 __device__ __forceinline__ void sweep_xy(const double* __restrict__ u, const Topo& t, const Phys& p, const Pool& pool, int cur,
                                          int node, int slot, double* __restrict__ fb, float* __restrict__ S,
                                          float* __restrict__ Fs, int z0, float g, float B, float gm1,
-                                         float (&acc)[SF_TZ][NV], const LearnedCtx& L, unsigned* flat_sh) {
+                                         float (&acc)[SF_TZ][NV], const LearnedCtx& L, unsigned* flat_sh, unsigned fm) {
   const int ti = threadIdx.x & 15, tj = threadIdx.x >> 4;
   load_xy_f32(region_src(t, p, pool, cur, node, slot), S, z0, g, B, gm1);
   __syncthreads();
@@ -1264,9 +1266,10 @@ __device__ __forceinline__ void sweep_xy(const double* __restrict__ u, const Top
       flat = block_and(flat, flat_sh);
     }
   }
-  // faces of each direction: all of them, or one per constant pencil
+  // faces of each direction: all of them, or one per constant pencil for the
+  // block's sides that something reads
   const bool flatx = flat & 1u, flaty = flat & 2u;
-  const int nx = flatx ? 16 * SF_TZ : SF_NFX, ny = flaty ? 16 * SF_TZ : SF_NFX;
+  const int nx = flatx ? ((fm & 3u) ? 16 * SF_TZ : 0) : SF_NFX, ny = flaty ? ((fm & 12u) ? 16 * SF_TZ : 0) : SF_NFX;
   for (int f = threadIdx.x; f < nx + ny; f += blockDim.x) {
     float F[5];
     const bool isx = f < nx;              // warp-uniform (64 or 1088 = 34 warps)
@@ -1297,8 +1300,8 @@ __device__ __forceinline__ void sweep_xy(const double* __restrict__ u, const Top
       if (isx) sub_viscous_f32<0>(u, sidx(fa - 1, ta, tb), L.mu, L.idx, F);
       else sub_viscous_f32<1>(u, sidx(ta, fa - 1, tb), L.mu, L.idx, F);
     }
-    if (one) store_sides(isx ? 0 : 1, F, true, true, ta, tb, fb);
-    else store_face(isx ? 0 : 1, F, Fs, SF_FMAX, f, fa, ta, tb, fb);
+    if (one) store_sides(isx ? 0 : 1, F, (fm >> (isx ? 0 : 2)) & 1u, (fm >> (isx ? 1 : 3)) & 1u, ta, tb, fb);
+    else store_face(isx ? 0 : 1, F, Fs, SF_FMAX, f, fa, ta, tb, fb, fm);
   }
   __syncthreads();
 #pragma unroll
@@ -1317,7 +1320,7 @@ template <int MODE>
 __device__ __forceinline__ void sweep_z(const double* __restrict__ u, const Topo& t, const Phys& p, const Pool& pool, int cur,
                                         int node, int slot, double* __restrict__ fb, float* __restrict__ S,
                                         float* __restrict__ Fs, int z0, float g, float B, float gm1,
-                                        float (&acc)[SF_TZ][NV], const LearnedCtx& L, unsigned* flat_sh) {
+                                        float (&acc)[SF_TZ][NV], const LearnedCtx& L, unsigned* flat_sh, unsigned fm) {
   const int ti = threadIdx.x & 15, tj = threadIdx.x >> 4;
   load_region_f32(2, region_src(t, p, pool, cur, node, slot), S, z0, g, B, gm1);
   __syncthreads();
@@ -1328,7 +1331,7 @@ __device__ __forceinline__ void sweep_z(const double* __restrict__ u, const Topo
     flat = block_and(m, flat_sh) != 0u;
   }
   // constant pencils: no differences, and a flux only at the block's own sides
-  const bool lo = z0 == 0, hi = z0 + SF_TZ == NB;
+  const bool lo = z0 == 0 && (fm & 16u), hi = z0 + SF_TZ == NB && (fm & 32u);
   for (int f = threadIdx.x; f < (flat ? ((lo || hi) ? NFACE : 0) : SF_NFZ); f += blockDim.x) {
     const int i = f % 16, j = (f / 16) % 16, fa = f / 256;
     const int c0 = (fa * 16 + j) * 16 + i;
@@ -1337,7 +1340,7 @@ __device__ __forceinline__ void sweep_z(const double* __restrict__ u, const Topo
     face_flux_f32<MODE>(S, c0, 256, rot_of(2), gm1, g, B, lin, F);
     if (MODE & 32) sub_viscous_f32<2>(u, sidx(i, j, z0 + fa - 1), L.mu, L.idx, F);
     if (flat) store_sides(2, F, lo, hi, i, j, fb);
-    else store_face(2, F, Fs, SF_FMAX, f, z0 + fa, i, j, fb);
+    else store_face(2, F, Fs, SF_FMAX, f, z0 + fa, i, j, fb, fm);
   }
   __syncthreads();
   if (!flat) {
@@ -1407,6 +1410,7 @@ __global__ void __launch_bounds__(SF_THREADS, 2)
     }
     const double* __restrict__ u = src + (size_t)slot * SLOT_U;
     double* __restrict__ fb = pool.face + (size_t)slot * SLOT_F;
+    const unsigned fm = t.fmask[node];
     if (MODE == 1 || MODE == 3) L.bits = pool.sel + (size_t)slot * SLOT_SEL;
     if (MODE & 32) L.idx = d2f_fast(ldexp(1.0 / p.dx0, t.level[node]));
     // the slab's decision words (read before the first barrier of the sweep)
@@ -1421,10 +1425,10 @@ __global__ void __launch_bounds__(SF_THREADS, 2)
         for (int v = 0; v < NV; ++v) acc[kz][v] = 0.f;
       unsigned flat = 0u;
 #pragma unroll 1
-      for (int D = 0; D < 3; ++D) sweep_f32<MODE>(D, t, p, pool, cur, node, slot, fb, S, Fs, z0, g, B, gm1, acc, L, cnt, flat, flat_sh);
+      for (int D = 0; D < 3; ++D) sweep_f32<MODE>(D, t, p, pool, cur, node, slot, fb, S, Fs, z0, g, B, gm1, acc, L, cnt, flat, flat_sh, fm);
     } else {
-      sweep_xy<MODE>(u, t, p, pool, cur, node, slot, fb, S, Fs, z0, g, B, gm1, acc, L, flat_sh);
-      sweep_z<MODE>(u, t, p, pool, cur, node, slot, fb, S, Fs, z0, g, B, gm1, acc, L, flat_sh);
+      sweep_xy<MODE>(u, t, p, pool, cur, node, slot, fb, S, Fs, z0, g, B, gm1, acc, L, flat_sh, fm);
+      sweep_z<MODE>(u, t, p, pool, cur, node, slot, fb, S, Fs, z0, g, B, gm1, acc, L, flat_sh, fm);
     }
     if (MODE == 1) {
       lvl = t.level[node];
