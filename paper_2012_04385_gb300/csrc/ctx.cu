@@ -768,8 +768,7 @@ int mrb_set_cons(mrb_ctx* c, const uint64_t* keys_host, int64_t n, const double*
     if (n < 0 || (n > 0 && (!keys_host || !cons_dev))) throw Err(MRB_EINVAL, "bad arguments");
     std::vector<int32_t> v = c->nodes_of(keys_host, n);
     c->upload_list(v);
-    launch_set_cons(c->topo(), c->P, c->cur, c->d_list, (int)n, cons_dev, c->st);
-    launch_shadow(c->topo(), c->phys, c->P, c->cur, SH_LIST, c->d_list, (int)n, 1, c->st);
+    launch_set_cons(c->topo(), c->phys, c->P, c->cur, c->d_list, (int)n, cons_dev, c->st);
     c->list_used();
   });
 }

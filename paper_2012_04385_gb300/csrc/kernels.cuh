@@ -151,8 +151,11 @@ __device__ __forceinline__ double ldexp_(double x, int e) { return ldexp(x, e); 
 // (defined in kern_f64.cu / kern_f32.cu; all asynchronous on `st`)
 void launch_set_state(const Topo& t, const Phys& p, const Pool& pool, int cur, const int32_t* nodes, int n,
                       const double* prim, cudaStream_t st);
-void launch_set_cons(const Topo& t, const Pool& pool, int cur, const int32_t* nodes, int n, const double* cons,
-                     cudaStream_t st);
+// (with the FP32 records of the cells, mixed precision)
+void launch_set_cons(const Topo& t, const Phys& p, const Pool& pool, int cur, const int32_t* nodes, int n,
+                     const double* cons, cudaStream_t st);
+void launch_set_cons_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, const int32_t* nodes, int n,
+                         const double* cons, cudaStream_t st);
 void launch_get_state(const Topo& t, const Pool& pool, int cur, const int32_t* nodes, int n, double* out,
                       int with_halo, cudaStream_t st);
 // stored halos facing same-level nodes, and ghost cells beyond the boundary, of every node

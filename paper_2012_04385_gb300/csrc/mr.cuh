@@ -606,9 +606,17 @@ __global__ void __launch_bounds__(256) k_refine_fill_t(Topo t, Pool pool, int cu
 // (internal node, octant): the octant's 512 parent cells come from one child.
 // A thread forms all five variables of a parent cell (twenty 16-byte loads in
 // flight) and, on the mixed-precision path (REC), its FP32 record, which a
-// kernel of its own used to read the average back for.  Bound by reading eight
-// children per cell; shock-bubble (levels 0..4): averaging and records 450 ->
-// 393 us per stage.
+// kernel of its own used to read the average back for.  Bound by the FP64 pipe
+// (eight instructions per value) where the children differ, by reading them
+// where they do not; shock-bubble (levels 0..4): averaging and records 450 ->
+// 301 us per stage.
+// A 16-byte load that stays where it is written (the compiler moved the loads of
+// later variables behind the arithmetic of earlier ones: four in flight).
+__device__ __forceinline__ double2 load_now(const double* p) {
+  double2 x;
+  asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(x.x), "=d"(x.y) : "l"(p));
+  return x;
+}
 struct NoRecord {
   __device__ __forceinline__ void operator()(int, int, const double*) const {}
 };
@@ -632,16 +640,24 @@ static __device__ __forceinline__ void project_level(const Topo& t, const Pool& 
       for (int v = 0; v < NV; ++v) {
         // 2 I is even: each x-pair of children is one aligned 16-byte load
         const double* u = C + v * NCELL + sidx(2 * I, 2 * J, 2 * K);
-        a[v][0] = *reinterpret_cast<const double2*>(u);
-        a[v][1] = *reinterpret_cast<const double2*>(u + NS);
-        a[v][2] = *reinterpret_cast<const double2*>(u + NS * NS);
-        a[v][3] = *reinterpret_cast<const double2*>(u + NS * NS + NS);
+        a[v][0] = load_now(u);
+        a[v][1] = load_now(u + NS);
+        a[v][2] = load_now(u + NS * NS);
+        a[v][3] = load_now(u + NS * NS + NS);
       }
       double U[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        U[v] = 0.125 * (((a[v][0].x + a[v][0].y) + (a[v][1].x + a[v][1].y)) +
-                        ((a[v][2].x + a[v][2].y) + (a[v][3].x + a[v][3].y)));
+        // eight equal values have themselves as mean (2x, 4x, 8x and x/8 are
+        // exact, but for overflow): the sums are FP64-pipe work (eight
+        // instructions of 16 cycles a warp), the comparison is not
+        const unsigned long long x = d2bits(a[v][0].x);
+        const bool same = x == d2bits(a[v][0].y) && x == d2bits(a[v][1].x) && x == d2bits(a[v][1].y) &&
+                          x == d2bits(a[v][2].x) && x == d2bits(a[v][2].y) && x == d2bits(a[v][3].x) &&
+                          x == d2bits(a[v][3].y) && ((x >> 52) & 2047u) < 2040u;
+        if (same) U[v] = a[v][0].x;
+        else U[v] = 0.125 * (((a[v][0].x + a[v][0].y) + (a[v][1].x + a[v][1].y)) +
+                             ((a[v][2].x + a[v][2].y) + (a[v][3].x + a[v][3].y)));
         Pp[v * NCELL + sidx(ox + I, oy + J, oz + K)] = U[v];
       }
       rec(slot, iidx(ox + I, oy + J, oz + K), U);
