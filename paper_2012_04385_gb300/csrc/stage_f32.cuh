@@ -754,15 +754,6 @@ __device__ __forceinline__ void make_record(double r64, double mx64, double my64
   rec[5] = E;
 }
 
-// One FP32 primitive record from the FP64 conserved state at s.
-__device__ __forceinline__ void put_record(const double* __restrict__ src, int s, float* __restrict__ S, int idx,
-                                           float g, float B, float gm1) {
-  float rec[6];
-  make_record(src[s], src[NCELL + s], src[2 * NCELL + s], src[3 * NCELL + s], src[4 * NCELL + s], g, B, gm1, rec);
-#pragma unroll
-  for (int f = 0; f < SF_NREC; ++f) S[f * SF_REG + idx] = rec[f];
-}
-
 // 16-byte asynchronous copy from global to shared memory (L2 only); both
 // addresses 16-byte aligned.
 __device__ __forceinline__ void cp_async16(float* smem, const float* gmem) {
@@ -841,26 +832,52 @@ __device__ __forceinline__ const float* chunk_src(const RegionSrc& R, int x0, in
   return n + (z * NB + y) * NB + x0;
 }
 
-// The chunk at (x0, y, z) and the same chunk on the next nk - 1 planes (z + k,
+// The chunk at (x0, y, z) and the same chunk on the next NK - 1 planes (z + k,
 // same source block) -> slots slot + k * slot_step of S: one 16-byte
 // asynchronous copy per field and plane, or four ghost records, or (own halo)
 // four records converted from FP64.
-__device__ __forceinline__ void chunk_planes(const RegionSrc& R, int x0, int y, int z, int nk, float* __restrict__ S,
+// A 16-byte load that stays where it is written.
+__device__ __forceinline__ double2 load_pair_now(const double* p) {
+  double2 x;
+  asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(x.x), "=d"(x.y) : "l"(p));
+  return x;
+}
+template <int NK>
+__device__ __forceinline__ void chunk_planes(const RegionSrc& R, int x0, int y, int z, float* __restrict__ S,
                                              int slot, int slot_step, float g, float B, float gm1) {
   int side;
   const float* src = chunk_src(R, x0, y, z, side);
-  const bool ghost = !src && side >= 0 && ((R.bnd >> side) & 1u);
-  for (int k = 0; k < nk; ++k) {
-    if (src) {
+  if (src) {
+#pragma unroll
+    for (int k = 0; k < NK; ++k)
 #pragma unroll
       for (int f = 0; f < SF_NREC; ++f)
         cp_async16(S + f * SF_REG + slot + k * slot_step, src + f * NINT + k * NB * NB);
-    } else if (ghost) {
-      ghost_chunk(R, side, x0, y, z + k, S, slot + k * slot_step);
-    } else {
+  } else if (side >= 0 && ((R.bnd >> side) & 1u)) {
 #pragma unroll
-      for (int c = 0; c < 4; ++c) put_record(R.u, sidx(x0 + c, y, z + k), S, slot + k * slot_step + c, g, B, gm1);
-    }
+    for (int k = 0; k < NK; ++k) ghost_chunk(R, side, x0, y, z + k, S, slot + k * slot_step);
+  } else {
+    // every load of the chunk's planes before the first conversion: one
+    // memory latency, not one per plane (x0 even: aligned pairs)
+    double2 q[NK][2][NV];
+#pragma unroll
+    for (int k = 0; k < NK; ++k)
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+          q[k][h][v] = load_pair_now(R.u + v * NCELL + sidx(x0 + 2 * h, y, z + k));
+#pragma unroll
+    for (int k = 0; k < NK; ++k)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        float rec[6];
+        const int h = c >> 1;
+        if (c & 1) make_record(q[k][h][0].y, q[k][h][1].y, q[k][h][2].y, q[k][h][3].y, q[k][h][4].y, g, B, gm1, rec);
+        else make_record(q[k][h][0].x, q[k][h][1].x, q[k][h][2].x, q[k][h][3].x, q[k][h][4].x, g, B, gm1, rec);
+#pragma unroll
+        for (int f = 0; f < SF_NREC; ++f) S[f * SF_REG + slot + k * slot_step + c] = rec[f];
+      }
   }
 }
 
@@ -874,19 +891,19 @@ __device__ __forceinline__ void load_region_f32(int D, const RegionSrc& R, float
   if (D == 0) {                 // 96 chunk positions per plane (16 rows of 6), two planes per thread
     if (t < 192) {
       const int c = t % 96, kz = t / 96, y = c / 6, q = c % 6;
-      chunk_planes(R, 4 * q - 4, y, z0 + kz, 1, S, (kz * 16 + y) * 24 + 4 * q, 0, g, B, gm1);
-      chunk_planes(R, 4 * q - 4, y, z0 + kz + 2, 1, S, ((kz + 2) * 16 + y) * 24 + 4 * q, 0, g, B, gm1);
+      chunk_planes<1>(R, 4 * q - 4, y, z0 + kz, S, (kz * 16 + y) * 24 + 4 * q, 0, g, B, gm1);
+      chunk_planes<1>(R, 4 * q - 4, y, z0 + kz + 2, S, ((kz + 2) * 16 + y) * 24 + 4 * q, 0, g, B, gm1);
     }
   } else if (D == 1) {          // 88 chunk positions per plane (22 rows of 4), two planes per thread
     if (t < 176) {
       const int c = t % 88, kz = t / 88, r = c / 4, q = c % 4;
-      chunk_planes(R, 4 * q, r - 3, z0 + kz, 1, S, (kz * 22 + r) * 16 + 4 * q, 0, g, B, gm1);
-      chunk_planes(R, 4 * q, r - 3, z0 + kz + 2, 1, S, ((kz + 2) * 22 + r) * 16 + 4 * q, 0, g, B, gm1);
+      chunk_planes<1>(R, 4 * q, r - 3, z0 + kz, S, (kz * 22 + r) * 16 + 4 * q, 0, g, B, gm1);
+      chunk_planes<1>(R, 4 * q, r - 3, z0 + kz + 2, S, ((kz + 2) * 22 + r) * 16 + 4 * q, 0, g, B, gm1);
     }
   } else {                      // 64 chunk positions per plane, planes t/64, +4, +8 (ten planes)
     const int c = t % 64, lane = t / 64, y = c / 4, q = c % 4;
     for (int zz = lane; zz < SF_TZ + 6; zz += 4)
-      chunk_planes(R, 4 * q, y, z0 - 3 + zz, 1, S, (zz * 16 + y) * 16 + 4 * q, 0, g, B, gm1);
+      chunk_planes<1>(R, 4 * q, y, z0 - 3 + zz, S, (zz * 16 + y) * 16 + 4 * q, 0, g, B, gm1);
   }
   cp_async_wait_all();
 }
@@ -910,7 +927,7 @@ __device__ __forceinline__ void load_xy_f32(const RegionSrc& R, float* __restric
       y = (r < 3) ? r - 3 : r + 13;
       x0 = 4 * ((c - 96) % 4);
     }
-    chunk_planes(R, x0, y, z0 + kz, 2, S, xy_slot(x0, y, kz), xy_slot(0, 0, 1) - xy_slot(0, 0, 0), g, B, gm1);
+    chunk_planes<2>(R, x0, y, z0 + kz, S, xy_slot(x0, y, kz), xy_slot(0, 0, 1) - xy_slot(0, 0, 0), g, B, gm1);
   }
   cp_async_wait_all();
 }
