@@ -1,6 +1,7 @@
 // Learned reconstruction selector: training-data generation from the solver's
 // own faces, training (forward and backward of the BF16-operand perceptron
 // with FP32 accumulation, Adam), and tensor-core inference.  See learned.cuh.
+#include <cstddef>
 #include <cstring>
 #include <algorithm>
 
@@ -137,7 +138,8 @@ void launch_face_samples(const Topo& t, const Phys& p, const Pool& pool, int cur
 }
 
 // ---------------------------------------------------------------- training
-constexpr int TR_T = 128;                 // samples per tile = threads per CTA
+constexpr int TR_T = 128;                 // samples per tile
+constexpr int TR_Q = 4;                    // threads per sample
 constexpr int TR_GRID_MAX = 512;
 constexpr int TR_LD = 33;                  // padded row length of the activation tiles
 constexpr size_t TR_SMEM = sizeof(float) * (MLP_NPARAM + (MLP_NPARAM + 1) + TR_T * 16 + 6 * TR_T * TR_LD + TR_T);
@@ -152,12 +154,16 @@ __device__ __forceinline__ float gelu_grad_acc(float z) {
   return 0.5f * (1.f + t) + 0.5f * z * (1.f - t * t) * GELU_K0 * (1.f + 3.f * GELU_K1 * z * z);
 }
 
-// Per CTA: forward and backward of its sample tiles (one thread per sample),
-// then each thread sums its gradient entries over the tile's samples in a
-// fixed order.  Writes the CTA's gradient and loss sums to work[cta].
-__global__ void __launch_bounds__(TR_T) k_mlp_grad(const float* __restrict__ P, const float* __restrict__ X,
-                                                   const uint8_t* __restrict__ Y, int64_t n, float posw,
-                                                   float* __restrict__ work) {
+// Per CTA: forward and backward of its sample tiles (four threads per sample,
+// eight units of a layer each), then each thread sums its gradient entries over
+// the tile's samples in a fixed order.  Writes the CTA's gradient and loss sums
+// to work[cta].  Every sum keeps one thread and its order; what bounds the kernel
+// is the latency of those chains at one CTA per SM, so the units are spread over
+// threads: with one thread per sample (4 warps) a batch of 16,384 took 38 us, so
+// 23 us.
+__global__ void __launch_bounds__(TR_T * TR_Q) k_mlp_grad(const float* __restrict__ P, const float* __restrict__ X,
+                                                          const uint8_t* __restrict__ Y, int64_t n, float posw,
+                                                          float* __restrict__ work) {
   extern __shared__ __align__(16) float tr[];
   float* Wr = tr;                               // weights rounded to BF16, biases FP32
   float* gacc = Wr + MLP_NPARAM;                // gradient + loss accumulator
@@ -169,6 +175,7 @@ __global__ void __launch_bounds__(TR_T) k_mlp_grad(const float* __restrict__ P, 
   float* z1 = d2 + TR_T * TR_LD;                // pre-activations [T][33]
   float* z2 = z1 + TR_T * TR_LD;
   float* d3 = z2 + TR_T * TR_LD;                // [T]
+  constexpr int U = MLP_H / TR_Q;               // units per thread
   for (int e = threadIdx.x; e < MLP_NPARAM; e += blockDim.x) {
     const bool is_bias = (e >= OFF_B1 && e < OFF_W2) || (e >= OFF_B2 && e < OFF_W3) || e == OFF_B3;
     Wr[e] = is_bias ? P[e] : bf16_round(P[e]);
@@ -177,32 +184,37 @@ __global__ void __launch_bounds__(TR_T) k_mlp_grad(const float* __restrict__ P, 
   __syncthreads();
   const float inv_n = 1.0f / (float)n;
   const int64_t ntiles = (n + TR_T - 1) / TR_T;
+  // a warp holds one quarter of the units of 32 samples: its weight reads are broadcasts
+  const int s = threadIdx.x % TR_T, o0 = (threadIdx.x / TR_T) * U;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int s = threadIdx.x;
     const int64_t gi = tile * TR_T + s;
     const bool act = gi < n;
     float x[16];
 #pragma unroll
     for (int k = 0; k < 16; ++k) x[k] = (act && k < MLP_IN) ? bf16_round(X[gi * 16 + k]) : 0.f;
+    if (o0 == 0) {
 #pragma unroll
-    for (int k = 0; k < 16; ++k) xs[s * 16 + k] = x[k];
-#pragma unroll 1
-    for (int o = 0; o < MLP_H; ++o) {
+      for (int k = 0; k < 16; ++k) xs[s * 16 + k] = x[k];
+    }
+#pragma unroll 2
+    for (int o = o0; o < o0 + U; ++o) {
       float a = Wr[OFF_B1 + o];
 #pragma unroll
       for (int k = 0; k < MLP_IN; ++k) a = fmaf(Wr[OFF_W1 + o * MLP_IN + k], x[k], a);
       z1[s * TR_LD + o] = a;
       h1[s * TR_LD + o] = bf16_round(gelu_acc(a));
     }
-#pragma unroll 1
-    for (int o = 0; o < MLP_H; ++o) {
+    __syncthreads();
+#pragma unroll 2
+    for (int o = o0; o < o0 + U; ++o) {
       float a = Wr[OFF_B2 + o];
 #pragma unroll 8
       for (int k = 0; k < MLP_H; ++k) a = fmaf(Wr[OFF_W2 + o * MLP_H + k], h1[s * TR_LD + k], a);
       z2[s * TR_LD + o] = a;
       h2[s * TR_LD + o] = bf16_round(gelu_acc(a));
     }
-    float z3 = Wr[OFF_B3];
+    __syncthreads();
+    float z3 = Wr[OFF_B3];                      // (by each of the sample's threads alike)
 #pragma unroll 8
     for (int k = 0; k < MLP_H; ++k) z3 = fmaf(Wr[OFF_W3 + k], h2[s * TR_LD + k], z3);
     float dz3 = 0.f, loss = 0.f;
@@ -213,21 +225,26 @@ __global__ void __launch_bounds__(TR_T) k_mlp_grad(const float* __restrict__ P, 
       const float sig = 1.f / (1.f + expf(-z3));
       dz3 = w * (sig - y) * inv_n;
     }
-    d3[s] = dz3;
-#pragma unroll 1
-    for (int o = 0; o < MLP_H; ++o) d2[s * TR_LD + o] = dz3 * Wr[OFF_W3 + o] * gelu_grad_acc(z2[s * TR_LD + o]);
-#pragma unroll 1
-    for (int k = 0; k < MLP_H; ++k) {
+    if (o0 == 0) {
+      d3[s] = dz3;
+      xs[s * 16 + 15] = loss;
+    }
+#pragma unroll 2
+    for (int o = o0; o < o0 + U; ++o) d2[s * TR_LD + o] = dz3 * Wr[OFF_W3 + o] * gelu_grad_acc(z2[s * TR_LD + o]);
+    __syncthreads();
+#pragma unroll 2
+    for (int k = o0; k < o0 + U; ++k) {
       float a = 0.f;
 #pragma unroll 8
       for (int o = 0; o < MLP_H; ++o) a = fmaf(Wr[OFF_W2 + o * MLP_H + k], d2[s * TR_LD + o], a);
       d1[s * TR_LD + k] = a * gelu_grad_acc(z1[s * TR_LD + k]);
     }
-    // loss of the tile in a fixed order (thread 0)
-    xs[s * 16 + 15] = loss;
     __syncthreads();
-    if (threadIdx.x == 0) {
+    // loss of the tile in a fixed order (one thread of the last warp, which has
+    // the fewest gradient entries)
+    if (threadIdx.x == blockDim.x - 1) {
       float ls = 0.f;
+#pragma unroll 8
       for (int q = 0; q < TR_T; ++q) ls += xs[q * 16 + 15];
       gacc[MLP_NPARAM] += ls;
     }
@@ -236,20 +253,26 @@ __global__ void __launch_bounds__(TR_T) k_mlp_grad(const float* __restrict__ P, 
       float a = 0.f;
       if (e < OFF_B1) {
         const int o = e / MLP_IN, k = e % MLP_IN;
-        for (int q = 0; q < TR_T; ++q) a = fmaf(d1[q * TR_LD + o], (k == 15) ? 0.f : xs[q * 16 + k], a);
+#pragma unroll 8
+        for (int q = 0; q < TR_T; ++q) a = fmaf(d1[q * TR_LD + o], xs[q * 16 + k], a);
       } else if (e < OFF_W2) {
         const int o = e - OFF_B1;
+#pragma unroll 8
         for (int q = 0; q < TR_T; ++q) a += d1[q * TR_LD + o];
       } else if (e < OFF_B2) {
         const int o = (e - OFF_W2) / MLP_H, k = (e - OFF_W2) % MLP_H;
+#pragma unroll 8
         for (int q = 0; q < TR_T; ++q) a = fmaf(d2[q * TR_LD + o], h1[q * TR_LD + k], a);
       } else if (e < OFF_W3) {
         const int o = e - OFF_B2;
+#pragma unroll 8
         for (int q = 0; q < TR_T; ++q) a += d2[q * TR_LD + o];
       } else if (e < OFF_B3) {
         const int k = e - OFF_W3;
+#pragma unroll 8
         for (int q = 0; q < TR_T; ++q) a = fmaf(d3[q], h2[q * TR_LD + k], a);
       } else {
+#pragma unroll 8
         for (int q = 0; q < TR_T; ++q) a += d3[q];
       }
       gacc[e] += a;
@@ -266,6 +289,7 @@ __global__ void k_mlp_adam(float* __restrict__ P, float* __restrict__ m, float* 
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e > MLP_NPARAM) return;
   float gsum = 0.f;
+#pragma unroll 16
   for (int b = 0; b < nblk; ++b) gsum += work[(size_t)b * (MLP_NPARAM + 1) + e];
   if (e == MLP_NPARAM) {
     if (loss_out) *loss_out = gsum / (float)n;
@@ -323,7 +347,7 @@ extern "C" int mrb_mlp_logits(const float* params_dev, const float* feats_dev, i
 
 // ---------------------------------------------------------------- threshold
 // Order statistics of the logits of label-1 samples by radix selection on
-// the float's order-preserving 32-bit key, eight bits per pass (most
+// the float's order-preserving 32-bit key, six or seven bits per pass (most
 // significant first): each pass histograms the next digit of the keys that
 // share the digits chosen so far.
 __device__ __forceinline__ uint32_t order_key(float x) {
@@ -337,51 +361,99 @@ static float key_value(uint32_t k) {
   return x;
 }
 
-__global__ void __launch_bounds__(256) k_key_hist(const float* __restrict__ z, const uint8_t* __restrict__ y,
-                                                  int64_t n, uint32_t prefix, int shift,
-                                                  unsigned long long* __restrict__ hist) {
-  __shared__ unsigned int h[256];
-  h[threadIdx.x] = 0;
+// Selection state in the caller's scratch (MRB_THRESHOLD_WORK uint64): 128 bins
+// and the words below.
+constexpr int KS_BINS = 128;
+struct KeySelect {
+  unsigned long long bins[KS_BINS];
+  unsigned long long rank;        // of the wanted key among those that share the prefix
+  unsigned long long m;           // label-1 samples
+  unsigned long long ticket;      // CTAs done with the pass
+  uint32_t prefix;                // digits chosen so far
+  uint32_t next;                  // smallest key above the selected one
+  uint32_t want_next;             // the following order statistic lies above the selected key
+};
+static_assert(sizeof(KeySelect) <= MRB_THRESHOLD_WORK * sizeof(uint64_t), "selection state fits the caller's scratch");
+
+// The position of the q-quantile among m values: its lower order statistic.
+__host__ __device__ inline int64_t quantile_index(int64_t m, double q) { return (int64_t)((double)(m - 1) * q); }
+
+// One digit (bits shift .. shift + width - 1): every CTA adds its histogram of the
+// keys that share the chosen prefix, the last one to finish picks the bin that
+// holds the wanted rank.  (The first pass counts the samples and derives the
+// rank from q.)  A pass is launch and latency.  With the host
+// reading each histogram back, a threshold took up to twelve passes with a fill, a
+// copy and a round trip each: 64 us of device time for 131,073 logits, 29 us in six
+// launches and one copy.
+__global__ void __launch_bounds__(256) k_key_select(const float* __restrict__ z, const uint8_t* __restrict__ y, int64_t n,
+                                                    double q, int shift, int width, KeySelect* __restrict__ S) {
+  __shared__ unsigned int h[KS_BINS];
+  __shared__ bool last;
+  if (threadIdx.x < KS_BINS) h[threadIdx.x] = 0;
+  const int top = shift + width;                 // bits from here up are chosen
+  const uint32_t prefix = S->prefix;
   __syncthreads();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     if (!y[i]) continue;
     const uint32_t k = order_key(z[i]);
-    if (shift < 24 && (k >> (shift + 8)) != (prefix >> (shift + 8))) continue;
-    atomicAdd(&h[(k >> shift) & 255u], 1u);
+    if (top < 32 && (k >> top) != (prefix >> top)) continue;
+    atomicAdd(&h[(k >> shift) & ((1u << width) - 1u)], 1u);
   }
   __syncthreads();
-  if (h[threadIdx.x]) atomicAdd(&hist[threadIdx.x], (unsigned long long)h[threadIdx.x]);
-}
-
-// The kth smallest (from 0) label-1 logit; *m receives the number of label-1
-// samples (from the first pass).
-static int select_kth(const float* z, const uint8_t* y, int64_t n, int64_t kth, unsigned long long* hist,
-                      cudaStream_t st, float* out, int64_t* m) {
-  const int grid = (int)std::min<int64_t>((n + 255) / 256, (int64_t)sm_count() * 4);
-  uint32_t prefix = 0;
-  unsigned long long h[256];
-  for (int shift = 24; shift >= 0; shift -= 8) {
-    if (cudaMemsetAsync(hist, 0, 256 * sizeof(unsigned long long), st) != cudaSuccess) return MRB_ECUDA;
-    k_key_hist<<<grid, 256, 0, st>>>(z, y, n, prefix, shift, hist);
-    ++g_kernel_launches;
-    if (cudaMemcpyAsync(h, hist, sizeof h, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
-      return MRB_ECUDA;
-    if (shift == 24) {
-      int64_t total = 0;
-      for (int d = 0; d < 256; ++d) total += (int64_t)h[d];
-      *m = total;
-      if (kth >= total) return MRB_EINVAL;
-    }
-    int d = 0;
-    for (; d < 256; ++d) {
-      if (kth < (int64_t)h[d]) break;
-      kth -= (int64_t)h[d];
-    }
-    prefix |= (uint32_t)d << shift;
+  if (threadIdx.x < KS_BINS && h[threadIdx.x]) atomicAdd(&S->bins[threadIdx.x], (unsigned long long)h[threadIdx.x]);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(&S->ticket, 1ull) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (threadIdx.x >= 32) return;
+  // four bins per lane and a scan over the lanes
+  unsigned long long c[KS_BINS / 32], own = 0;
+#pragma unroll
+  for (int i = 0; i < KS_BINS / 32; ++i) {
+    c[i] = __ldcg(&S->bins[threadIdx.x * (KS_BINS / 32) + i]);
+    S->bins[threadIdx.x * (KS_BINS / 32) + i] = 0;
+    own += c[i];
   }
-  *out = key_value(prefix);
-  return MRB_OK;
+  unsigned long long upto = own;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long v = __shfl_up_sync(0xffffffffu, upto, o);
+    if (threadIdx.x >= o) upto += v;
+  }
+  const unsigned long long m = __shfl_sync(0xffffffffu, upto, 31);
+  unsigned long long rank = S->rank;
+  if (top == 32) rank = m ? (unsigned long long)quantile_index((int64_t)m, q) : 0;
+  __syncwarp();                                  // (S->rank is read by every lane before one writes it)
+  if (threadIdx.x == 0) {
+    if (top == 32) S->m = m;
+    S->next = 0xffffffffu;
+    S->ticket = 0;
+  }
+  // one lane's bins hold the rank (none where there is no sample at all)
+  if (rank < upto && rank >= upto - own) {
+    rank -= upto - own;
+    int d = 0;
+    while (rank >= c[d]) rank -= c[d++];
+    S->prefix = prefix | ((uint32_t)(threadIdx.x * (KS_BINS / 32) + d) << shift);
+    S->rank = rank;
+    if (shift == 0) S->want_next = rank + 1 >= c[d];     // the selected key's copies end here
+  }
+}
+// The smallest key above the selected one, if the next order statistic needs it.
+__global__ void __launch_bounds__(256) k_key_next(const float* __restrict__ z, const uint8_t* __restrict__ y, int64_t n,
+                                                  KeySelect* __restrict__ S) {
+  if (!S->want_next) return;
+  const uint32_t key = S->prefix;
+  uint32_t best = 0xffffffffu;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    if (!y[i]) continue;
+    const uint32_t k = order_key(z[i]);
+    if (k > key && k < best) best = k;
+  }
+  best = __reduce_min_sync(0xffffffffu, best);
+  if ((threadIdx.x & 31) == 0 && best != 0xffffffffu) atomicMin(&S->next, best);
 }
 
 extern "C" int mrb_mlp_threshold(const float* logits_dev, const uint8_t* labels_dev, int64_t n, double q,
@@ -391,21 +463,28 @@ extern "C" int mrb_mlp_threshold(const float* logits_dev, const uint8_t* labels_
   *tau_out = 0.f;
   if (n == 0) return MRB_OK;
   cudaStream_t st = (cudaStream_t)stream;
-  unsigned long long* hist = reinterpret_cast<unsigned long long*>(work_dev);
-  // count the label-1 samples with a first selection of the smallest one
-  float lo = 0.f;
-  int64_t m = 0;
-  int rc = select_kth(logits_dev, labels_dev, n, 0, hist, st, &lo, &m);
-  if (rc == MRB_EINVAL && m == 0) return MRB_OK;     // no label-1 sample: threshold 0
-  if (rc != MRB_OK) return rc;
+  KeySelect* S = reinterpret_cast<KeySelect*>(work_dev);
+  const int grid = (int)std::min<int64_t>((n + 1023) / 1024, (int64_t)sm_count() * 4);
+  if (cudaMemsetAsync(S, 0, sizeof(KeySelect), st) != cudaSuccess) return MRB_ECUDA;
+  const int shifts[5] = {25, 18, 12, 6, 0}, widths[5] = {7, 7, 6, 6, 6};
+  for (int d = 0; d < 5; ++d)
+    k_key_select<<<grid, 256, 0, st>>>(logits_dev, labels_dev, n, q, shifts[d], widths[d], S);
+  k_key_next<<<grid, 256, 0, st>>>(logits_dev, labels_dev, n, S);
+  g_kernel_launches += 6;
+  KeySelect h;
+  if (cudaGetLastError() != cudaSuccess ||
+      cudaMemcpyAsync((char*)&h + offsetof(KeySelect, rank), (char*)S + offsetof(KeySelect, rank),
+                      sizeof(KeySelect) - offsetof(KeySelect, rank), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+      cudaStreamSynchronize(st) != cudaSuccess)
+    return MRB_ECUDA;
+  const int64_t m = (int64_t)h.m;
+  if (m == 0) return MRB_OK;                         // no label-1 sample: threshold 0
   // linear interpolation between the order statistics around (m - 1) q
   const double pos = (double)(m - 1) * q;
-  const int64_t k = (int64_t)pos;
+  const int64_t k = quantile_index(m, q);
   const float frac = (float)(pos - (double)k);
-  float a = lo, b = lo;
-  if (k > 0 && (rc = select_kth(logits_dev, labels_dev, n, k, hist, st, &a, &m)) != MRB_OK) return rc;
-  b = a;
-  if (k + 1 < m && (rc = select_kth(logits_dev, labels_dev, n, k + 1, hist, st, &b, &m)) != MRB_OK) return rc;
+  const float a = key_value(h.prefix);
+  const float b = (k + 1 < m && h.want_next) ? key_value(h.next) : a;
   *tau_out = a + frac * (b - a);
   return MRB_OK;
 }
@@ -423,8 +502,8 @@ extern "C" int mrb_mlp_train_step(float* params_dev, float* adam_m_dev, float* a
   const int64_t ntiles = (n + TR_T - 1) / TR_T;
   const int grid = (int)std::min<int64_t>(ntiles, (int64_t)std::min(TR_GRID_MAX, sm_count() * 3));
   cudaStream_t st = (cudaStream_t)stream;
-  k_mlp_grad<<<grid, TR_T, TR_SMEM, st>>>(params_dev, feats_dev, labels_dev, n, pos_weight, work_dev);
-  k_mlp_adam<<<(MLP_NPARAM + 1 + 255) / 256, 256, 0, st>>>(params_dev, adam_m_dev, adam_v_dev, t_step, work_dev, grid,
+  k_mlp_grad<<<grid, TR_T * TR_Q, TR_SMEM, st>>>(params_dev, feats_dev, labels_dev, n, pos_weight, work_dev);
+  k_mlp_adam<<<(MLP_NPARAM + 1 + 63) / 64, 64, 0, st>>>(params_dev, adam_m_dev, adam_v_dev, t_step, work_dev, grid,
                                                            lr, loss_dev, grad_dev, n);
   g_kernel_launches += 2;
   return cudaGetLastError() == cudaSuccess ? MRB_OK : MRB_ECUDA;
