@@ -29,6 +29,13 @@ void launch_predict_f32(const Topo& t, const Phys& p, const Pool& pool, int cur,
   ++g_kernel_launches;
 }
 
+void launch_predict_lts_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, int dst, int level, double th,
+                            cudaStream_t st) {
+  k_predict_t<float, true><<<sm_count() * g_tune.fill_pred, 256, 0, st>>>(t, p, pool, cur, t.pst, t.cnt, level, t.smask,
+                                                                          FILL_STAGE, dst, th);
+  ++g_kernel_launches;
+}
+
 void launch_fill_list_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, const int32_t* list, int n,
                           cudaStream_t st) {
   const NodeSet ns{list, n};

@@ -162,6 +162,17 @@ void launch_predict(const Topo& t, const Phys& p, const Pool& pool, int cur, int
   ++g_kernel_launches;
 }
 
+void launch_predict_lts(const Topo& t, const Phys& p, const Pool& pool, int cur, int dst, int level, double th,
+                        cudaStream_t st) {
+  if (p.precision == 1) {
+    launch_predict_lts_f32(t, p, pool, cur, dst, level, th, st);
+    return;
+  }
+  k_predict_t<double, true><<<sm_count() * g_tune.fill_pred, 256, 0, st>>>(t, p, pool, cur, t.pst, t.cnt, level, t.smask,
+                                                                           FILL_STAGE, dst, th);
+  ++g_kernel_launches;
+}
+
 void launch_fill_list(const Topo& t, const Phys& p, const Pool& pool, int cur, const int32_t* list, int n,
                       cudaStream_t st) {
   if (n <= 0) return;
@@ -251,58 +262,78 @@ void launch_lts_interp(const Topo& t, const Pool& pool, int cur, int below, cons
   ++g_kernel_launches;
 }
 
-// Internal cells (and FP32 records) of the nodes of `level`: cur^1 -> cur.
-__global__ void k_lts_copyback(Topo t, Pool pool, int cur, int level) {
+// Internal cells (and FP32 records) of the nodes of `level`: cur^1 -> cur.  Items
+// are 2048 16-byte words of a node (a variable, or a third of the records), every
+// thread with its eight in flight: a level has few nodes, and with one CTA per node
+// and a word per pass each took 74 us on the shock-bubble with levels 1 and 2 (360
+// nodes), so 18 us.
+__global__ void __launch_bounds__(256) k_lts_copyback(Topo t, Pool pool, int cur, int level) {
   const int beg = t.cnt[CNT_LVL + level], end = t.cnt[CNT_LVL + level + 1];
-  for (int w = beg + blockIdx.x; w < end; w += gridDim.x) {
-    const size_t slot = (size_t)t.slot[t.lvl_nodes[w]];
-    double* U = pool.bufp(cur) + slot * SLOT_U;
-    const double* O = pool.bufp(cur ^ 1) + slot * SLOT_U;
-    for (int e = threadIdx.x; e < NV * NINT; e += blockDim.x) {
-      const int v = e / NINT, ii = e % NINT;
-      const int s = v * NCELL + sidx(ii % 16, (ii / 16) % 16, ii / 256);
-      U[s] = O[s];
+  const int parts = pool.shp(0) ? 8 : NV;
+  for (int w = blockIdx.x; w < (end - beg) * parts; w += gridDim.x) {
+    const size_t slot = (size_t)t.slot[t.lvl_nodes[beg + w / parts]];
+    const int part = w % parts;
+    double2 x[8];
+    double* O;
+    const double* I;
+    int at, step;
+    if (part < NV) {
+      // pair (8 per row) p of the variable: rows of a plane 32 apart per pass
+      const int row = threadIdx.x >> 3;
+      at = part * NCELL + sidx(2 * (threadIdx.x & 7), row & 15, row >> 4);
+      step = 2 * NS * NS;
+      O = pool.bufp(cur) + slot * SLOT_U;
+      I = pool.bufp(cur ^ 1) + slot * SLOT_U;
+    } else {
+      at = ((part - NV) * 2048 + threadIdx.x) * 2;
+      step = 512;
+      O = reinterpret_cast<double*>(pool.shp(cur) + slot * SLOT_SH);
+      I = reinterpret_cast<const double*>(pool.shp(cur ^ 1) + slot * SLOT_SH);
     }
-    if (pool.shp(0)) {
-      float* R = pool.shp(cur) + slot * SLOT_SH;
-      const float* Q = pool.shp(cur ^ 1) + slot * SLOT_SH;
-      for (int e = threadIdx.x; e < SLOT_SH; e += blockDim.x) R[e] = Q[e];
-    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[i] = load_now(I + at + i * step);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) *reinterpret_cast<double2*>(O + at + i * step) = x[i];
   }
 }
+static_assert(SLOT_SH * sizeof(float) == 3 * 2048 * sizeof(double2) && NINT * sizeof(double) == 2048 * sizeof(double2),
+              "parts of k_lts_copyback");
 
 void launch_lts_copyback(const Topo& t, const Pool& pool, int cur, int level, cudaStream_t st) {
-  k_lts_copyback<<<sm_count() * 4, 256, 0, st>>>(t, pool, cur, level);
+  k_lts_copyback<<<sm_count() * 6, 256, 0, st>>>(t, pool, cur, level);
   ++g_kernel_launches;
 }
 
 // Integrated boundary-face fluxes of leaves: zero all (zero = 1) or, for the
 // leaves of `level`, add (w_stage x dt 2^(lmax - level)) x the stage's face fluxes.
-__global__ void k_lts_fmac(Topo t, Phys p, Pool pool, int level, int stage, const double* __restrict__ dt, int zero) {
+// Items are (leaf, side) pairs: NV * NFACE values, in 16-byte words.
+__global__ void __launch_bounds__(256) k_lts_fmac(Topo t, Phys p, Pool pool, int level, int stage,
+                                                  const double* __restrict__ dt, int zero) {
   const int beg = zero ? 0 : t.cnt[CNT_LVL + level];
   const int end = zero ? t.cnt[CNT_NLEAVES] : t.cnt[CNT_LVL + level + 1];
-  for (int w = beg + blockIdx.x; w < end; w += gridDim.x) {
-    const int node = zero ? t.leaves[w] : t.lvl_nodes[w];
+  constexpr int NP = NV * NFACE / 2;
+  for (int w = blockIdx.x; w < (end - beg) * 6; w += gridDim.x) {
+    const int node = zero ? t.leaves[beg + w / 6] : t.lvl_nodes[beg + w / 6], sd = w % 6;
     if (t.child0[node] >= 0) continue;
-    const size_t slot = (size_t)t.slot[node];
-    double* M = pool.fmac + slot * SLOT_F;
+    const size_t at = (size_t)t.slot[node] * SLOT_F + sd * NV * NFACE;
+    double2* M = reinterpret_cast<double2*>(pool.fmac + at);
     if (zero) {
-      for (int e = threadIdx.x; e < SLOT_F; e += blockDim.x) M[e] = 0.0;
+      for (int e = threadIdx.x; e < NP; e += blockDim.x) M[e] = make_double2(0.0, 0.0);
       continue;
     }
-    const double* F = pool.face + slot * SLOT_F;
+    if (!((t.fmask[node] >> sd) & 1u)) continue;                   // (the sides that the reflux reads)
+    const double2* F = reinterpret_cast<const double2*>(pool.face + at);
     const double wgt = kRkW[rk_row(p)][stage] * ldexp(dt[t.inst[node]], p.lmax[t.inst[node]] - level);
-    const uint32_t fm = t.fmask[node];          // (the sides that the reflux reads)
-    for (int sd = 0; sd < 6; ++sd) {
-      if (!((fm >> sd) & 1u)) continue;
-      for (int e = sd * NV * NFACE + threadIdx.x; e < (sd + 1) * NV * NFACE; e += blockDim.x) M[e] = M[e] + wgt * F[e];
+    for (int e = threadIdx.x; e < NP; e += blockDim.x) {
+      const double2 m = M[e], x = F[e];
+      M[e] = make_double2(m.x + wgt * x.x, m.y + wgt * x.y);
     }
   }
 }
 
 void launch_lts_fmac(const Topo& t, const Phys& p, const Pool& pool, int level, int stage, const double* dt,
                      int zero, cudaStream_t st) {
-  k_lts_fmac<<<sm_count() * 4, 256, 0, st>>>(t, p, pool, level, stage, dt, zero);
+  k_lts_fmac<<<sm_count() * 8, 256, 0, st>>>(t, p, pool, level, stage, dt, zero);
   ++g_kernel_launches;
 }
 

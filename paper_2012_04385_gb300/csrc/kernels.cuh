@@ -163,6 +163,10 @@ void launch_fill_copies(const Topo& t, const Phys& p, const Pool& pool, int cur,
 void launch_fill_bc(const Topo& t, const Phys& p, const Pool& pool, int cur, cudaStream_t st);
 // predicted regions of the nodes of `level` (after those of the coarser levels)
 void launch_predict(const Topo& t, const Phys& p, const Pool& pool, int cur, int level, int mode, cudaStream_t st);
+// The stage's predictions of `level` into buffer dst, the coarser level taken at
+// fraction th of its step (local time stepping).
+void launch_predict_lts(const Topo& t, const Phys& p, const Pool& pool, int cur, int dst, int level, double th,
+                        cudaStream_t st);
 // every halo region of the listed nodes (device list of n node indices), all variables
 void launch_fill_list(const Topo& t, const Phys& p, const Pool& pool, int cur, const int32_t* list, int n,
                       cudaStream_t st);
@@ -218,6 +222,8 @@ void launch_masks(const Topo& t, const Phys& p, uint32_t* miss, uint32_t* smask,
 void launch_sums(const Topo& t, const Phys& p, const Pool& pool, int cur, double* partial, double* out,
                  int nleaves_cap, cudaStream_t st);
 // mixed-precision variants (kern_f32.cu)
+void launch_predict_lts_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, int dst, int level, double th,
+                            cudaStream_t st);
 void launch_predict_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, int level, int mode, cudaStream_t st);
 void launch_fill_list_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, const int32_t* list, int n,
                           cudaStream_t st);

@@ -171,6 +171,40 @@ __device__ __forceinline__ double box_value(const ParentBox& b, unsigned w, int 
   return (v >= 1 && v <= 3 && ((w >> (19 + v)) & 1u)) ? -x : x;
 }
 
+// Local time stepping: the box's parent level at time fraction q of its step,
+// (1 - q) u^n + q u, blended where it is read (stored halos already hold
+// predictions of blended values).  n[]: bases of u^n by region, null where the
+// region is a stored halo; tab: offsets in its 16^3 layout.
+struct BlendBox {
+  const double* n[8];
+  int tab[3][16];
+};
+// (threads 0 .. 47, after parent_box of the same item; the caller synchronises)
+__device__ __forceinline__ void blend_box(const Topo& t, const double* __restrict__ un, int par, int ch,
+                                          const ParentBox& b, BlendBox& l) {
+  const int q = threadIdx.x;
+  if (q < 8) {
+    int r = 13, shift = 0;
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+      if ((q >> d) & 1) {
+        const int s = ((ch >> d) & 1) ? 1 : -1;
+        r += s * (d == 0 ? 1 : (d == 1 ? 3 : 9));
+        shift += s * (d == 0 ? NB : (d == 1 ? NB * NB : NB * NB * NB));
+      }
+    const int nb = q == 0 ? par : t.nbr[(size_t)par * 27 + r];
+    l.n[q] = nb < 0 ? nullptr : un + (size_t)t.slot[nb] * SLOT_N - shift;
+  }
+  if (q < 48) {
+    const int d = q >> 4, x = (int)(b.tab[d][q & 15] & 0xffffu) / (d == 0 ? 1 : (d == 1 ? NS : NS * NS)) - HW;
+    l.tab[d][q & 15] = x * (d == 0 ? 1 : (d == 1 ? NB : NB * NB));
+  }
+}
+// (rounded alike in every translation unit)
+__device__ __forceinline__ double blend(double q, double n, double u) {
+  return __dadd_rn(__dmul_rn(1.0 - q, n), __dmul_rn(q, u));
+}
+
 // A value c whose box of equal values predicts c: every difference and mixed
 // difference is +0, every Q-term +0, and c + (+-0) is c unless c is -0; c + c stays
 // finite.
@@ -188,9 +222,9 @@ __device__ __forceinline__ bool same_bits(double a, double b) { return __double_
 // q-th at s + q * nx ny nz; all threads.  A group of 8 or 16 lanes owns a row.
 // Returns the variables (bit q) whose cells staged by this thread all equal the
 // box's first cell.
-template <class R>
+template <class R, bool BLEND = false>
 __device__ __forceinline__ unsigned stage_box(R* __restrict__ s, const ParentBox& b, bool detail_only, int i0, int j0,
-                                          int k0, int nx, int ny, int nz) {
+                                          int k0, int nx, int ny, int nz, const BlendBox* l = nullptr, double th = 0.0) {
   const int lg = nx > 8 ? 4 : 3, i = threadIdx.x & ((1 << lg) - 1);
   unsigned eq = 31u;
   if (i >= nx) return eq;
@@ -199,7 +233,18 @@ __device__ __forceinline__ unsigned stage_box(R* __restrict__ s, const ParentBox
   R first[NV];
 #pragma unroll
   for (int q = 0; q < NV; ++q)
-    if (!detail_only || q < 2) first[q] = to_r<R>(box_value(b, w0, detail_only ? 4 * q : q));
+    if (!detail_only || q < 2) {
+      double y = box_value(b, w0, detail_only ? 4 * q : q);
+      if (BLEND) {
+        const double* un = l->n[(w0 >> 16) & 7u];
+        const bool flip = q >= 1 && q <= 3 && ((w0 >> (19 + q)) & 1u);
+        if (un) {
+          y = blend(th, un[q * NINT + l->tab[0][i0] + l->tab[1][j0] + l->tab[2][k0]], flip ? -y : y);
+          if (flip) y = -y;
+        }
+      }
+      first[q] = to_r<R>(y);
+    }
   for (int row = threadIdx.x >> lg; row < ny * nz; row += blockDim.x >> lg) {
     const int k = (row * inv) >> 16, j = row - k * ny;
     const unsigned w = wi + b.tab[1][j0 + j] + b.tab[2][k0 + k];
@@ -213,9 +258,12 @@ __device__ __forceinline__ unsigned stage_box(R* __restrict__ s, const ParentBox
         o[q * n] = x;
       }
     } else {
+      const double* __restrict__ un = BLEND ? l->n[(w >> 16) & 7u] : nullptr;
+      if (BLEND && un) un += l->tab[0][i0 + i] + l->tab[1][j0 + j] + l->tab[2][k0 + k];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        const double y = c[v * NCELL];
+        double y = c[v * NCELL];
+        if (BLEND && un) y = blend(th, un[v * NINT], y);
         const R x = to_r<R>((v >= 1 && v <= 3 && ((w >> (19 + v)) & 1u)) ? -y : y);
         if (!same_bits(x, first[v])) eq &= ~(1u << v);
         o[v * n] = x;
@@ -310,16 +358,21 @@ static __global__ void __launch_bounds__(256) k_fill_regions(Topo t, Pool pool, 
 // and writes their eight fine cells.  Jumps lie where the solution is smooth, so
 // most boxes hold one value: it predicts itself (const_safe), without the 125
 // shared-memory loads of the Q-terms.
+// BLEND (local time stepping): the parent level at fraction th of its step, and
+// the halos go to the nodes' places in stage buffer dst, where their level is.
 constexpr int PRED_SPLIT = 4;
-template <class R>
+template <class R, bool BLEND = false>
 __global__ void __launch_bounds__(256) k_predict_t(Topo t, Phys p, Pool pool, int cur, const int32_t* __restrict__ list,
                                                    const int32_t* __restrict__ cnt, int n,
-                                                   const uint32_t* __restrict__ mask, int mode) {
+                                                   const uint32_t* __restrict__ mask, int mode, int dst = 0,
+                                                   double th = 0.0) {
   // the nodes of level n in a list grouped by level (cnt given), or n listed nodes
   __shared__ R box[NV * 864];
   __shared__ ParentBox pb;
+  __shared__ BlendBox lb;
   __shared__ unsigned eqs[8];
   double* buf = pool.bufp(cur);
+  double* out = BLEND ? pool.bufp(dst) : buf;
   const int nnode = cnt ? cnt[(mode == FILL_STAGE ? CNT_PST : CNT_PALL) + n] : n, nitems = nnode * PRED_SPLIT;
   if (cnt) list += cnt[CNT_LVL + n];
   // (the parts of all nodes one after the other: the first holds most of the
@@ -334,9 +387,13 @@ __global__ void __launch_bounds__(256) k_predict_t(Topo t, Phys p, Pool pool, in
     __syncthreads();                                         // the previous item's box is free
     parent_box(t, p, buf, par, ch, pb);
     __syncthreads();
-    const bool detail_only = mode == FILL_DETAIL && t.child0[node] < 0;
+    if (BLEND) {
+      blend_box(t, pool.un, par, ch, pb, lb);
+      __syncthreads();
+    }
+    const bool detail_only = !BLEND && mode == FILL_DETAIL && t.child0[node] < 0;
     const int nvar = detail_only ? 2 : NV;
-    double* u = buf + (size_t)t.slot[node] * SLOT_U;
+    double* u = out + (size_t)t.slot[node] * SLOT_U;
     for (int rank = 0; m; ++rank) {
       const int r = __ffs(m) - 1;
       m &= m - 1;
@@ -349,7 +406,7 @@ __global__ void __launch_bounds__(256) k_predict_t(Topo t, Phys p, Pool pool, in
       const int bx0 = qx0 + 2, by0 = qy0 + 2, bz0 = qz0 + 2;
       const int nx = (1 << lx) + 4, ny = (1 << ly) + 4, nz = (1 << lz) + 4;
       const int nb = nx * ny * nz;
-      const unsigned eq = __reduce_and_sync(0xffffffffu, stage_box<R>(box, pb, detail_only, bx0, by0, bz0, nx, ny, nz));
+      const unsigned eq = __reduce_and_sync(0xffffffffu, stage_box<R, BLEND>(box, pb, detail_only, bx0, by0, bz0, nx, ny, nz, &lb, th));
       if ((threadIdx.x & 31) == 0) eqs[threadIdx.x >> 5] = eq;
       __syncthreads();
       unsigned constant = eqs[0];
