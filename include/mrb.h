@@ -363,8 +363,8 @@ int mrb_profile(mrb_ctx* ctx, int32_t enable);
  * params[MRB_NTUNE]: [0] stage-kernel waves (CTAs = SMs x resident CTAs per SM
  * x waves, 1..8), [1] stage work-item order (0 strided over the grid, 1 one
  * contiguous run of (block, z-slab) items per CTA), [2] region-copy halo-fill
- * CTAs per SM, [3] prediction halo-fill CTAs per SM, [4] averaging CTAs per SM
- * (1..32 each).  Defaults 1, 0, 8, 4, 8.  Per context; mrb_set_tune returns
+ * CTAs per SM in fours, [3] prediction halo-fill CTAs per SM (up to four times as
+ * many where there are that many blocks), [4] averaging CTAs per SM (1..32 each).  Defaults 1, 0, 8, 4, 8.  Per context; mrb_set_tune returns
  * EINVAL outside the ranges and re-captures the step graphs at the next
  * mrb_step. */
 #define MRB_NTUNE 5

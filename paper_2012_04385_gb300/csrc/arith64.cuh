@@ -215,4 +215,32 @@ __host__ __device__ __forceinline__ double sqrt64(double x) {
   return bits2d(((uint64_t)(uint32_t)(((ex - 1023 - (int32_t)odd) >> 1) + 1022) << 52) + m);
 }
 
+// The mean 0.125 (((u0 + u1) + (u2 + u3)) + ((u4 + u5) + (u6 + u7))), each sum
+// rounded to nearest even.  Values of one sign and exponent (the usual eight
+// children of a cell): a sum of two has the next exponent and drops one bit, so
+// each level of sums is a rounded mean of 52-bit fractions; about 65 integer
+// instructions for eight of the FP64 pipe, which cost 64 issue slots each.  The
+// last sum's exponent is three above, so it stays finite.  Eight equal values
+// without an exponent (zeros) are their own mean.
+__host__ __device__ __forceinline__ uint64_t mean_even(uint64_t a, uint64_t b) {
+  const uint64_t x = a + b, q = x >> 1;
+  return q + (x & q & 1u);
+}
+__host__ __device__ __forceinline__ double mean8(const double (&v)[8]) {
+  constexpr uint64_t M = 0x000fffffffffffffull;
+  const uint64_t u0 = d2bits(v[0]);
+  uint64_t d = 0;
+#pragma unroll
+  for (int i = 1; i < 8; ++i) d |= d2bits(v[i]) ^ u0;
+  const uint32_t e = (uint32_t)(u0 >> 52) & 2047u;
+  if (e == 0 ? d == 0 : (d <= M && e < 2043u)) {
+    if (e == 0) return v[0];
+    uint64_t m[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) m[i] = mean_even(d2bits(v[2 * i]) & M, d2bits(v[2 * i + 1]) & M);
+    return bits2d((u0 & ~M) | mean_even(mean_even(m[0], m[1]), mean_even(m[2], m[3])));
+  }
+  return 0.125 * (((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7])));
+}
+
 }  // namespace mrb

@@ -257,9 +257,10 @@ struct mrb_ctx {
   void list_used() { CK(cudaEventRecord(list_ev, st)); }
 
   // ---- the steps
+  int level_nodes(int l) const { return h_cnt[CNT_LVL + l + 1] - h_cnt[CNT_LVL + l]; }
   void fill_halos(int mode = FILL_FULL) {
-    if (mode == FILL_FULL) launch_fill_copies(topo(), phys, P, cur, st);
-    for (int l = 1; l <= max_lmax; ++l) launch_predict(topo(), phys, P, cur, l, mode, st);
+    if (mode == FILL_FULL) launch_fill_copies(topo(), P, cur, h_cnt[CNT_NNODES], st);
+    for (int l = 1; l <= max_lmax; ++l) launch_predict(topo(), phys, P, cur, l, level_nodes(l), mode, st);
     if (mode == FILL_FULL) launch_fill_bc(topo(), phys, P, cur, st);
   }
   // the stage kernels read face neighbours' cells and map boundary cells
@@ -334,12 +335,12 @@ struct mrb_ctx {
           const int at = full ? cur : cur ^ (s & 1);             // the level's stage buffer
           if (full) {
             launch_lts_interp(topo(), P, cur, l, th, 0, st);
-            launch_fill_copies(topo(), phys, P, cur, st);
-            for (int ll = 1; ll <= l; ++ll) launch_predict(topo(), phys, P, cur, ll, fmode, st);
+            launch_fill_copies(topo(), P, cur, h_cnt[CNT_NNODES], st);
+            for (int ll = 1; ll <= l; ++ll) launch_predict(topo(), phys, P, cur, ll, level_nodes(ll), fmode, st);
             launch_fill_bc(topo(), phys, P, cur, st);
           } else {
             for (int ll = 1; ll <= l; ++ll)
-              launch_predict_lts(topo(), phys, P, cur, ll == l ? at : cur, ll, th.th[ll - 1], st);
+              launch_predict_lts(topo(), phys, P, cur, ll == l ? at : cur, ll, level_nodes(ll), th.th[ll - 1], st);
           }
           if (cfg.precision == MRB_FP32_ACC64) launch_rhs_rk_f32(topo(), phys, P, at, s, d_dt, nullptr, st, l);
           else launch_rhs_rk_f64(topo(), phys, P, at, s, d_dt, nullptr, st, l);
@@ -841,7 +842,7 @@ int mrb_mr_predict_and_tag(mrb_ctx* c, int32_t allow_refine, int8_t* tags_dev, d
   return guarded(c, [&] {
     if (!tags_dev) throw Err(MRB_EINVAL, "null tags");
     launch_delta_tags(c->topo(), c->phys, c->P, c->cur, c->d_delta_node, allow_refine ? 1 : 0, tags_dev, delta_dev,
-                      c->n_leaves(), c->st);
+                      c->n_leaves(), c->h_cnt[CNT_NNODES], c->st);
   });
 }
 
@@ -917,7 +918,7 @@ int mrb_step(mrb_ctx* c, int32_t nsteps, double* dt_hist_dev) {
         c->fill_halos(FILL_DETAIL);
         c->detail_filled = true;
         launch_delta_tags(c->topo(), c->phys, c->P, c->cur, c->d_delta_node, 1, c->d_tags, nullptr, c->n_leaves(),
-                          c->st);
+                          c->h_cnt[CNT_NNODES], c->st);
         c->remesh(c->d_tags);
       }
       if (c->prof && !c->phys.lts) {   // (the macro steps of local time stepping are not profiled per stage)

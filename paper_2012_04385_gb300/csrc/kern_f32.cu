@@ -22,17 +22,18 @@ void launch_rhs_rk_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, 
   } else launch_stage_f32<0>(t, p, pool, cur, stage, dt, rhs_out, st, level);
 }
 
-void launch_predict_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, int level, int mode, cudaStream_t st) {
+void launch_predict_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, int level, int n_nodes, int mode,
+                        cudaStream_t st) {
   const bool stage = mode == FILL_STAGE;
-  k_predict_t<float><<<sm_count() * g_tune.fill_pred, 256, 0, st>>>(t, p, pool, cur, stage ? t.pst : t.pall,
-                                                                    t.cnt, level, stage ? t.smask : t.miss, mode);
+  k_predict_t<float><<<predict_grid(n_nodes), 256, 0, st>>>(t, p, pool, cur, stage ? t.pst : t.pall, t.cnt, level,
+                                                            stage ? t.smask : t.miss, mode);
   ++g_kernel_launches;
 }
 
-void launch_predict_lts_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, int dst, int level, double th,
-                            cudaStream_t st) {
-  k_predict_t<float, true><<<sm_count() * g_tune.fill_pred, 256, 0, st>>>(t, p, pool, cur, t.pst, t.cnt, level, t.smask,
-                                                                          FILL_STAGE, dst, th);
+void launch_predict_lts_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, int dst, int level, int n_nodes,
+                            double th, cudaStream_t st) {
+  k_predict_t<float, true><<<predict_grid(n_nodes), 256, 0, st>>>(t, p, pool, cur, t.pst, t.cnt, level, t.smask,
+                                                                  FILL_STAGE, dst, th);
   ++g_kernel_launches;
 }
 
@@ -100,8 +101,9 @@ __global__ void __launch_bounds__(256) k_set_cons_f32(Topo t, Phys p, Pool pool,
 
 void launch_set_cons_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, const int32_t* nodes, int n,
                          const double* cons, cudaStream_t st) {
-  if (((uintptr_t)cons & 15) == 0) k_set_cons_f32<true><<<sm_count() * 4, 256, 0, st>>>(t, p, pool, cur, nodes, n, cons);
-  else k_set_cons_f32<false><<<sm_count() * 4, 256, 0, st>>>(t, p, pool, cur, nodes, n, cons);
+  const int grid = item_grid((int64_t)n * 4);
+  if (((uintptr_t)cons & 15) == 0) k_set_cons_f32<true><<<grid, 256, 0, st>>>(t, p, pool, cur, nodes, n, cons);
+  else k_set_cons_f32<false><<<grid, 256, 0, st>>>(t, p, pool, cur, nodes, n, cons);
   ++g_kernel_launches;
 }
 
@@ -200,12 +202,17 @@ void launch_get_records(const Topo& t, const Phys& p, const Pool& pool, int cur,
 // the parent box staged once as (rho, E) pairs, the Q-terms of Eq.
 // Prediction and the eight predictions of each parent cell computed two
 // variables per instruction.  delta = max over both variables of
-// |u - P(u_parent)| / |u|, as k_delta_t.
+// |u - P(u_parent)| / |u|, as k_delta_f64.
+// A half-warp takes a 4 x 4 tile of parent cells of one plane: with rows 20 pairs
+// apart its 16 eight-byte reads fall into 32 different banks (twelve in a row and
+// four of the next one, rows 16 apart, collided: twice the wavefronts of 125 reads per
+// cell; shock-bubble levels 0..4: 862 -> 678 us).
+constexpr int DP_X = 20, DP_XY = 16 * DP_X;
 struct SAcc2 {
   const float2* s;
   int i0, j0, k0;
   __device__ __forceinline__ float2 operator()(int i, int j, int k) const {
-    return s[(k - k0) * 256 + (j - j0) * 16 + (i - i0)];
+    return s[(k - k0) * DP_XY + (j - j0) * DP_X + (i - i0)];
   }
 };
 
@@ -231,7 +238,7 @@ __device__ __forceinline__ float2 mix3p(const SAcc2& P, int i, int j, int k, int
 __global__ void __launch_bounds__(256) k_delta_p(Topo t, Phys p, Pool pool, int cur, double* __restrict__ delta_node,
                                                  int all_nodes) {
   __shared__ double sh[8];
-  __shared__ float2 box[4096];      // (rho, E) of the parent's cells 8 cb - 4 .. 8 cb + 11 per axis
+  __shared__ float2 box[16 * DP_XY];   // (rho, E) of the parent's cells 8 cb - 4 .. 8 cb + 11 per axis
   __shared__ ParentBox pb;
   __shared__ const double* own[27]; // the node's stored cells by region
   const int nitems = all_nodes ? t.cnt[CNT_NNODES] : t.cnt[CNT_NLEAVES];
@@ -264,14 +271,15 @@ __global__ void __launch_bounds__(256) k_delta_p(Topo t, Phys p, Pool pool, int 
       const unsigned w = box_word(pb, e & 15, (e >> 4) & 15, e >> 8);
       const double* __restrict__ c = pb.p[(w >> 16) & 7u] + (w & 0xffffu);
       const float2 x = make_float2(d2f_fast(c[0]), d2f_fast(c[4 * NCELL]));
-      box[e] = x;
+      box[(e >> 4) * DP_X + (e & 15)] = x;
       eq = eq && same_bits(x.x, first.x) && same_bits(x.y, first.y);
     }
     const bool constant = __syncthreads_and(eq);      // (a box of one value predicts it)
     const SAcc2 A{box, 0, 0, 0};
     float m = 0.f;
     for (int q = threadIdx.x; q < 1728; q += blockDim.x) {
-      const int rx = q % 12 - 2, ry = (q / 12) % 12 - 2, rz = q / 144 - 2;
+      const int tile = q >> 4;                            // 3 x 3 tiles in a plane
+      const int rx = 4 * (tile % 3) + (q & 3) - 2, ry = 4 * ((tile / 3) % 3) + ((q >> 2) & 3) - 2, rz = q / 144 - 2;
       const bool ghost = (rx < 0 && gl[0]) || (rx >= 8 && gh[0]) || (ry < 0 && gl[1]) || (ry >= 8 && gh[1]) ||
                          (rz < 0 && gl[2]) || (rz >= 8 && gh[2]);
       if (ghost) continue;
@@ -356,8 +364,8 @@ __global__ void __launch_bounds__(256) k_delta_p(Topo t, Phys p, Pool pool, int 
 }
 
 void launch_delta_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, double* delta_node, int all_nodes,
-                      cudaStream_t st) {
-  k_delta_p<<<sm_count() * 4, 256, 0, st>>>(t, p, pool, cur, delta_node, all_nodes);
+                      int n_nodes, cudaStream_t st) {
+  k_delta_p<<<item_grid(n_nodes), 256, 0, st>>>(t, p, pool, cur, delta_node, all_nodes);
   ++g_kernel_launches;
 }
 

@@ -97,16 +97,18 @@ void launch_set_cons(const Topo& t, const Phys& p, const Pool& pool, int cur, co
     launch_set_cons_f32(t, p, pool, cur, nodes, n, cons, st);
     return;
   }
-  if (((uintptr_t)cons & 15) == 0) k_set_cons<true><<<sm_count() * 8, 256, 0, st>>>(t, pool, cur, nodes, n, cons);
-  else k_set_cons<false><<<sm_count() * 8, 256, 0, st>>>(t, pool, cur, nodes, n, cons);
+  const int grid = item_grid((int64_t)n * NV);
+  if (((uintptr_t)cons & 15) == 0) k_set_cons<true><<<grid, 256, 0, st>>>(t, pool, cur, nodes, n, cons);
+  else k_set_cons<false><<<grid, 256, 0, st>>>(t, pool, cur, nodes, n, cons);
   ++g_kernel_launches;
 }
 
+constexpr int GET_PARTS = 27;     // of a block with its halo
 template <bool VEC>
 __global__ void __launch_bounds__(256) k_get_state(Topo t, Pool pool, int cur, const int32_t* __restrict__ nodes, int n,
                                                    double* __restrict__ out, int with_halo) {
   if (with_halo) {        // a block's stored cells are contiguous
-    constexpr int PARTS = 27, PER = SLOT_U / 2 / PARTS;       // 27 x 1280 pairs
+    constexpr int PARTS = GET_PARTS, PER = SLOT_U / 2 / PARTS;       // 27 x 1280 pairs
     static_assert(PARTS * PER * 2 == SLOT_U && PER == 5 * 256, "whole parts");
     for (int w = blockIdx.x; w < n * PARTS; w += gridDim.x) {
       const size_t off = (size_t)(w % PARTS) * 2 * PER + 2 * threadIdx.x;
@@ -134,15 +136,16 @@ __global__ void __launch_bounds__(256) k_get_state(Topo t, Pool pool, int cur, c
 void launch_get_state(const Topo& t, const Pool& pool, int cur, const int32_t* nodes, int n, double* out,
                       int with_halo, cudaStream_t st) {
   if (n <= 0) return;
-  if (((uintptr_t)out & 15) == 0) k_get_state<true><<<sm_count() * 8, 256, 0, st>>>(t, pool, cur, nodes, n, out, with_halo);
-  else k_get_state<false><<<sm_count() * 8, 256, 0, st>>>(t, pool, cur, nodes, n, out, with_halo);
+  const int grid = item_grid((int64_t)n * (with_halo ? GET_PARTS : NV));
+  if (((uintptr_t)out & 15) == 0) k_get_state<true><<<grid, 256, 0, st>>>(t, pool, cur, nodes, n, out, with_halo);
+  else k_get_state<false><<<grid, 256, 0, st>>>(t, pool, cur, nodes, n, out, with_halo);
   ++g_kernel_launches;
 }
 
 // ---------------------------------------------------------------- halo fill (mr.cuh)
-void launch_fill_copies(const Topo& t, const Phys& p, const Pool& pool, int cur, cudaStream_t st) {
-  (void)p;
-  k_fill_regions<<<sm_count() * g_tune.fill_copy, 256, 0, st>>>(t, pool, cur, NodeSet{nullptr, 0});
+void launch_fill_copies(const Topo& t, const Pool& pool, int cur, int n_nodes, cudaStream_t st) {
+  const int64_t need = ((int64_t)n_nodes * 26 + 7) / 8;         // a warp per region
+  k_fill_regions<<<(int)std::min<int64_t>(need, 4 * sm_count() * g_tune.fill_copy), 256, 0, st>>>(t, pool, cur, NodeSet{nullptr, 0});
   ++g_kernel_launches;
 }
 
@@ -151,25 +154,28 @@ void launch_fill_bc(const Topo& t, const Phys& p, const Pool& pool, int cur, cud
   ++g_kernel_launches;
 }
 
-void launch_predict(const Topo& t, const Phys& p, const Pool& pool, int cur, int level, int mode, cudaStream_t st) {
+void launch_predict(const Topo& t, const Phys& p, const Pool& pool, int cur, int level, int n_nodes, int mode,
+                    cudaStream_t st) {
+  if (n_nodes <= 0) return;
   if (p.precision == 1) {
-    launch_predict_f32(t, p, pool, cur, level, mode, st);
+    launch_predict_f32(t, p, pool, cur, level, n_nodes, mode, st);
     return;
   }
   const bool stage = mode == FILL_STAGE;
-  k_predict_t<double><<<sm_count() * g_tune.fill_pred, 256, 0, st>>>(t, p, pool, cur, stage ? t.pst : t.pall, t.cnt,
-                                                                     level, stage ? t.smask : t.miss, mode);
+  k_predict_t<double><<<predict_grid(n_nodes), 256, 0, st>>>(t, p, pool, cur, stage ? t.pst : t.pall, t.cnt, level,
+                                                             stage ? t.smask : t.miss, mode);
   ++g_kernel_launches;
 }
 
-void launch_predict_lts(const Topo& t, const Phys& p, const Pool& pool, int cur, int dst, int level, double th,
-                        cudaStream_t st) {
+void launch_predict_lts(const Topo& t, const Phys& p, const Pool& pool, int cur, int dst, int level, int n_nodes,
+                        double th, cudaStream_t st) {
+  if (n_nodes <= 0) return;
   if (p.precision == 1) {
-    launch_predict_lts_f32(t, p, pool, cur, dst, level, th, st);
+    launch_predict_lts_f32(t, p, pool, cur, dst, level, n_nodes, th, st);
     return;
   }
-  k_predict_t<double, true><<<sm_count() * g_tune.fill_pred, 256, 0, st>>>(t, p, pool, cur, t.pst, t.cnt, level, t.smask,
-                                                                           FILL_STAGE, dst, th);
+  k_predict_t<double, true><<<predict_grid(n_nodes), 256, 0, st>>>(t, p, pool, cur, t.pst, t.cnt, level, t.smask,
+                                                                   FILL_STAGE, dst, th);
   ++g_kernel_launches;
 }
 
@@ -437,7 +443,7 @@ __global__ void k_jump(Topo t, Phys p, Pool pool, int target, int stage, const d
 
 void launch_jump(const Topo& t, const Phys& p, const Pool& pool, int target, int stage, const double* dt,
                  double* rhs_out, cudaStream_t st) {
-  k_jump<<<sm_count() * 4, 256, 0, st>>>(t, p, pool, target, stage, dt, rhs_out);
+  k_jump<<<sm_count() * 8, 256, 0, st>>>(t, p, pool, target, stage, dt, rhs_out);
   ++g_kernel_launches;
 }
 
@@ -571,10 +577,11 @@ __global__ void k_tags(Topo t, Phys p, const double* __restrict__ delta_node, in
 }
 
 void launch_delta_tags(const Topo& t, const Phys& p, const Pool& pool, int cur, double* delta_node,
-                       int allow_refine, int8_t* tags, double* delta_leaf, int n_leaves_cap, cudaStream_t st) {
-  if (p.precision == 1) launch_delta_f32(t, p, pool, cur, delta_node, allow_refine, st);
+                       int allow_refine, int8_t* tags, double* delta_leaf, int n_leaves_cap, int n_nodes, cudaStream_t st) {
+  if (p.precision == 1) launch_delta_f32(t, p, pool, cur, delta_node, allow_refine, allow_refine ? n_nodes : n_leaves_cap, st);
   else {
-    k_delta_t<double><<<sm_count() * 4, 256, 0, st>>>(t, p, pool, cur, delta_node, allow_refine);
+    cudaMemsetAsync(delta_node, 0, (size_t)n_nodes * sizeof(double), st);
+    k_delta_f64<<<item_grid((int64_t)(allow_refine ? n_nodes : n_leaves_cap) * 4), 256, 0, st>>>(t, p, pool, cur, delta_node, allow_refine);
     ++g_kernel_launches;
   }
   k_tags<<<(n_leaves_cap + 255) / 256, 256, 0, st>>>(t, p, delta_node, allow_refine, tags, delta_leaf);
@@ -632,8 +639,8 @@ void launch_flux_census(const Topo& t, const Phys& p, const Pool& pool, int cur,
 void launch_refine_fill(const Topo& t, const Phys& p, const Pool& pool, int cur, const int32_t* pairs, int n,
                         cudaStream_t st) {
   if (n <= 0) return;
-  if (p.precision == 1) k_refine_fill_t<float><<<sm_count() * 8, 256, 0, st>>>(t, pool, cur, pairs, n);
-  else k_refine_fill_t<double><<<sm_count() * 8, 256, 0, st>>>(t, pool, cur, pairs, n);
+  if (p.precision == 1) k_refine_fill_t<float><<<item_grid((int64_t)n * NV), 256, 0, st>>>(t, pool, cur, pairs, n);
+  else k_refine_fill_t<double><<<item_grid((int64_t)n * NV), 256, 0, st>>>(t, pool, cur, pairs, n);
   ++g_kernel_launches;
 }
 
@@ -850,7 +857,7 @@ __global__ void __launch_bounds__(256) k_sums_finish(Topo t, Phys p, const doubl
 void launch_sums(const Topo& t, const Phys& p, const Pool& pool, int cur, double* partial, double* out,
                  int nleaves_cap, cudaStream_t st) {
   (void)nleaves_cap;
-  k_sums_partial<<<sm_count() * 4, 256, 0, st>>>(t, p, pool, cur, partial);
+  k_sums_partial<<<sm_count() * 16, 256, 0, st>>>(t, p, pool, cur, partial);
   ++g_kernel_launches;
   k_sums_finish<<<p.n_inst, 256, 0, st>>>(t, p, partial, out);
   ++g_kernel_launches;

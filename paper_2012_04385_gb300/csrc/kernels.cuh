@@ -5,6 +5,7 @@
 // lets the stage sequence be replayed from a CUDA graph).
 #pragma once
 
+#include <algorithm>
 #include "physics.cuh"
 
 namespace mrb {
@@ -159,14 +160,15 @@ void launch_set_cons_f32(const Topo& t, const Phys& p, const Pool& pool, int cur
 void launch_get_state(const Topo& t, const Pool& pool, int cur, const int32_t* nodes, int n, double* out,
                       int with_halo, cudaStream_t st);
 // stored halos facing same-level nodes, and ghost cells beyond the boundary, of every node
-void launch_fill_copies(const Topo& t, const Phys& p, const Pool& pool, int cur, cudaStream_t st);
+void launch_fill_copies(const Topo& t, const Pool& pool, int cur, int n_nodes, cudaStream_t st);
 void launch_fill_bc(const Topo& t, const Phys& p, const Pool& pool, int cur, cudaStream_t st);
 // predicted regions of the nodes of `level` (after those of the coarser levels)
-void launch_predict(const Topo& t, const Phys& p, const Pool& pool, int cur, int level, int mode, cudaStream_t st);
+void launch_predict(const Topo& t, const Phys& p, const Pool& pool, int cur, int level, int n_nodes, int mode,
+                    cudaStream_t st);
 // The stage's predictions of `level` into buffer dst, the coarser level taken at
 // fraction th of its step (local time stepping).
-void launch_predict_lts(const Topo& t, const Phys& p, const Pool& pool, int cur, int dst, int level, double th,
-                        cudaStream_t st);
+void launch_predict_lts(const Topo& t, const Phys& p, const Pool& pool, int cur, int dst, int level, int n_nodes,
+                        double th, cudaStream_t st);
 // every halo region of the listed nodes (device list of n node indices), all variables
 void launch_fill_list(const Topo& t, const Phys& p, const Pool& pool, int cur, const int32_t* list, int n,
                       cudaStream_t st);
@@ -207,7 +209,8 @@ void launch_project_level_f32(const Topo& t, const Phys& p, const Pool& pool, in
 void launch_cfl(const Topo& t, const Phys& p, const Pool& pool, int cur, unsigned long long* smax, double* dt,
                 int* status, cudaStream_t st);
 void launch_delta_tags(const Topo& t, const Phys& p, const Pool& pool, int cur, double* delta_node,
-                       int allow_refine, int8_t* tags, double* delta_leaf, int n_leaves_cap, cudaStream_t st);
+                       int allow_refine, int8_t* tags, double* delta_leaf, int n_leaves_cap, int n_nodes,
+                       cudaStream_t st);
 void launch_refine_fill(const Topo& t, const Phys& p, const Pool& pool, int cur, const int32_t* pairs, int n,
                         cudaStream_t st);
 // Leaves with resolution jumps (a same-level face neighbour that is refined):
@@ -222,9 +225,10 @@ void launch_masks(const Topo& t, const Phys& p, uint32_t* miss, uint32_t* smask,
 void launch_sums(const Topo& t, const Phys& p, const Pool& pool, int cur, double* partial, double* out,
                  int nleaves_cap, cudaStream_t st);
 // mixed-precision variants (kern_f32.cu)
-void launch_predict_lts_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, int dst, int level, double th,
-                            cudaStream_t st);
-void launch_predict_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, int level, int mode, cudaStream_t st);
+void launch_predict_lts_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, int dst, int level, int n_nodes,
+                            double th, cudaStream_t st);
+void launch_predict_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, int level, int n_nodes, int mode,
+                        cudaStream_t st);
 void launch_fill_list_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, const int32_t* list, int n,
                           cudaStream_t st);
 // Roe / LLF census of every leaf face (FP64 decisions on the stage buffer):
@@ -232,7 +236,7 @@ void launch_fill_list_f32(const Topo& t, const Phys& p, const Pool& pool, int cu
 void launch_flux_census(const Topo& t, const Phys& p, const Pool& pool, int cur, unsigned long long* counts,
                         cudaStream_t st);
 void launch_delta_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, double* delta_node, int all_nodes,
-                      cudaStream_t st);
+                      int n_nodes, cudaStream_t st);
 void launch_cfl_speeds_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, unsigned long long* smax,
                            int* status, cudaStream_t st);
 // FP32 records of stage buffer b from its FP64 internal cells (mixed-precision
@@ -248,6 +252,19 @@ void launch_get_records(const Topo& t, const Phys& p, const Pool& pool, int cur,
 void launch_face_samples(const Topo& t, const Phys& p, const Pool& pool, int cur, float tau_lab, int64_t stride,
                          float* feats, uint8_t* labels, int64_t* where, int64_t cap, cudaStream_t st);
 int sm_count();
+// Grids of kernels whose items differ in length (a detail box of one value, a copy
+// that meets the cache): a CTA per item up to 32 per SM, handed out as CTAs end.
+// With four per SM, of which the registers admit three, the fourth ran alone
+// afterwards: details of the shock-bubble (levels 0..4) 679 -> 474 us, get_state 344
+// -> 326, set_cons 464 -> 416.
+inline int item_grid(int64_t items) { return (int)std::min<int64_t>(items, 32 * (int64_t)sm_count()); }
+// Predictions: a CTA per node (up to four items of one), between fill_pred and four
+// times that per SM.  Shock-bubble, 16 launches: 840 us with 4 per SM, 709 with 16;
+// on a few hundred nodes 16 per SM cost a microsecond a launch more than 4.
+inline int predict_grid(int n_nodes) {
+  const int per = g_tune.fill_pred * sm_count();
+  return std::min(std::max(n_nodes, per), 4 * per);
+}
 // kernel launches issued by this process (host-side counter, bumped by every launch_* wrapper)
 extern long long g_kernel_launches;
 

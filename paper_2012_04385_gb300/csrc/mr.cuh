@@ -526,28 +526,28 @@ static __global__ void __launch_bounds__(256) k_fill_bc(Topo t, Phys p, Pool poo
 // delta of a node at level >= 1: max over its stored cells that are not ghost
 // cells and over rho, E of |u - P(u_parent)| / |u|.  Every leaf, and with
 // `all_nodes` every node (the tags then also read the details of the parents
-// of leaf groups).
+// of leaf groups).  In FP64 the pipe bounds it.  Items are a variable and half of the
+// planes of a node, so that a few hundred nodes spread evenly over the SMs; their
+// maxima meet in delta_node, which starts at zero.  Shock-bubble with levels 1 and 2:
+// 1119 -> 650 us.
 // Region of the fine cells of parent cell (rx, ry, rz) (-2 .. 9 relative to the child's origin).
 __device__ __forceinline__ int own_region(int rx, int ry, int rz) {
   return (rx < 0 ? 0 : (rx < 8 ? 1 : 2)) + 3 * (ry < 0 ? 0 : (ry < 8 ? 1 : 2)) + 9 * (rz < 0 ? 0 : (rz < 8 ? 1 : 2));
 }
-template <class R>
-__global__ void __launch_bounds__(256) k_delta_t(Topo t, Phys p, Pool pool, int cur, double* __restrict__ delta_node,
+static __global__ void __launch_bounds__(256) k_delta_f64(Topo t, Phys p, Pool pool, int cur, double* __restrict__ delta_node,
                                                  int all_nodes) {
   __shared__ double sh[8];
-  __shared__ R box[4096];           // the parent's cells 8 cb - 4 .. 8 cb + 11 per axis, one variable
+  __shared__ double box[2560];      // the parent's cells 8 cb - 4 .. 8 cb + 11 in x and y, ten planes
   __shared__ ParentBox pb;
   __shared__ const double* own[27]; // the node's stored cells by region
 
-  const int nitems = all_nodes ? t.cnt[CNT_NNODES] : t.cnt[CNT_NLEAVES];
+  const int nnode = all_nodes ? t.cnt[CNT_NNODES] : t.cnt[CNT_NLEAVES];
   const double* B = pool.bufp(cur);
-  for (int li = blockIdx.x; li < nitems; li += gridDim.x) {
-    const int node = all_nodes ? li : t.leaves[li];
+  for (int it = blockIdx.x; it < nnode * 4; it += gridDim.x) {
+    const int node = all_nodes ? it % nnode : t.leaves[it % nnode];
+    const int v = (it / nnode) & 1 ? 4 : 0, rz0 = it / nnode < 2 ? -2 : 4;
     const int lvl = t.level[node];
-    if (lvl == 0) {
-      if (threadIdx.x == 0) delta_node[node] = 0.0;
-      continue;
-    }
+    if (lvl == 0) continue;
     const int par = t.parent[node];
     const int ch = (int)(t.keys[node] & 7ull);
     parent_box(t, p, B, par, ch, pb);
@@ -561,50 +561,55 @@ __global__ void __launch_bounds__(256) k_delta_t(Topo t, Phys p, Pool pool, int 
       gl[d] = (Xd == 0) && (p.bc[2 * d] != 1);
       gh[d] = (Xd == nl - 1) && (p.bc[2 * d + 1] != 1);
     }
-    R m = R(0);
-    for (int vi = 0; vi < 2; ++vi) {
-      const int v = vi == 0 ? 0 : 4;
-      const R first = to_r<R>(box_value(pb, box_word(pb, 0, 0, 0), v));
-      bool eq = const_safe(first);
-      for (int e = threadIdx.x; e < 4096; e += blockDim.x) {
-        const R x = to_r<R>(box_value(pb, box_word(pb, e & 15, (e >> 4) & 15, e >> 8), v));
-        box[e] = x;
-        eq = eq && same_bits(x, first);
-      }
-      const bool constant = __syncthreads_and(eq);       // (a box of one value predicts it)
-      const SAcc<R> A{box, 0, 0, 0, 16, 256};
-      for (int q = threadIdx.x; q < 1728; q += blockDim.x) {
-        const int rx = q % 12 - 2, ry = (q / 12) % 12 - 2, rz = q / 144 - 2;
-        // all eight fine cells of this parent cell share the ghost status
-        const bool ghost = (rx < 0 && gl[0]) || (rx >= 8 && gh[0]) || (ry < 0 && gl[1]) || (ry >= 8 && gh[1]) ||
-                           (rz < 0 && gl[2]) || (rz >= 8 && gh[2]);
-        if (ghost) continue;
-        const double* U = own[own_region(rx, ry, rz)] + v * NCELL + sidx(2 * rx, 2 * ry, 2 * rz);
-        double2 uf[4];
-#pragma unroll
-        for (int q2 = 0; q2 < 4; ++q2)
-          uf[q2] = *reinterpret_cast<const double2*>(U + ((q2 >> 1) * NS + (q2 & 1)) * NS);   // rows y + (q2 & 1), z + (q2 >> 1)
-        QT<R> qt;
-        if (!constant) qt = qterms_t<R>(A, rx + 4, ry + 4, rz + 4);
-#pragma unroll
-        for (int sub = 0; sub < 8; ++sub) {
-          const int a = sub & 1, b = (sub >> 1) & 1, c = (sub >> 2) & 1;
-          const R pr = constant ? first : predict_t<R>(qt, a ? R(-1) : R(1), b ? R(-1) : R(1), c ? R(-1) : R(1));
-          const R u0 = to_r<R>(a ? uf[b + 2 * c].y : uf[b + 2 * c].x);
-          const R r = (u0 - pr) / u0;
-          m = (r < R(0) ? -r : r) > m ? (r < R(0) ? -r : r) : m;
-        }
-      }
-      __syncthreads();
+    double m = 0.0;
+    const double first = box_value(pb, box_word(pb, 0, 0, rz0 + 2), v);
+    bool eq = const_safe(first);
+    for (int e = threadIdx.x; e < 2560; e += blockDim.x) {
+      const double x = box_value(pb, box_word(pb, e & 15, (e >> 4) & 15, rz0 + 2 + (e >> 8)), v);
+      box[e] = x;
+      eq = eq && same_bits(x, first);
     }
-    double md = from_r<R>(m);
-    for (int o = 16; o > 0; o >>= 1) md = fmax(md, __shfl_xor_sync(0xffffffffu, md, o));
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = md;
+    const bool constant = __syncthreads_and(eq);         // (a box of one value predicts it)
+    const SAcc<double> A{box, 0, 0, rz0 + 2, 16, 256};
+    // (the warp's lanes stay together: they share their maximum below)
+    for (int q0 = threadIdx.x & ~31; q0 < 864; q0 += blockDim.x) {
+      const int q = q0 + (threadIdx.x & 31);
+      const int rx = q % 12 - 2, ry = (q / 12) % 12 - 2, rz = q / 144 + rz0;
+      // all eight fine cells of this parent cell share the ghost status
+      const bool ghost = (rx < 0 && gl[0]) || (rx >= 8 && gh[0]) || (ry < 0 && gl[1]) || (ry >= 8 && gh[1]) ||
+                         (rz < 0 && gl[2]) || (rz >= 8 && gh[2]);
+      const unsigned live = __ballot_sync(0xffffffffu, !ghost);
+      if (ghost) continue;
+      const double* U = own[own_region(rx, ry, rz)] + v * NCELL + sidx(2 * rx, 2 * ry, 2 * rz);
+      double2 uf[4];
+#pragma unroll
+      for (int q2 = 0; q2 < 4; ++q2)
+        uf[q2] = *reinterpret_cast<const double2*>(U + ((q2 >> 1) * NS + (q2 & 1)) * NS);   // rows y + (q2 & 1), z + (q2 >> 1)
+      QT<double> qt;
+      if (!constant) qt = qterms_t<double>(A, rx + 4, ry + 4, rz + 4);
+#pragma unroll
+      for (int sub = 0; sub < 8; ++sub) {
+        const int a = sub & 1, b = (sub >> 1) & 1, c = (sub >> 2) & 1;
+        const double pr = constant ? first : predict_t<double>(qt, a ? -1.0 : 1.0, b ? -1.0 : 1.0, c ? -1.0 : 1.0);
+        const double u0 = a ? uf[b + 2 * c].y : uf[b + 2 * c].x, n = fabs(u0 - pr);
+        // A quotient |u - P| / |u| no greater than a maximum of the warp is not
+        // formed (a division is a dozen FP64 instructions): with x <= the maximum and
+        // the product rounded down, |u - P| <= x |u| bounds it.  The comparison is of
+        // bit patterns, in which a NaN is large and takes the division.
+        const double seen = __hiloint2double((int)__reduce_max_sync(live, (unsigned)__double2hiint(m)), 0);
+        if (d2bits(n) <= d2bits(__dmul_rd(seen, fabs(u0)))) continue;
+        const double r = n / fabs(u0);
+        m = r > m ? r : m;
+      }
+    }
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
     __syncthreads();
     if (threadIdx.x == 0) {
       double x = sh[0];
       for (int q = 1; q < (int)(blockDim.x >> 5); ++q) x = fmax(x, sh[q]);
-      delta_node[node] = x;
+      // (the parts of a node; bit patterns of non-negative doubles are ordered)
+      atomicMax(reinterpret_cast<unsigned long long*>(delta_node + node), (unsigned long long)d2bits(x));
     }
     __syncthreads();
   }
@@ -663,10 +668,12 @@ __global__ void __launch_bounds__(256) k_refine_fill_t(Topo t, Pool pool, int cu
 // (internal node, octant): the octant's 512 parent cells come from one child.
 // A thread forms all five variables of a parent cell (twenty 16-byte loads in
 // flight) and, on the mixed-precision path (REC), its FP32 record, which a
-// kernel of its own used to read the average back for.  Bound by the FP64 pipe
-// (eight instructions per value) where the children differ, by reading them
-// where they do not; shock-bubble (levels 0..4): averaging and records 450 ->
-// 301 us per stage.
+// kernel of its own used to read the average back for.  Eight FP64 instructions
+// per value bounded it where the children differ; with the means formed by integers
+// (mean8) it reads the children at 6.0 TB/s of memory traffic: an internal row is 128
+// bytes of 192, and memory is read 128 at a time, so half as much again as the cells
+// hold.  Averaging and records per stage: shock-bubble (levels 0..4) 450 -> 301 us
+// in one pass; ensemble of five 300 -> 269 us with mean8.
 // A 16-byte load that stays where it is written (the compiler moved the loads of
 // later variables behind the arithmetic of earlier ones: four in flight).
 __device__ __forceinline__ double2 load_now(const double* p) {
@@ -705,16 +712,8 @@ static __device__ __forceinline__ void project_level(const Topo& t, const Pool& 
       double U[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        // eight equal values have themselves as mean (2x, 4x, 8x and x/8 are
-        // exact, but for overflow): the sums are FP64-pipe work (eight
-        // instructions of 16 cycles a warp), the comparison is not
-        const unsigned long long x = d2bits(a[v][0].x);
-        const bool same = x == d2bits(a[v][0].y) && x == d2bits(a[v][1].x) && x == d2bits(a[v][1].y) &&
-                          x == d2bits(a[v][2].x) && x == d2bits(a[v][2].y) && x == d2bits(a[v][3].x) &&
-                          x == d2bits(a[v][3].y) && ((x >> 52) & 2047u) < 2040u;
-        if (same) U[v] = a[v][0].x;
-        else U[v] = 0.125 * (((a[v][0].x + a[v][0].y) + (a[v][1].x + a[v][1].y)) +
-                             ((a[v][2].x + a[v][2].y) + (a[v][3].x + a[v][3].y)));
+        const double x[8] = {a[v][0].x, a[v][0].y, a[v][1].x, a[v][1].y, a[v][2].x, a[v][2].y, a[v][3].x, a[v][3].y};
+        U[v] = mean8(x);
         Pp[v * NCELL + sidx(ox + I, oy + J, oz + K)] = U[v];
       }
       rec(slot, iidx(ox + I, oy + J, oz + K), U);
