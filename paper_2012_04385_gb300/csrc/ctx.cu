@@ -84,6 +84,7 @@ struct mrb_ctx {
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   cudaStream_t cap_st = nullptr;     // private stream for capture (the caller's may be the legacy stream)
   bool graph_dirty = true;
+  decltype(h_cnt) cap_cnt;          // the counts that shaped the captured launches
   bool detail_filled = false;        // stored halos are not complete (fill before the details)
   char* h_stage = nullptr;           // pinned staging of the topology uploads
   int32_t* h_list = nullptr;         // pinned staging of work lists
@@ -279,7 +280,7 @@ struct mrb_ctx {
     // inside a capture an event record is a graph node only when marked external
     const unsigned flags = (capturing >= 0) ? cudaEventRecordExternal : cudaEventRecordDefault;
     if (e0) CK(cudaEventRecordWithFlags(e0, st, flags));
-    if (cfg.precision == MRB_FP32_ACC64) launch_rhs_rk_f32(topo(), phys, P, cur, s, dt, nullptr, st);
+    if (cfg.precision == MRB_FP32_ACC64) launch_rhs_rk_f32(topo(), phys, P, cur, s, dt, nullptr, st, n_leaves());
     else launch_rhs_rk_f64(topo(), phys, P, cur, s, dt, nullptr, st);
     if (e1) CK(cudaEventRecordWithFlags(e1, st, flags));
     if (max_lmax > 0) {      // (no jumps on a single level)
@@ -342,7 +343,7 @@ struct mrb_ctx {
             for (int ll = 1; ll <= l; ++ll)
               launch_predict_lts(topo(), phys, P, cur, ll == l ? at : cur, ll, level_nodes(ll), th.th[ll - 1], st);
           }
-          if (cfg.precision == MRB_FP32_ACC64) launch_rhs_rk_f32(topo(), phys, P, at, s, d_dt, nullptr, st, l);
+          if (cfg.precision == MRB_FP32_ACC64) launch_rhs_rk_f32(topo(), phys, P, at, s, d_dt, nullptr, st, level_nodes(l), l);
           else launch_rhs_rk_f64(topo(), phys, P, at, s, d_dt, nullptr, st, l);
           if (full || (s == phys.rk - 1 && at == cur)) launch_lts_copyback(topo(), P, cur, l, st);
           launch_lts_fmac(topo(), phys, P, l, s, d_dt, 0, st);
@@ -360,6 +361,15 @@ struct mrb_ctx {
     project();
   }
 
+  // A count that shapes a captured launch has doubled or halved since: the graphs
+  // still give the same results, in grids for another tree.
+  bool shapes_stale() const {
+    auto off = [](int a, int b) { return std::max(a, b) > 32 && (a > 2 * b || b > 2 * a); };
+    if (off(h_cnt[CNT_NNODES], cap_cnt[CNT_NNODES]) || off(h_cnt[CNT_NLEAVES], cap_cnt[CNT_NLEAVES])) return true;
+    for (int l = 0; l <= max_lmax; ++l)
+      if (off(level_nodes(l), cap_cnt[CNT_LVL + l + 1] - cap_cnt[CNT_LVL + l])) return true;
+    return false;
+  }
   void capture_graphs() {
     for (int g = 0; g < 2; ++g) {
       if (graph[g]) cudaGraphExecDestroy(graph[g]);
@@ -399,6 +409,7 @@ struct mrb_ctx {
     st = user;
     cur = save;
     graph_dirty = false;
+    cap_cnt = h_cnt;
   }
 
   int64_t remesh(const int8_t* tags_dev) {
@@ -814,7 +825,8 @@ int mrb_fill_halos(mrb_ctx* c) {
 int mrb_compute_rhs(mrb_ctx* c, double* rhs_dev) {
   return guarded(c, [&] {
     if (!rhs_dev) throw Err(MRB_EINVAL, "null rhs");
-    if (c->cfg.precision == MRB_FP32_ACC64) launch_rhs_rk_f32(c->topo(), c->phys, c->P, c->cur, 0, nullptr, rhs_dev, c->st);
+    if (c->cfg.precision == MRB_FP32_ACC64)
+      launch_rhs_rk_f32(c->topo(), c->phys, c->P, c->cur, 0, nullptr, rhs_dev, c->st, c->n_leaves());
     else launch_rhs_rk_f64(c->topo(), c->phys, c->P, c->cur, 0, nullptr, rhs_dev, c->st);
     if (c->max_lmax > 0) launch_jump(c->topo(), c->phys, c->P, c->cur, 0, nullptr, rhs_dev, c->st);
   });
@@ -906,7 +918,7 @@ int mrb_step(mrb_ctx* c, int32_t nsteps, double* dt_hist_dev) {
       if (c->phys.lts) {
         c->step_lts();
       } else {
-        if (c->graph_dirty) c->capture_graphs();
+        if (c->graph_dirty || c->shapes_stale()) c->capture_graphs();
         CK(cudaGraphLaunch(c->graph[g], c->st));
         g_kernel_launches += c->graph_kernels[g];
         if (c->phys.rk & 1) c->cur ^= 1;   // every stage flips the stage buffer
@@ -1071,9 +1083,9 @@ int mrb_autotune(mrb_ctx* c, int32_t reps, double* times) {
     auto run = [&](int what) {
       if (what == 0) {
         if (c->cfg.precision == MRB_FP32_ACC64) {
-          launch_rhs_rk_f32(c->topo(), c->phys, c->P, c->cur, 0, c->d_dt, nullptr, c->st);
+          launch_rhs_rk_f32(c->topo(), c->phys, c->P, c->cur, 0, c->d_dt, nullptr, c->st, c->n_leaves());
           if (c->cfg.recon == MRB_RECON_LEARNED && c->cfg.mlp_weights)
-            launch_rhs_rk_f32(c->topo(), c->phys, c->P, c->cur, 1, c->d_dt, nullptr, c->st);
+            launch_rhs_rk_f32(c->topo(), c->phys, c->P, c->cur, 1, c->d_dt, nullptr, c->st, c->n_leaves());
         } else {
           launch_rhs_rk_f64(c->topo(), c->phys, c->P, c->cur, 0, c->d_dt, nullptr, c->st);
         }

@@ -8,8 +8,9 @@
 namespace mrb {
 
 void launch_rhs_rk_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, int stage, const double* dt,
-                       double* rhs_out, cudaStream_t st, int level) {
-  if (p.mu > 0.0) launch_stage_f32<32>(t, p, pool, cur, stage, dt, rhs_out, st, level);   // WENO5, Roe, viscous
+                       double* rhs_out, cudaStream_t st, int n_nodes, int level) {
+  if (thin_slabs(n_nodes) && !(p.recon == 1 && p.mlp)) launch_rhs_rk_f32_thin(t, p, pool, cur, stage, dt, rhs_out, st, level);
+  else if (p.mu > 0.0) launch_stage_f32<32>(t, p, pool, cur, stage, dt, rhs_out, st, level);   // WENO5, Roe, viscous
   else if (p.flux == 1) launch_rhs_rk_f32_llf(t, p, pool, cur, stage, dt, rhs_out, st, level);
   else if (p.flux == 2) launch_rhs_rk_f32_hllc(t, p, pool, cur, stage, dt, rhs_out, st, level);
   else if (p.recon == 2) launch_stage_f32<2>(t, p, pool, cur, stage, dt, rhs_out, st, level);

@@ -156,7 +156,6 @@ void launch_fill_bc(const Topo& t, const Phys& p, const Pool& pool, int cur, cud
 
 void launch_predict(const Topo& t, const Phys& p, const Pool& pool, int cur, int level, int n_nodes, int mode,
                     cudaStream_t st) {
-  if (n_nodes <= 0) return;
   if (p.precision == 1) {
     launch_predict_f32(t, p, pool, cur, level, n_nodes, mode, st);
     return;
@@ -169,7 +168,6 @@ void launch_predict(const Topo& t, const Phys& p, const Pool& pool, int cur, int
 
 void launch_predict_lts(const Topo& t, const Phys& p, const Pool& pool, int cur, int dst, int level, int n_nodes,
                         double th, cudaStream_t st) {
-  if (n_nodes <= 0) return;
   if (p.precision == 1) {
     launch_predict_lts_f32(t, p, pool, cur, dst, level, n_nodes, th, st);
     return;

@@ -177,7 +177,13 @@ void launch_fill_list(const Topo& t, const Phys& p, const Pool& pool, int cur, c
 void launch_rhs_rk_f64(const Topo& t, const Phys& p, const Pool& pool, int cur, int stage, const double* dt,
                        double* rhs_out, cudaStream_t st, int level = -1);
 void launch_rhs_rk_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, int stage, const double* dt,
-                       double* rhs_out, cudaStream_t st, int level = -1);
+                       double* rhs_out, cudaStream_t st, int n_nodes, int level = -1);
+// The same on slabs of two planes (n_nodes: the leaves, or the nodes of `level`).
+// Taken while all their slabs are resident at two CTAs per SM: the stage then lasts as
+// long as one item, 15 us instead of 23 on the Sod tube's 8 blocks; on blocks that vary
+// everywhere a step of 36 takes 115 us, one of 39 (slabs of four) 178.
+void launch_rhs_rk_f32_thin(const Topo& t, const Phys& p, const Pool& pool, int cur, int stage, const double* dt,
+                            double* rhs_out, cudaStream_t st, int level = -1);
 // FP32 stage kernels of the flux variants (separate translation units):
 // LLF on every field, and HLLC, each with every non-learned reconstruction.
 void launch_rhs_rk_f32_llf(const Topo& t, const Phys& p, const Pool& pool, int cur, int stage, const double* dt,
@@ -252,12 +258,16 @@ void launch_get_records(const Topo& t, const Phys& p, const Pool& pool, int cur,
 void launch_face_samples(const Topo& t, const Phys& p, const Pool& pool, int cur, float tau_lab, int64_t stride,
                          float* feats, uint8_t* labels, int64_t* where, int64_t cap, cudaStream_t st);
 int sm_count();
+inline bool thin_slabs(int n_nodes) { return n_nodes * 8 <= 2 * sm_count(); }
 // Grids of kernels whose items differ in length (a detail box of one value, a copy
 // that meets the cache): a CTA per item up to 32 per SM, handed out as CTAs end.
 // With four per SM, of which the registers admit three, the fourth ran alone
 // afterwards: details of the shock-bubble (levels 0..4) 679 -> 474 us, get_state 344
 // -> 326, set_cons 464 -> 416.
 inline int item_grid(int64_t items) { return (int)std::min<int64_t>(items, 32 * (int64_t)sm_count()); }
+// The counts that shape a launch are those at its capture where a graph replays it;
+// the kernels take every item on any grid.
+//
 // Predictions: a CTA per node (up to four items of one), between fill_pred and four
 // times that per SM.  Shock-bubble, 16 launches: 840 us with 4 per SM, 709 with 16;
 // on a few hundred nodes 16 per SM cost a microsecond a launch more than 4.

@@ -25,6 +25,10 @@
 // five values and needs one reciprocal: omega_k = d_k P_k / sum_j d_j P_j with
 // P_k the product of the other two (eps + beta)^2.
 //
+// Thin slabs (SF_THIN, a unit of its own) are 16 x 16 x 2 cells, for launches of so
+// few leaves that every CTA is resident and the length of an item is the length of
+// the stage (thin_slabs in kernels.cuh).
+//
 // The update keeps the stage's increment u^(s) - u^n of every cell in FP32
 // (pool.dl).  With a_s + b_s = 1 the Shu-Osher stage u^(s+1) = a_s u^n + b_s
 // (u^(s) + dt L) is u^n + b_s (increment + dt L): the new increment is formed
@@ -37,11 +41,15 @@
 #include "learned.cuh"
 
 namespace mrb {
-
+#ifdef SF_THIN
+inline namespace thin {
+constexpr int SF_TZ = 2;
+#else
 constexpr int SF_TZ = 4;
+#endif
 constexpr int SF_NSLAB = NB / SF_TZ;
 constexpr int SF_THREADS = 256;
-constexpr int SF_REG = NB * NB * (SF_TZ + 6);            // record slots: the z region, 2560 cells
+constexpr int SF_REG = NB * NB * (SF_TZ + 6);            // record slots: the z region, 2560 cells of slabs of four
 constexpr int SF_XY = 24 * 22 * SF_TZ;                   // x-y region (corners unused): 2112 slots
 constexpr int SF_NFX = 17 * 16 * SF_TZ;                  // x (and y) faces of a slab: 1088
 constexpr int SF_NFZ = NB * NB * (SF_TZ + 1);            // z faces of a slab: 1280
@@ -912,12 +920,12 @@ __device__ __forceinline__ void load_region_f32(int D, const RegionSrc& R, float
 __device__ __forceinline__ int xy_slot(int x, int y, int kz) { return (kz * 22 + y + 3) * 24 + x + 4; }
 
 // 120 chunk positions per plane (16 rows of 6 chunks, 6 rows of 4); threads
-// 0..239 own one position on two of the four planes.
+// 0..239 own one position on half of the planes.
 __device__ __forceinline__ void load_xy_f32(const RegionSrc& R, float* __restrict__ S, int z0, float g, float B,
                                             float gm1) {
   const int t = threadIdx.x;
   if (t < 240) {
-    const int c = t % 120, kz = 2 * (t / 120);
+    const int c = t % 120, kz = SF_TZ / 2 * (t / 120);
     int x0, y;
     if (c < 96) {               // rows y in [0, 16): x = -4 .. 19
       y = c / 6;
@@ -927,7 +935,7 @@ __device__ __forceinline__ void load_xy_f32(const RegionSrc& R, float* __restric
       y = (r < 3) ? r - 3 : r + 13;
       x0 = 4 * ((c - 96) % 4);
     }
-    chunk_planes<2>(R, x0, y, z0 + kz, S, xy_slot(x0, y, kz), xy_slot(0, 0, 1) - xy_slot(0, 0, 0), g, B, gm1);
+    chunk_planes<SF_TZ / 2>(R, x0, y, z0 + kz, S, xy_slot(x0, y, kz), xy_slot(0, 0, 1) - xy_slot(0, 0, 0), g, B, gm1);
   }
   cp_async_wait_all();
 }
@@ -1094,15 +1102,17 @@ __device__ __forceinline__ bool probe3(const float* __restrict__ p, int a, int b
 }
 __device__ __forceinline__ unsigned probe_xy(const float* __restrict__ S) {
   const float* p = S + 4 * SF_REG;
+  constexpr int m = SF_TZ / 2;
   const bool fx = probe3(p, xy_slot(-3, 0, 0), xy_slot(7, 0, 0), xy_slot(18, 0, 0)) &&
-                  probe3(p, xy_slot(-3, 11, 2), xy_slot(7, 11, 2), xy_slot(18, 11, 2));
+                  probe3(p, xy_slot(-3, 11, m), xy_slot(7, 11, m), xy_slot(18, 11, m));
   const bool fy = probe3(p, xy_slot(0, -3, 0), xy_slot(0, 7, 0), xy_slot(0, 18, 0)) &&
-                  probe3(p, xy_slot(11, -3, 2), xy_slot(11, 7, 2), xy_slot(11, 18, 2));
+                  probe3(p, xy_slot(11, -3, m), xy_slot(11, 7, m), xy_slot(11, 18, m));
   return (fx ? 1u : 0u) | (fy ? 2u : 0u);
 }
 __device__ __forceinline__ unsigned probe_z(const float* __restrict__ S) {
   const float* p = S + 4 * SF_REG;
-  return probe3(p, 0, 5 * 256, 9 * 256) && probe3(p, 187, 5 * 256 + 187, 9 * 256 + 187) ? 4u : 0u;
+  constexpr int m = (SF_TZ + 6) / 2 * 256, e = (SF_TZ + 5) * 256;
+  return probe3(p, 0, m, e) && probe3(p, 187, m + 187, e + 187) ? 4u : 0u;
 }
 
 // This thread's share of the tests on the x-y region (bit 0: constant along x,
@@ -1289,7 +1299,7 @@ __device__ __forceinline__ void sweep_xy(const double* __restrict__ u, const Top
   const int nx = flatx ? ((fm & 3u) ? 16 * SF_TZ : 0) : SF_NFX, ny = flaty ? ((fm & 12u) ? 16 * SF_TZ : 0) : SF_NFX;
   for (int f = threadIdx.x; f < nx + ny; f += blockDim.x) {
     float F[5];
-    const bool isx = f < nx;              // warp-uniform (64 or 1088 = 34 warps)
+    const bool isx = f < nx;              // warp-uniform (64 or 1088 = 34 warps; thin slabs 32 or 17 warps)
     const bool one = isx ? flatx : flaty;
     int fa, c0, ta, tb, st, wi;
     if (isx) {
@@ -1582,4 +1592,7 @@ static void launch_stage_f32(const Topo& t, const Phys& p, const Pool& pool, int
   ++g_kernel_launches;
 }
 
+#ifdef SF_THIN
+}  // inline namespace thin
+#endif
 }  // namespace mrb
