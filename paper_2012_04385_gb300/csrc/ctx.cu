@@ -73,6 +73,7 @@ struct mrb_ctx {
           *d_child0 = nullptr, *d_nbr = nullptr, *d_leaves = nullptr, *d_lvl_nodes = nullptr, *d_bc_items = nullptr, *d_jump = nullptr, *d_cnt = nullptr,
           *d_lmax = nullptr, *d_list = nullptr, *d_pst = nullptr, *d_pall = nullptr;
   uint32_t *d_miss = nullptr, *d_smask = nullptr, *d_fmask = nullptr;
+  int32_t* d_side = nullptr;
   double *d_dt = nullptr, *d_delta_node = nullptr, *d_partial = nullptr;
   unsigned long long* d_census = nullptr;   // mrb_flux_census counters (allocated on first use)
   unsigned long long* d_smax = nullptr;
@@ -118,6 +119,7 @@ struct mrb_ctx {
     t.pst = d_pst;
     t.pall = d_pall;
     t.fmask = d_fmask;
+    t.side = d_side;
     t.cnt = d_cnt;
     return t;
   }
@@ -229,7 +231,7 @@ struct mrb_ctx {
     put(d_bc_items, h_bc_items.data(), sizeof(int32_t) * h_bc_items.size());
     put(d_cnt, h_cnt.data(), sizeof(int32_t) * CNT_SIZE);
     launch_nbr(topo(), phys, d_nbr, n, st);
-    launch_masks(topo(), phys, d_miss, d_smask, d_fmask, d_pst, d_pall, d_cnt, max_lmax, st);
+    launch_masks(topo(), phys, d_miss, d_smask, d_fmask, d_side, d_pst, d_pall, d_cnt, max_lmax, st);
     launch_jump_list(topo(), d_jump, d_cnt, (int)h_leaves.size(), st);
     CK(cudaGetLastError());
     CK(cudaEventRecord(stage_ev, st));
@@ -682,6 +684,7 @@ int mrb_init_blocks(const mrb_config* cfg, void* pool, size_t pool_bytes, mrb_ct
     c->d_miss = c->dalloc<uint32_t>(n);
     c->d_smask = c->dalloc<uint32_t>(n);
     c->d_fmask = c->dalloc<uint32_t>(n);
+    c->d_side = c->dalloc<int32_t>(8 * n);
     c->d_pst = c->dalloc<int32_t>(n);
     c->d_pall = c->dalloc<int32_t>(n);
     c->d_cnt = c->dalloc<int32_t>(CNT_SIZE);

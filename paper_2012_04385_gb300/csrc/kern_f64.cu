@@ -701,7 +701,8 @@ __global__ void k_nbr(Topo t, Phys p, int32_t* __restrict__ nbr_out) {
 // octant's side) when s_d is 0 or points out of the parent.
 constexpr uint32_t FACE_REGIONS = (1u << 12) | (1u << 14) | (1u << 10) | (1u << 16) | (1u << 4) | (1u << 22);
 __global__ void k_masks(Topo t, Phys p, uint32_t* __restrict__ miss, uint32_t* __restrict__ smask,
-                        uint32_t* __restrict__ fmask, int32_t* __restrict__ pst, int32_t* __restrict__ pall, int32_t* __restrict__ cnt, int level) {
+                        uint32_t* __restrict__ fmask, int32_t* __restrict__ side, int32_t* __restrict__ pst,
+                        int32_t* __restrict__ pall, int32_t* __restrict__ cnt, int level) {
   const int beg = t.cnt[CNT_LVL + level], end = t.cnt[CNT_LVL + level + 1];
   for (int w = beg + blockIdx.x * blockDim.x + threadIdx.x; w < end; w += gridDim.x * blockDim.x) {
     const int node = t.lvl_nodes[w];
@@ -733,8 +734,12 @@ __global__ void k_masks(Topo t, Phys p, uint32_t* __restrict__ miss, uint32_t* _
     for (int sd = 0; sd < 6; ++sd) {
       const int nb = t.nbr[(size_t)node * 27 + rn[sd]];
       if (nb == -1 || (nb >= 0 && t.child0[nb] >= 0)) fm |= 1u << sd;
+      side[(size_t)node * 8 + sd] = nb >= 0 ? t.slot[nb] : nb;
     }
-    fmask[node] = c0 < 0 ? fm : 0u;
+    if (c0 >= 0) fm = 0u;
+    fmask[node] = fm;
+    side[(size_t)node * 8 + 6] = t.slot[node];
+    side[(size_t)node * 8 + 7] = (int32_t)(fm | ((uint32_t)level << 8));
     miss[node] = ms;
     smask[node] = need & ms;
     if (need & ms) pst[beg + atomicAdd(&cnt[CNT_PST + level], 1)] = node;
@@ -742,10 +747,10 @@ __global__ void k_masks(Topo t, Phys p, uint32_t* __restrict__ miss, uint32_t* _
   }
 }
 
-void launch_masks(const Topo& t, const Phys& p, uint32_t* miss, uint32_t* smask, uint32_t* fmask, int32_t* pst,
-                  int32_t* pall, int32_t* cnt, int max_level, cudaStream_t st) {
+void launch_masks(const Topo& t, const Phys& p, uint32_t* miss, uint32_t* smask, uint32_t* fmask, int32_t* side,
+                  int32_t* pst, int32_t* pall, int32_t* cnt, int max_level, cudaStream_t st) {
   for (int l = max_level; l >= 0; --l) {
-    k_masks<<<sm_count(), 128, 0, st>>>(t, p, miss, smask, fmask, pst, pall, cnt, l);
+    k_masks<<<sm_count(), 128, 0, st>>>(t, p, miss, smask, fmask, side, pst, pall, cnt, l);
     ++g_kernel_launches;
   }
 }

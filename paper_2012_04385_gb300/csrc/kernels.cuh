@@ -52,6 +52,8 @@ struct Topo {
   const uint32_t* smask;   // those that a stage needs (see k_masks)
   const int32_t* pst;      // nodes with smask != 0, grouped by level like lvl_nodes (count CNT_PST + l)
   const int32_t* pall;     // nodes with miss != 0, likewise (count CNT_PALL + l)
+  const int32_t* side;     // [8] per node: slots of the face neighbours (x-, x+, y-, y+, z-, z+; -1 none, -2
+                           // beyond the boundary), own slot, fmask | level << 8: what a stage item asks first
   const uint32_t* fmask;   // 6-bit mask of a leaf's sides whose face fluxes something reads: next to a refined
                            // neighbour (the jump correction's coarse side) or to none (its fine side)
   const int32_t* cnt;      // counts, see CNT_*
@@ -226,7 +228,7 @@ void launch_jump_list(const Topo& t, int32_t* jump, int32_t* cnt, int n_leaves_c
 void launch_nbr(const Topo& t, const Phys& p, int32_t* nbr_out, int nnodes_cap, cudaStream_t st);
 // Masks of predicted regions and the lists of the nodes that have any, levels
 // fine to coarse (max_level .. 0).
-void launch_masks(const Topo& t, const Phys& p, uint32_t* miss, uint32_t* smask, uint32_t* fmask, int32_t* pst,
+void launch_masks(const Topo& t, const Phys& p, uint32_t* miss, uint32_t* smask, uint32_t* fmask, int32_t* side, int32_t* pst,
                   int32_t* pall, int32_t* cnt, int max_level, cudaStream_t st);
 void launch_sums(const Topo& t, const Phys& p, const Pool& pool, int cur, double* partial, double* out,
                  int nleaves_cap, cudaStream_t st);

@@ -946,17 +946,19 @@ __device__ __forceinline__ RegionSrc region_src(const Topo& t, const Phys& p, co
                                                 int slot) {
   RegionSrc R;
   R.u = pool.bufp(cur) + (size_t)slot * SLOT_U;
-  R.sh = pool.shp(cur) ? pool.shp(cur) + (size_t)slot * SLOT_SH : nullptr;
+  const float* sh = pool.shp(cur);
+  R.sh = sh ? sh + (size_t)slot * SLOT_SH : nullptr;
   R.bnd = R.mir = 0u;
-  const int rn[6] = {12, 14, 10, 16, 4, 22};
+  const int4 a = *reinterpret_cast<const int4*>(t.side + (size_t)node * 8);
+  const int2 b = *reinterpret_cast<const int2*>(t.side + (size_t)node * 8 + 4);
+  const int nb[6] = {a.x, a.y, a.z, a.w, b.x, b.y};
 #pragma unroll
   for (int q = 0; q < 6; ++q) {
-    const int nb = R.sh ? t.nbr[(size_t)node * 27 + rn[q]] : -1;
-    if (nb == -2) {
+    if (sh && nb[q] == -2) {
       R.bnd |= 1u << q;
       if (p.bc[q] == 2) R.mir |= 1u << q;
     }
-    R.nsh[q] = (nb >= 0) ? pool.shp(cur) + (size_t)t.slot[nb] * SLOT_SH : nullptr;
+    R.nsh[q] = (sh && nb[q] >= 0) ? sh + (size_t)nb[q] * SLOT_SH : nullptr;
   }
   return R;
 }
@@ -1447,19 +1449,20 @@ __global__ void __launch_bounds__(SF_THREADS, 2)
   for (int w = IR.first; w < IR.end; w += IR.step) {
     const int li = w / SF_NSLAB, z0 = (w % SF_NSLAB) * SF_TZ;
     const int node = stage_node(t, level, li);
-    const int slot = t.slot[node];
+    const int4 own = *reinterpret_cast<const int4*>(t.side + (size_t)node * 8 + 4);
+    const int slot = own.z;
     // the update's per-block scalars, loaded here so that their latency is
     // hidden behind the sweeps (after them in the register-bound selector
     // variant)
     int lvl = 0;
     double h = 0.0;
     if (MODE != 1) {
-      lvl = t.level[node];
+      lvl = own.w >> 8;
       h = dt ? node_dt(t, p, dt, node, level) : 0.0;
     }
     const double* __restrict__ u = src + (size_t)slot * SLOT_U;
     double* __restrict__ fb = pool.face + (size_t)slot * SLOT_F;
-    const unsigned fm = t.fmask[node];
+    const unsigned fm = (unsigned)own.w & 63u;
     if (MODE == 1 || MODE == 3) L.bits = pool.sel + (size_t)slot * SLOT_SEL;
     if (MODE & 32) L.idx = d2f_fast(ldexp(1.0 / p.dx0, t.level[node]));
     update_prefetch(u, pool, slot, z0, rhs_out ? 0 : stage, pool.dl && stage != 0 && !rhs_out && !p.has_grav);
