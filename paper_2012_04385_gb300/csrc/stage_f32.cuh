@@ -768,6 +768,10 @@ __device__ __forceinline__ void cp_async16(float* smem, const float* gmem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
+__device__ __forceinline__ void cp_async4(int* smem, const int* gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
 __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
 }
@@ -942,15 +946,15 @@ __device__ __forceinline__ void load_xy_f32(const RegionSrc& R, float* __restric
 
 // Sources of the block at `slot` with its same-level face neighbours (stage
 // buffer `cur`).
-__device__ __forceinline__ RegionSrc region_src(const Topo& t, const Phys& p, const Pool& pool, int cur, int node,
+__device__ __forceinline__ RegionSrc region_src(const int* __restrict__ side, const Phys& p, const Pool& pool, int cur,
                                                 int slot) {
   RegionSrc R;
   R.u = pool.bufp(cur) + (size_t)slot * SLOT_U;
   const float* sh = pool.shp(cur);
   R.sh = sh ? sh + (size_t)slot * SLOT_SH : nullptr;
   R.bnd = R.mir = 0u;
-  const int4 a = *reinterpret_cast<const int4*>(t.side + (size_t)node * 8);
-  const int2 b = *reinterpret_cast<const int2*>(t.side + (size_t)node * 8 + 4);
+  const int4 a = *reinterpret_cast<const int4*>(side);
+  const int2 b = *reinterpret_cast<const int2*>(side + 4);
   const int nb[6] = {a.x, a.y, a.z, a.w, b.x, b.y};
 #pragma unroll
   for (int q = 0; q < 6; ++q) {
@@ -1175,7 +1179,7 @@ __device__ __forceinline__ void store_sides(int D, const float F[5], bool lo, bo
 // Per-direction sweep (the stage-0 selector variant, MODE 1): region of D,
 // faces with WENO5 fluxes and the selector's decisions, flux differences.
 template <int MODE>
-__device__ __forceinline__ void sweep_f32(int D, const Topo& t, const Phys& p, const Pool& pool, int cur, int node, int slot,
+__device__ __forceinline__ void sweep_f32(int D, const int* side, const Phys& p, const Pool& pool, int cur, int slot,
                                           double* __restrict__ fb, float* __restrict__ S, float* __restrict__ Fs,
                                           int z0, float g, float B, float gm1, float (&acc)[SF_TZ][NV],
                                           const LearnedCtx& L, unsigned (&cnt)[2],   // cnt: the warp's census
@@ -1185,8 +1189,8 @@ __device__ __forceinline__ void sweep_f32(int D, const Topo& t, const Phys& p, c
   // the x-y region serves the x and the y faces (loaded for D = 0 and kept
   // for D = 1), the z region the z faces
   if (D != 1) {
-    if (D == 0) load_xy_f32(region_src(t, p, pool, cur, node, slot), S, z0, g, B, gm1);
-    else load_region_f32(2, region_src(t, p, pool, cur, node, slot), S, z0, g, B, gm1);
+    if (D == 0) load_xy_f32(region_src(side, p, pool, cur, slot), S, z0, g, B, gm1);
+    else load_region_f32(2, region_src(side, p, pool, cur, slot), S, z0, g, B, gm1);
     __syncthreads();
     flat = D == 0 ? probe_xy(S) : probe_z(S);
     if (flat) flat = block_and(D == 0 ? flat_xy(S, B, flat) : flat_z(S, B), flat_sh);
@@ -1279,12 +1283,12 @@ __device__ __forceinline__ void sweep_f32(int D, const Topo& t, const Phys& p, c
 // stride and the rotation's offsets, so one inlined copy serves both; 1.5%
 // faster than one copy per direction).
 template <int MODE>
-__device__ __forceinline__ void sweep_xy(const double* __restrict__ u, const Topo& t, const Phys& p, const Pool& pool, int cur,
-                                         int node, int slot, double* __restrict__ fb, float* __restrict__ S,
+__device__ __forceinline__ void sweep_xy(const double* __restrict__ u, const int* side, const Phys& p, const Pool& pool, int cur,
+                                         int slot, double* __restrict__ fb, float* __restrict__ S,
                                          float* __restrict__ Fs, int z0, float g, float B, float gm1,
                                          float (&acc)[SF_TZ][NV], const LearnedCtx& L, unsigned* flat_sh, unsigned fm) {
   const int ti = threadIdx.x & 15, tj = threadIdx.x >> 4;
-  load_xy_f32(region_src(t, p, pool, cur, node, slot), S, z0, g, B, gm1);
+  load_xy_f32(region_src(side, p, pool, cur, slot), S, z0, g, B, gm1);
   __syncthreads();
   unsigned flat = 0u;
   if (!(MODE & 32)) {                     // (viscous fluxes read other pencils)
@@ -1346,12 +1350,12 @@ __device__ __forceinline__ void sweep_xy(const double* __restrict__ u, const Top
 
 // z direction of the slab (MODES 0, 2, 3).
 template <int MODE>
-__device__ __forceinline__ void sweep_z(const double* __restrict__ u, const Topo& t, const Phys& p, const Pool& pool, int cur,
-                                        int node, int slot, double* __restrict__ fb, float* __restrict__ S,
+__device__ __forceinline__ void sweep_z(const double* __restrict__ u, const int* side, const Phys& p, const Pool& pool, int cur,
+                                        int slot, double* __restrict__ fb, float* __restrict__ S,
                                         float* __restrict__ Fs, int z0, float g, float B, float gm1,
                                         float (&acc)[SF_TZ][NV], const LearnedCtx& L, unsigned* flat_sh, unsigned fm) {
   const int ti = threadIdx.x & 15, tj = threadIdx.x >> 4;
-  load_region_f32(2, region_src(t, p, pool, cur, node, slot), S, z0, g, B, gm1);
+  load_region_f32(2, region_src(side, p, pool, cur, slot), S, z0, g, B, gm1);
   __syncthreads();
   bool flat = false;
   if (!(MODE & 32) && probe_z(S)) {
@@ -1446,10 +1450,32 @@ __global__ void __launch_bounds__(SF_THREADS, 2)
   // atomic pair per 32 faces, all on the same two addresses, serialised in L2
   // and held the kernel up once the all-flat warps had become cheap
   unsigned cnt[2] = {0u, 0u};
-  for (int w = IR.first; w < IR.end; w += IR.step) {
+  // An item starts with its node and the node's words of t.side, copied into shared
+  // memory while the items before it ran (node one item earlier than words; the
+  // copies land with the regions'): no load of it waits for another one.
+  // (A CTA of thin slabs has one.)
+  constexpr bool AHEAD = SF_TZ == 4;
+  __shared__ __align__(16) int side_sh[2][8];
+  __shared__ int node_sh[3];
+  const int32_t* __restrict__ nodes = level < 0 ? t.leaves : t.lvl_nodes + t.cnt[CNT_LVL + level];
+  int b2 = 0, b3 = 0;
+  for (int w = IR.first; w < IR.end; w += IR.step, b2 ^= 1, b3 = b3 == 2 ? 0 : b3 + 1) {
     const int li = w / SF_NSLAB, z0 = (w % SF_NSLAB) * SF_TZ;
-    const int node = stage_node(t, level, li);
-    const int4 own = *reinterpret_cast<const int4*>(t.side + (size_t)node * 8 + 4);
+    const bool first = !AHEAD || w == IR.first;  // (reads both where they are)
+    const int node = first ? nodes[li] : node_sh[b3];
+    const int* side = first ? t.side + (size_t)node * 8 : side_sh[b2];
+    if (AHEAD && threadIdx.x == 0) {
+      const int w1 = w + IR.step, w2 = w1 + IR.step;
+      if (w1 < IR.end) {
+        const int n1 = first ? nodes[w1 / SF_NSLAB] : node_sh[b3 == 2 ? 0 : b3 + 1];
+        const int32_t* src1 = t.side + (size_t)n1 * 8;
+        cp_async16(reinterpret_cast<float*>(side_sh[b2 ^ 1]), reinterpret_cast<const float*>(src1));
+        cp_async16(reinterpret_cast<float*>(side_sh[b2 ^ 1] + 4), reinterpret_cast<const float*>(src1 + 4));
+      }
+      if (first && w1 < IR.end) cp_async4(node_sh + 1, nodes + w1 / SF_NSLAB);
+      if (w2 < IR.end) cp_async4(node_sh + (b3 == 0 ? 2 : b3 - 1), nodes + w2 / SF_NSLAB);
+    }
+    const int4 own = *reinterpret_cast<const int4*>(side + 4);
     const int slot = own.z;
     // the update's per-block scalars, loaded here so that their latency is
     // hidden behind the sweeps (after them in the register-bound selector
@@ -1464,7 +1490,7 @@ __global__ void __launch_bounds__(SF_THREADS, 2)
     double* __restrict__ fb = pool.face + (size_t)slot * SLOT_F;
     const unsigned fm = (unsigned)own.w & 63u;
     if (MODE == 1 || MODE == 3) L.bits = pool.sel + (size_t)slot * SLOT_SEL;
-    if (MODE & 32) L.idx = d2f_fast(ldexp(1.0 / p.dx0, t.level[node]));
+    if (MODE & 32) L.idx = d2f_fast(ldexp(1.0 / p.dx0, own.w >> 8));
     update_prefetch(u, pool, slot, z0, rhs_out ? 0 : stage, pool.dl && stage != 0 && !rhs_out && !p.has_grav);
     // the slab's decision words (read before the first barrier of the sweep)
     if (MODE == 3 && threadIdx.x < 108) sel_sh[threadIdx.x] = L.bits[(z0 / SF_TZ) * 108 + threadIdx.x];
@@ -1478,13 +1504,13 @@ __global__ void __launch_bounds__(SF_THREADS, 2)
         for (int v = 0; v < NV; ++v) acc[kz][v] = 0.f;
       unsigned flat = 0u;
 #pragma unroll 1
-      for (int D = 0; D < 3; ++D) sweep_f32<MODE>(D, t, p, pool, cur, node, slot, fb, S, Fs, z0, g, B, gm1, acc, L, cnt, flat, flat_sh, fm);
+      for (int D = 0; D < 3; ++D) sweep_f32<MODE>(D, side, p, pool, cur, slot, fb, S, Fs, z0, g, B, gm1, acc, L, cnt, flat, flat_sh, fm);
     } else {
-      sweep_xy<MODE>(u, t, p, pool, cur, node, slot, fb, S, Fs, z0, g, B, gm1, acc, L, flat_sh, fm);
-      sweep_z<MODE>(u, t, p, pool, cur, node, slot, fb, S, Fs, z0, g, B, gm1, acc, L, flat_sh, fm);
+      sweep_xy<MODE>(u, side, p, pool, cur, slot, fb, S, Fs, z0, g, B, gm1, acc, L, flat_sh, fm);
+      sweep_z<MODE>(u, side, p, pool, cur, slot, fb, S, Fs, z0, g, B, gm1, acc, L, flat_sh, fm);
     }
     if (MODE == 1) {
-      lvl = t.level[node];
+      lvl = side[7] >> 8;
       h = dt ? node_dt(t, p, dt, node, level) : 0.0;
     }
     // 1 / dx = 2^level / dx0 (exact power-of-two scaling, no division)
