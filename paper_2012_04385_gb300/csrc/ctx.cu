@@ -77,6 +77,8 @@ struct mrb_ctx {
   double *d_dt = nullptr, *d_delta_node = nullptr, *d_partial = nullptr;
   unsigned long long* d_census = nullptr;   // mrb_flux_census counters (allocated on first use)
   unsigned long long* d_smax = nullptr;
+  double** d_hist = nullptr;        // where the next step's time steps also go (mrb_step's dt_hist)
+  bool hist_set = false;
   int8_t* d_tags = nullptr;
   int* d_status = nullptr;
   unsigned long long* d_lin = nullptr;
@@ -271,10 +273,10 @@ struct mrb_ctx {
   int stage_fill() const { return cfg.mu > 0.0 ? FILL_FULL : FILL_STAGE; }
   void stage(int s, const double* dt) {
     cudaEvent_t e0 = nullptr, e1 = nullptr;
-    if (capturing >= 0) {
+    if (capturing >= 0 && prof) {
       e0 = gev[capturing][s][0];
       e1 = gev[capturing][s][1];
-    } else if (prof) {
+    } else if (capturing < 0 && prof) {
       CK(cudaEventCreate(&e0));
       CK(cudaEventCreate(&e1));
       pend.push_back({e0, e1});
@@ -295,7 +297,7 @@ struct mrb_ctx {
     for (int l = max_lmax - 1; l >= 0; --l) launch_project_level(topo(), phys, P, cur, l, st);
   }
   void step_stages() {
-    launch_cfl(topo(), phys, P, cur, d_smax, d_dt, d_status, st);
+    launch_cfl(topo(), phys, P, cur, n_leaves(), d_smax, d_dt, d_hist, d_status, st);
     for (int s = 0; s < phys.rk; ++s) {
       fill_halos(stage_fill());
       stage(s, d_dt);
@@ -315,7 +317,7 @@ struct mrb_ctx {
   // shock-bubble with levels 1 and 2 the passes that did so for every stage were
   // half of a macro step: 7.1 ms, now 3.7 ms.)
   void step_lts() {
-    launch_cfl(topo(), phys, P, cur, d_smax, d_dt, d_status, st);
+    launch_cfl(topo(), phys, P, cur, n_leaves(), d_smax, d_dt, d_hist, d_status, st);
     launch_lts_fmac(topo(), phys, P, 0, 0, d_dt, 1, st);
     const int L = max_lmax;
     const int fmode = stage_fill();
@@ -691,7 +693,8 @@ int mrb_init_blocks(const mrb_config* cfg, void* pool, size_t pool_bytes, mrb_ct
     c->d_lmax = c->dalloc<int32_t>(cfg->n_instances);
     c->d_list = c->dalloc<int32_t>(2 * n);
     c->d_dt = c->dalloc<double>(cfg->n_instances);
-    c->d_smax = c->dalloc<unsigned long long>(4 * (size_t)cfg->n_instances);
+    c->d_smax = c->dalloc<unsigned long long>(4 * (size_t)cfg->n_instances + 1);
+    c->d_hist = c->dalloc<double*>(1);
     c->d_delta_node = c->dalloc<double>(n);
     c->d_partial = c->dalloc<double>(5 * n);
     c->d_tags = c->dalloc<int8_t>(n);
@@ -845,7 +848,7 @@ int mrb_rk_stage(mrb_ctx* c, int32_t stage, const double* dt_dev) {
 int mrb_cfl_dt(mrb_ctx* c, double* dt_dev) {
   return guarded(c, [&] {
     if (!dt_dev) throw Err(MRB_EINVAL, "null dt");
-    launch_cfl(c->topo(), c->phys, c->P, c->cur, c->d_smax, dt_dev, c->d_status, c->st);
+    launch_cfl(c->topo(), c->phys, c->P, c->cur, c->n_leaves(), c->d_smax, dt_dev, nullptr, c->d_status, c->st);
   });
 }
 
@@ -916,6 +919,10 @@ int mrb_refine_keys(mrb_ctx* c, const uint64_t* keys_host, int64_t n, int64_t* n
 int mrb_step(mrb_ctx* c, int32_t nsteps, double* dt_hist_dev) {
   return guarded(c, [&] {
     bool mr = c->max_lmax > 0;
+    if (nsteps > 0 && (dt_hist_dev || c->hist_set)) {
+      launch_set_hist(c->d_hist, dt_hist_dev, c->st);
+      c->hist_set = dt_hist_dev != nullptr;
+    }
     for (int s = 0; s < nsteps; ++s) {
       const int g = c->cur;
       if (c->phys.lts) {
@@ -926,9 +933,6 @@ int mrb_step(mrb_ctx* c, int32_t nsteps, double* dt_hist_dev) {
         g_kernel_launches += c->graph_kernels[g];
         if (c->phys.rk & 1) c->cur ^= 1;   // every stage flips the stage buffer
       }
-      if (dt_hist_dev)
-        CK(cudaMemcpyAsync(dt_hist_dev + (size_t)s * c->cfg.n_instances, c->d_dt, sizeof(double) * c->cfg.n_instances,
-                           cudaMemcpyDeviceToDevice, c->st));
       if (mr) {
         c->fill_halos(FILL_DETAIL);
         c->detail_filled = true;
@@ -980,6 +984,7 @@ int mrb_profile(mrb_ctx* c, int32_t enable) {
       cudaEventDestroy(pr.second);
     }
     c->pend.clear();
+    if (c->prof != (enable != 0)) c->graph_dirty = true;   // (the graphs record events only while profiling)
     c->prof = enable != 0;
     c->prof_ms = 0.0;
     c->prof_rhs = 0;
@@ -1082,7 +1087,7 @@ int mrb_autotune(mrb_ctx* c, int32_t reps, double* times) {
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     const int fmode = c->stage_fill();
-    launch_cfl(c->topo(), c->phys, c->P, c->cur, c->d_smax, c->d_dt, c->d_status, c->st);
+    launch_cfl(c->topo(), c->phys, c->P, c->cur, c->n_leaves(), c->d_smax, c->d_dt, nullptr, c->d_status, c->st);
     auto run = [&](int what) {
       if (what == 0) {
         if (c->cfg.precision == MRB_FP32_ACC64) {

@@ -376,7 +376,8 @@ void launch_delta_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, d
 // levels 0..4: 242 -> 115 us), maxima (exact) and the time step of Eq. (Cfl) in
 // FP64.
 __global__ void __launch_bounds__(256) k_cfl_f32(Topo t, Phys p, Pool pool, int cur,
-                                                 unsigned long long* __restrict__ smax, int* __restrict__ status) {
+                                                 unsigned long long* __restrict__ smax, int* __restrict__ status,
+                                                 double* __restrict__ dt, double** hist) {
   __shared__ float sh[4][8];
   const int nleaves = t.cnt[CNT_NLEAVES];
   const float g = (float)p.gamma, B = (float)p.B;
@@ -431,11 +432,12 @@ __global__ void __launch_bounds__(256) k_cfl_f32(Topo t, Phys p, Pool pool, int 
     }
     __syncthreads();
   }
+  cfl_finish(p, smax, dt, hist);
 }
 
-void launch_cfl_speeds_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, unsigned long long* smax,
-                           int* status, cudaStream_t st) {
-  k_cfl_f32<<<sm_count() * 4, 256, 0, st>>>(t, p, pool, cur, smax, status);
+void launch_cfl_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, int n_leaves, unsigned long long* smax,
+                    double* dt, double** hist, int* status, cudaStream_t st) {
+  k_cfl_f32<<<std::min(n_leaves, 4 * sm_count()), 256, 0, st>>>(t, p, pool, cur, smax, status, dt, hist);
   ++g_kernel_launches;
 }
 

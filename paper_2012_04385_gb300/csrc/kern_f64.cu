@@ -480,16 +480,18 @@ __device__ __forceinline__ void block_max(double v[N], double* sh) {
   __syncthreads();
 }
 
-__global__ void __launch_bounds__(256) k_cfl(Topo t, Phys p, Pool pool, int cur,
-                                             unsigned long long* __restrict__ smax, int* __restrict__ status) {
+// Items are quarters of a leaf (FP64-pipe work, so that few leaves spread over the
+// SMs: Sod tube's 8 blocks 38 -> 16 us).
+__global__ void __launch_bounds__(256) k_cfl(Topo t, Phys p, Pool pool, int cur, unsigned long long* __restrict__ smax,
+                                             int* __restrict__ status, double* __restrict__ dt, double** hist) {
   __shared__ double sh[32];
-  const int nleaves = t.cnt[CNT_NLEAVES];
-  for (int li = blockIdx.x; li < nleaves; li += gridDim.x) {
-    const int node = t.leaves[li];
+  const int nitems = t.cnt[CNT_NLEAVES] * 4;
+  for (int w = blockIdx.x; w < nitems; w += gridDim.x) {
+    const int node = t.leaves[w >> 2];
     const double* U = pool.bufp(cur) + (size_t)t.slot[node] * SLOT_U;
     double m[4] = {0.0, 0.0, 0.0, 0.0};   // max |u_d| + c per direction, max 1/rho
     bool bad = false;
-    for (int e = threadIdx.x; e < NINT; e += blockDim.x) {
+    for (int e = (w & 3) * (NINT / 4) + threadIdx.x; e < ((w & 3) + 1) * (NINT / 4); e += blockDim.x) {
       const int s = sidx(e % 16, (e / 16) % 16, e / 256);
       double Uc[5];
 #pragma unroll
@@ -508,34 +510,22 @@ __global__ void __launch_bounds__(256) k_cfl(Topo t, Phys p, Pool pool, int cur,
       for (int d = 0; d < 4; ++d) atomicMax(&smax[inst * 4 + d], (unsigned long long)__double_as_longlong(m[d]));
     }
   }
+  cfl_finish(p, smax, dt, hist);
 }
 
-__global__ void k_cfl_finish(Phys p, const unsigned long long* __restrict__ smax, double* __restrict__ dt) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= p.n_inst) return;
-  const double s0 = __longlong_as_double((long long)smax[i * 4]);
-  const double s1 = __longlong_as_double((long long)smax[i * 4 + 1]);
-  const double s2 = __longlong_as_double((long long)smax[i * 4 + 2]);
-  const double dxl = ldexp(p.dx0, -p.lmax[i]);
-  double h = p.cfl * dxl / ((s0 + s1) + s2);
-  if (p.mu > 0.0) {
-    // explicit diffusion limit of the viscous terms: k dx^2 / (6 max(mu / rho))
-    const double mr = __longlong_as_double((long long)smax[i * 4 + 3]);
-    const double hv = (p.cfl * (dxl * dxl)) / ((6.0 * p.mu) * mr);
-    h = (hv < h) ? hv : h;
+void launch_cfl(const Topo& t, const Phys& p, const Pool& pool, int cur, int n_leaves, unsigned long long* smax,
+                double* dt, double** hist, int* status, cudaStream_t st) {
+  if (p.precision == 1) {
+    launch_cfl_f32(t, p, pool, cur, n_leaves, smax, dt, hist, status, st);
+    return;
   }
-  dt[i] = h;
+  k_cfl<<<std::min(4 * n_leaves, 4 * sm_count()), 256, 0, st>>>(t, p, pool, cur, smax, status, dt, hist);
+  ++g_kernel_launches;
 }
 
-void launch_cfl(const Topo& t, const Phys& p, const Pool& pool, int cur, unsigned long long* smax, double* dt,
-                int* status, cudaStream_t st) {
-  cudaMemsetAsync(smax, 0, sizeof(unsigned long long) * 4 * p.n_inst, st);
-  if (p.precision == 1) launch_cfl_speeds_f32(t, p, pool, cur, smax, status, st);
-  else {
-    k_cfl<<<sm_count() * 4, 256, 0, st>>>(t, p, pool, cur, smax, status);
-    ++g_kernel_launches;
-  }
-  k_cfl_finish<<<(p.n_inst + 127) / 128, 128, 0, st>>>(p, smax, dt);
+static __global__ void k_set_hist(double** hist, double* row) { *hist = row; }
+void launch_set_hist(double** hist, double* row, cudaStream_t st) {
+  k_set_hist<<<1, 1, 0, st>>>(hist, row);
   ++g_kernel_launches;
 }
 

@@ -214,8 +214,11 @@ void launch_jump(const Topo& t, const Phys& p, const Pool& pool, int target, int
 // averaging of the internal nodes of `level`, with their FP32 records (mixed precision)
 void launch_project_level(const Topo& t, const Phys& p, const Pool& pool, int buf, int level, cudaStream_t st);
 void launch_project_level_f32(const Topo& t, const Phys& p, const Pool& pool, int buf, int level, cudaStream_t st);
-void launch_cfl(const Topo& t, const Phys& p, const Pool& pool, int cur, unsigned long long* smax, double* dt,
-                int* status, cudaStream_t st);
+// smax: 4 maxima per instance and a count, all zero between launches.  hist (nullable): device pointer to where the
+// next row of time steps also goes.
+void launch_cfl(const Topo& t, const Phys& p, const Pool& pool, int cur, int n_leaves, unsigned long long* smax,
+                double* dt, double** hist, int* status, cudaStream_t st);
+void launch_set_hist(double** hist, double* row, cudaStream_t st);
 void launch_delta_tags(const Topo& t, const Phys& p, const Pool& pool, int cur, double* delta_node,
                        int allow_refine, int8_t* tags, double* delta_leaf, int n_leaves_cap, int n_nodes,
                        cudaStream_t st);
@@ -245,8 +248,8 @@ void launch_flux_census(const Topo& t, const Phys& p, const Pool& pool, int cur,
                         cudaStream_t st);
 void launch_delta_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, double* delta_node, int all_nodes,
                       int n_nodes, cudaStream_t st);
-void launch_cfl_speeds_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, unsigned long long* smax,
-                           int* status, cudaStream_t st);
+void launch_cfl_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, int n_leaves, unsigned long long* smax,
+                    double* dt, double** hist, int* status, cudaStream_t st);
 // FP32 records of stage buffer b from its FP64 internal cells (mixed-precision
 // path): SH_JUMP the boundary planes that the jump correction changed, SH_LIST
 // the nodes of a device list of n entries (every `stride`-th entry is a node

@@ -721,4 +721,43 @@ static __device__ __forceinline__ void project_level(const Topo& t, const Pool& 
   }
 }
 
+// ---------------------------------------------------------------- time step
+// The end of a CFL kernel: the CTA that finishes last turns the instances' maxima
+// into time steps (Eq. (Cfl)), and leaves the maxima and the count of CTAs
+// (smax[4 n_inst]) at zero for the next one; with `hist` the steps also go to
+// *hist, which moves on by one row.  (A fill before, a kernel and a copy after
+// it cost a single-level step three launches of six, and their gaps.)
+static __device__ __forceinline__ void cfl_finish(const Phys& p, unsigned long long* __restrict__ smax,
+                                                  double* __restrict__ dt, double** hist) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(&smax[4 * p.n_inst], 1ull) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double* row = hist ? *hist : nullptr;
+  for (int i = threadIdx.x; i < p.n_inst; i += blockDim.x) {
+    double s[4];
+    for (int d = 0; d < 4; ++d) {
+      s[d] = __longlong_as_double((long long)__ldcg(&smax[i * 4 + d]));
+      smax[i * 4 + d] = 0ull;
+    }
+    const double dxl = ldexp(p.dx0, -p.lmax[i]);
+    double h = p.cfl * dxl / ((s[0] + s[1]) + s[2]);
+    if (p.mu > 0.0) {
+      // explicit diffusion limit of the viscous terms: k dx^2 / (6 max(mu / rho))
+      const double hv = (p.cfl * (dxl * dxl)) / ((6.0 * p.mu) * s[3]);
+      h = (hv < h) ? hv : h;
+    }
+    dt[i] = h;
+    if (row) row[i] = h;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    smax[4 * p.n_inst] = 0ull;
+    if (row) *hist = row + p.n_inst;
+  }
+}
+
 }  // namespace mrb
