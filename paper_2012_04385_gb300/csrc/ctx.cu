@@ -243,8 +243,14 @@ struct mrb_ctx {
 
   std::vector<int32_t> nodes_of(const uint64_t* keys, int64_t n) const {
     std::vector<int32_t> out((size_t)n);
+    // ascending ids, as mrb_list_blocks gives them, follow the last one found by a few
+    // nodes; others are searched
+    int64_t i = -1;
+    const int64_t nn = (int64_t)nodes.size();
     for (int64_t b = 0; b < n; ++b) {
-      int64_t i = find(keys[b]);
+      int64_t j = i + 1;
+      while (j < nn && j < i + 12 && nodes[j].key < keys[b]) ++j;
+      i = (j < nn && nodes[j].key == keys[b]) ? j : find(keys[b]);
       if (i < 0) throw Err(MRB_EINVAL, "unknown block id");
       out[b] = (int32_t)i;
     }
