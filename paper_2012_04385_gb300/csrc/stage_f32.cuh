@@ -1510,7 +1510,7 @@ __global__ void __launch_bounds__(SF_THREADS, 2)
       sweep_z<MODE>(u, side, p, pool, cur, slot, fb, S, Fs, z0, g, B, gm1, acc, L, flat_sh, fm);
     }
     if (MODE == 1) {
-      lvl = side[7] >> 8;
+      lvl = t.level[node];                   // (not side: thread 0 may be an item ahead)
       h = dt ? node_dt(t, p, dt, node, level) : 0.0;
     }
     // 1 / dx = 2^level / dx0 (exact power-of-two scaling, no division)
