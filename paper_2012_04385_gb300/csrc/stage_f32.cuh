@@ -1274,7 +1274,7 @@ __device__ __forceinline__ void sweep_f32(int D, const int* side, const Phys& p,
     else { lo = (kz * 16 + tj) * 16 + ti; hi = lo + 256; }
     add_diff(D, Fs, SF_NFZ, lo, hi, acc[kz]);
   }
-  __syncthreads();
+  if (D == 0) __syncthreads();       // (the barrier of the next region's load does for the others)
 }
 
 // x and y directions of the slab together (MODES 0, 2, 3): one region, one
@@ -1345,16 +1345,16 @@ __device__ __forceinline__ void sweep_xy(const double* __restrict__ u, const int
     if (!flatx) add_diff(0, Fs, SF_FMAX, lx, lx + 1, acc[kz]);
     if (!flaty) add_diff(1, Fs, SF_FMAX, ly, ly + 16, acc[kz]);
   }
-  __syncthreads();
+  // (the flux slots are written again after the barrier of the z region's load)
 }
 
-// z direction of the slab (MODES 0, 2, 3).
+// z faces of the slab (MODES 0, 2, 3); true where it is constant along z.  The caller
+// synchronises and adds the differences (add_z).
 template <int MODE>
-__device__ __forceinline__ void sweep_z(const double* __restrict__ u, const int* side, const Phys& p, const Pool& pool, int cur,
+__device__ __forceinline__ bool sweep_z(const double* __restrict__ u, const int* side, const Phys& p, const Pool& pool, int cur,
                                         int slot, double* __restrict__ fb, float* __restrict__ S,
                                         float* __restrict__ Fs, int z0, float g, float B, float gm1,
-                                        float (&acc)[SF_TZ][NV], const LearnedCtx& L, unsigned* flat_sh, unsigned fm) {
-  const int ti = threadIdx.x & 15, tj = threadIdx.x >> 4;
+                                        const LearnedCtx& L, unsigned* flat_sh, unsigned fm) {
   load_region_f32(2, region_src(side, p, pool, cur, slot), S, z0, g, B, gm1);
   __syncthreads();
   bool flat = false;
@@ -1375,14 +1375,13 @@ __device__ __forceinline__ void sweep_z(const double* __restrict__ u, const int*
     if (flat) store_sides(2, F, lo, hi, i, j, fb);
     else store_face(2, F, Fs, SF_FMAX, f, z0 + fa, i, j, fb, fm);
   }
-  __syncthreads();
-  if (!flat) {
+  return flat;
+}
+__device__ __forceinline__ void add_z(const float* __restrict__ Fs, float (&acc)[SF_TZ][NV]) {
 #pragma unroll
-    for (int kz = 0; kz < SF_TZ; ++kz) {
-      const int lz = (kz * 16 + tj) * 16 + ti;
-      add_diff(2, Fs, SF_FMAX, lz, lz + 256, acc[kz]);
-    }
-    __syncthreads();
+  for (int kz = 0; kz < SF_TZ; ++kz) {
+    const int lz = (kz * 16 + (threadIdx.x >> 4)) * 16 + (threadIdx.x & 15);
+    add_diff(2, Fs, SF_FMAX, lz, lz + 256, acc[kz]);
   }
 }
 
@@ -1495,6 +1494,7 @@ __global__ void __launch_bounds__(SF_THREADS, 2)
     // the slab's decision words (read before the first barrier of the sweep)
     if (MODE == 3 && threadIdx.x < 108) sel_sh[threadIdx.x] = L.bits[(z0 / SF_TZ) * 108 + threadIdx.x];
     float acc[SF_TZ][NV];
+    bool constant_z = true;
     if (MODE == 1) {
       // with the selector inlined, one copy of the sweep (direction at run
       // time) keeps the kernel within the instruction cache
@@ -1507,7 +1507,7 @@ __global__ void __launch_bounds__(SF_THREADS, 2)
       for (int D = 0; D < 3; ++D) sweep_f32<MODE>(D, side, p, pool, cur, slot, fb, S, Fs, z0, g, B, gm1, acc, L, cnt, flat, flat_sh, fm);
     } else {
       sweep_xy<MODE>(u, side, p, pool, cur, slot, fb, S, Fs, z0, g, B, gm1, acc, L, flat_sh, fm);
-      sweep_z<MODE>(u, side, p, pool, cur, slot, fb, S, Fs, z0, g, B, gm1, acc, L, flat_sh, fm);
+      constant_z = sweep_z<MODE>(u, side, p, pool, cur, slot, fb, S, Fs, z0, g, B, gm1, L, flat_sh, fm);
     }
     if (MODE == 1) {
       lvl = t.level[node];                   // (not side: thread 0 may be an item ahead)
@@ -1524,13 +1524,13 @@ __global__ void __launch_bounds__(SF_THREADS, 2)
     const double ka = kRkA[rk_row(p)][stage], kb = kRkB[rk_row(p)][stage];
     const float hf = d2f_fast(hdx), bhf = d2f_fast(kb * hdx), kbf = d2f_fast(kb);
     const bool incr = pool.dl && stage != 0 && !rhs_out && !p.has_grav;
-    // the thread's four cells in groups of KC: every FP64 operand of a group is
-    // loaded before its first store, so those loads are in flight together
-    // (groups of one cell in the register-bound selector variant)
+    // the thread's cells in groups of KC: every FP64 operand of a group is loaded
+    // before its first store, so those loads are in flight together (groups of one
+    // cell in the register-bound selector variant) -- and, the group being all of
+    // them, before the wait for the other warps' z faces
     constexpr int KC = (MODE == 1) ? 1 : SF_TZ;
-#pragma unroll
-    for (int k0 = 0; k0 < SF_TZ; k0 += KC) {
-      double us[KC][NV], un[KC][NV];
+    double us[KC][NV], un[KC][NV];
+    auto load_group = [&](int k0) {
 #pragma unroll
       for (int c = 0; c < KC; ++c) {
         const int s = sidx(ti, tj, z0 + k0 + c), ii = iidx(ti, tj, z0 + k0 + c);
@@ -1542,6 +1542,15 @@ __global__ void __launch_bounds__(SF_THREADS, 2)
           un[c][v] = (stage != 0 && !rhs_out) ? pool.un[(size_t)slot * SLOT_N + v * NINT + ii] : 0.0;
         }
       }
+    };
+    if (MODE != 1) {
+      load_group(0);
+      __syncthreads();
+      if (!constant_z) add_z(Fs, acc);
+    }
+#pragma unroll
+    for (int k0 = 0; k0 < SF_TZ; k0 += KC) {
+      if (MODE == 1) load_group(k0);
 #pragma unroll
       for (int c = 0; c < KC; ++c) {
         const int kz = k0 + c, k = z0 + kz;
