@@ -26,8 +26,8 @@
 // Measured (GB300; flux and update kernels together, before: one kernel per
 // z-slab with compiler divisions): shock-bubble on levels 0..2, 316 leaves,
 // 27.1 ms -> 7.6 ms per stage; TENO5 and LLF on 60 periodic leaves without
-// uniform data 5.34 ms -> 2.33 ms; Sod tube on 8 leaves 2.78 ms -> 0.25 ms.  The
-// FP64 pipe is 77% busy, with 14% of the issue slots used.
+// uniform data 5.34 ms -> 2.17 ms; Sod tube on 8 leaves 2.78 ms -> 0.23 ms.  With
+// eight warps a CTA the FP64 pipe was 77% busy, with 14% of the issue slots used.
 //
 // Scratch.  The differences live in the stage buffer that the stage is about to
 // write: those of x at the cells themselves, those of y and z in its halo,
@@ -40,7 +40,12 @@ namespace mrb {
 
 constexpr int F64_P = 32;                     // pencils per item (16 on small trees)
 constexpr int F64_L = NB + 6;                 // cells per pencil
-constexpr int F64_WARPS = 8;                  // two CTAs and 128 registers a thread per SM
+// 17 face planes are two rounds of nine warps (of eight: three, the last with one
+// warp), which outweighs the 112 registers a thread that two such CTAs leave (128).
+// Flux kernel with 8 -> 9 warps: 60 smooth blocks 2.33 -> 2.16 ms, Sod tube 231 -> 218
+// us, shock-bubble 7.54 -> 7.48 ms; 6 warps and 168 registers 2.18, 234, 7.76; 11 warps
+// and 88 registers 2.21, 217, 7.66.
+constexpr int F64_WARPS = 9;
 constexpr int F64_THREADS = 32 * F64_WARPS;
 constexpr size_t F64_SMEM = sizeof(double) * (CQ_N * F64_L * F64_P + NV * (NB + 1) * F64_P);
 
@@ -86,7 +91,8 @@ static __global__ void __launch_bounds__(F64_THREADS, 2)
   for (int w = IR.first; w < IR.end; w += IR.step) {
     const int node = stage_node(t, level, w / per_leaf);
     const int D = (w % per_leaf) / per_dir, pp = ((w % per_dir) << lp) + pl;
-    const int slot = t.slot[node];
+    const int4 own = *reinterpret_cast<const int4*>(t.side + (size_t)node * 8 + 4);
+    const int slot = own.z;
     const double* __restrict__ u = src + (size_t)slot * SLOT_U;
     for (int i = warp * nsub + sub; i < F64_L; i += F64_WARPS * nsub) {
       // beyond the block: the face neighbour's internal cells, the block's own
@@ -95,9 +101,9 @@ static __global__ void __launch_bounds__(F64_THREADS, 2)
       const double* __restrict__ cells = u;
       bool flip = false;
       if (c < 0 || c >= NB) {
-        const int hi = c >= NB, nb = t.nbr[(size_t)node * 27 + 13 + (hi ? 1 : -1) * (D == 0 ? 1 : (D == 1 ? 3 : 9))];
+        const int hi = c >= NB, nb = t.side[(size_t)node * 8 + 2 * D + hi];
         if (nb >= 0) {
-          cells = src + (size_t)t.slot[nb] * SLOT_U;
+          cells = src + (size_t)nb * SLOT_U;
           c += hi ? -NB : NB;
         } else if (nb == -2) {
           const bool mirror = p.bc[2 * D + hi] == 2;
@@ -163,7 +169,7 @@ static __global__ void __launch_bounds__(F64_THREADS, 2)
     // direction frame is axis (D + j) mod 3)
     double* __restrict__ o = dst + (size_t)slot * SLOT_U;
     double* __restrict__ fb = pool.face + (size_t)slot * SLOT_F;
-    const unsigned fm = t.fmask[node];          // sides whose fluxes something reads
+    const unsigned fm = (unsigned)own.w & 63u;  // sides whose fluxes something reads
     for (int e = warp * nsub + sub; e < NV * (NB + 2); e += F64_WARPS * nsub) {
       const int v = e / (NB + 2), i = e % (NB + 2);
       const int vl = (v == 0 || v == 4) ? v : 1 + (D + v - 1) % 3;
