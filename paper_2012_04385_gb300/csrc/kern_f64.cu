@@ -809,15 +809,12 @@ __global__ void __launch_bounds__(256) k_sums_partial(Topo t, Phys p, Pool pool,
   }
 }
 
-// One CTA per instance, whose leaves are consecutive.  The partial sums are
-// added in leaf order (the fixed order of the totals), a serial chain of FP64
-// additions; the CTA stages them ahead of the five threads that add.  Before,
-// every addition waited for three dependent loads: 513 us for 3,200 leaves.
-__global__ void __launch_bounds__(256) k_sums_finish(Topo t, Phys p, const double* __restrict__ partial,
-                                                     double* __restrict__ out) {
-  constexpr int CH = 256;
-  __shared__ double buf[2][CH * NV];
-  const int inst = blockIdx.x, nleaves = t.cnt[CNT_NLEAVES];
+// One CTA per instance, whose leaves are consecutive; a warp per variable.  (One
+// thread per variable adding in leaf order was a chain of FP64 additions 49 ns apart:
+// 149 us for 3,056 leaves, so 14.)
+__global__ void __launch_bounds__(32 * NV) k_sums_finish(Topo t, Phys p, const double* __restrict__ partial,
+                                                         double* __restrict__ out) {
+  const int inst = blockIdx.x, nleaves = t.cnt[CNT_NLEAVES], v = threadIdx.x >> 5;
   int below = 0, mine = nleaves;
   if (p.n_inst > 1) {
     __shared__ int cnt[2];
@@ -835,16 +832,8 @@ __global__ void __launch_bounds__(256) k_sums_finish(Topo t, Phys p, const doubl
     below = cnt[0];
     mine = cnt[1];
   }
-  const double* __restrict__ src = partial + (size_t)below * NV;
-  double acc = 0.0;
-  for (int c = 0, b = 0; c < mine; c += CH, b ^= 1) {
-    const int m = (mine - c < CH ? mine - c : CH) * NV;
-    for (int e = threadIdx.x; e < m; e += blockDim.x) buf[b][e] = src[(size_t)c * NV + e];
-    __syncthreads();       // (the other buffer is read until the next barrier at most)
-    if (threadIdx.x < NV)
-      for (int e = threadIdx.x; e < m; e += NV) acc += buf[b][e];
-  }
-  if (threadIdx.x < NV) out[inst * NV + threadIdx.x] = acc;
+  const double total = block_total(partial + (size_t)below * NV, mine, v);
+  if ((threadIdx.x & 31) == 0) out[inst * NV + v] = total;
 }
 
 void launch_sums(const Topo& t, const Phys& p, const Pool& pool, int cur, double* partial, double* out,
@@ -852,7 +841,7 @@ void launch_sums(const Topo& t, const Phys& p, const Pool& pool, int cur, double
   (void)nleaves_cap;
   k_sums_partial<<<sm_count() * 16, 256, 0, st>>>(t, p, pool, cur, partial);
   ++g_kernel_launches;
-  k_sums_finish<<<p.n_inst, 256, 0, st>>>(t, p, partial, out);
+  k_sums_finish<<<p.n_inst, 32 * NV, 0, st>>>(t, p, partial, out);
   ++g_kernel_launches;
 }
 

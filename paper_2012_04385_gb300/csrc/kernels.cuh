@@ -283,4 +283,19 @@ inline int predict_grid(int n_nodes) {
 // kernel launches issued by this process (host-side counter, bumped by every launch_* wrapper)
 extern long long g_kernel_launches;
 
+// Total of the per-block sums src[b][NV], b < n, of variable v: lane l adds blocks l,
+// l + 32, ... in turn, then the lanes' sums pairwise -- the fixed order of every
+// total (one warp per variable; the result is in every lane).
+__device__ __forceinline__ double block_total(const double* __restrict__ src, int64_t n, int v) {
+  double acc = 0.0;
+  int64_t b = threadIdx.x & 31;
+  for (; b + 96 < n; b += 128) {                 // (four loads in flight)
+    const double x0 = src[b * NV + v], x1 = src[(b + 32) * NV + v], x2 = src[(b + 64) * NV + v], x3 = src[(b + 96) * NV + v];
+    acc = ((((acc + x0) + x1) + x2) + x3);
+  }
+  for (; b < n; b += 32) acc += src[b * NV + v];
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  return acc;
+}
+
 }  // namespace mrb

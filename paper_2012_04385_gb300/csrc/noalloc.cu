@@ -65,11 +65,9 @@ __global__ void __launch_bounds__(256) k_noalloc_partial(const double* __restric
 }
 
 __global__ void k_noalloc_finish(const double* __restrict__ partial, int64_t n, double* __restrict__ out) {
-  const int v = threadIdx.x;
-  if (v >= 5) return;
-  double acc = 0.0;
-  for (int64_t b = 0; b < n; ++b) acc += partial[(size_t)b * 5 + v];
-  out[v] = acc;
+  const int v = threadIdx.x >> 5;               // a warp per variable
+  const double total = block_total(partial, n, v);
+  if ((threadIdx.x & 31) == 0) out[v] = total;
 }
 
 namespace {
@@ -116,7 +114,7 @@ extern "C" int mrb_block_sums_noalloc(const double* blocks_dev, int64_t n_blocks
   if (e == cudaSuccess) {
     const double* partial = scratch;
     void* a2[] = {(void*)&partial, (void*)&n_blocks, (void*)&sums_dev};
-    e = cudaLaunchKernel((const void*)k_noalloc_finish, dim3(1), dim3(32), a2, 0, st);
+    e = cudaLaunchKernel((const void*)k_noalloc_finish, dim3(1), dim3(32 * NV), a2, 0, st);
     if (e == cudaSuccess) ++g_kernel_launches;
   }
   if (e != cudaSuccess) {
