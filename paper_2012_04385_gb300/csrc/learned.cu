@@ -1,7 +1,6 @@
 // Learned reconstruction selector: training-data generation from the solver's
 // own faces, training (forward and backward of the BF16-operand perceptron
 // with FP32 accumulation, Adam), and tensor-core inference.  See learned.cuh.
-#include <cstddef>
 #include <cstring>
 #include <algorithm>
 

@@ -27,7 +27,8 @@
 // z-slab with compiler divisions): shock-bubble on levels 0..2, 316 leaves,
 // 27.1 ms -> 7.6 ms per stage; TENO5 and LLF on 60 periodic leaves without
 // uniform data 5.34 ms -> 2.17 ms; Sod tube on 8 leaves 2.78 ms -> 0.23 ms.  With
-// eight warps a CTA the FP64 pipe was 77% busy, with 14% of the issue slots used.
+// nine warps a CTA the FP64 pipe is 83% busy (eight: 77%), with 15% of the issue
+// slots used.
 //
 // Scratch.  The differences live in the stage buffer that the stage is about to
 // write: those of x at the cells themselves, those of y and z in its halo,
@@ -41,7 +42,7 @@ namespace mrb {
 constexpr int F64_P = 32;                     // pencils per item (16 on small trees)
 constexpr int F64_L = NB + 6;                 // cells per pencil
 // 17 face planes are two rounds of nine warps (of eight: three, the last with one
-// warp), which outweighs the 112 registers a thread that two such CTAs leave (128).
+// warp), which outweighs the 96 registers a thread that two such CTAs leave (128).
 // Flux kernel with 8 -> 9 warps: 60 smooth blocks 2.33 -> 2.16 ms, Sod tube 231 -> 218
 // us, shock-bubble 7.54 -> 7.48 ms; 6 warps and 168 registers 2.18, 234, 7.76; 11 warps
 // and 88 registers 2.21, 217, 7.66.
