@@ -268,13 +268,12 @@ def roofline_numbers(linear_fraction=0.0, split=None, table=None):
 
 
 # DRAM bytes (read + write) per leaf cell of one launch of the stage kernels
-# on the shock-bubble workload (levels 0..4, 5,720 leaves), from the
-# full-size ncu capture summarised in
-# profiles/stage_kernels_shock_bubble_512.md: the mean over one step, for the
-# learned path k_stage_f32<1> (250.8) and k_stage_f32<3> twice (222.6), for
-# the WENO5 path k_stage_f32<0> (247.2 at stage 0, 222.2 at stages 1 and 2).
+# on the shock-bubble workload (levels 0..4, 5,608 leaves), from the
+# full-size ncu capture summarised in profiles/stage_kernels.md: the mean over
+# one step, for the learned path k_stage_f32<1> (261.9) and k_stage_f32<3>
+# (228.9, 228.3), for the WENO5 path k_stage_f32<0> (261.1, 223.4, 223.3).
 # Traffic grows in proportion to the leaf cells of a launch.
-TRAFFIC_BYTES_PER_CELL = {"learned": 232.2, "weno": 230.6}
+TRAFFIC_BYTES_PER_CELL = {"learned": 239.7, "weno": 235.9}
 
 
 def measured_peaks():
