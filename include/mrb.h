@@ -171,7 +171,9 @@ int mrb_set_state(mrb_ctx* ctx, const uint64_t* keys_host, int64_t n, const doub
 int mrb_set_cons(mrb_ctx* ctx, const uint64_t* keys_host, int64_t n, const double* cons_dev);
 
 /* Conserved state of the listed blocks into cons_dev: [n][5][16^3] internal
- * cells (with_halo = 0) or [n][5][24^3] stored cells (with_halo = 1). */
+ * cells (with_halo = 0) or [n][5][24^3] stored cells (with_halo = 1; the halos
+ * are those of the last mrb_fill_halos, as long as the state has not moved on:
+ * stages and steps fill only the predicted regions they read). */
 int mrb_get_state(mrb_ctx* ctx, const uint64_t* keys_host, int64_t n, double* cons_dev, int32_t with_halo);
 
 /* FP32 primitive records (rho, u, v, w, p, E) of the internal cells of the
@@ -194,7 +196,8 @@ int mrb_fill_halos(mrb_ctx* ctx);
  * Sec. 2.2: characteristic WENO5-JS, Roe flux with local Lax-Friedrichs
  * fallback per field), with the jump flux correction applied (Sec. 4), into
  * rhs_dev [n_leaves][5][16^3] in leaf order.  Inspection form: the time
- * stepping uses the fused mrb_rk_stage.  Halos must be filled. */
+ * stepping uses the fused mrb_rk_stage.  Halos must be filled.  (The halo of the
+ * other stage buffer is scratch.) */
 int mrb_compute_rhs(mrb_ctx* ctx, double* rhs_dev);
 
 /* One Runge-Kutta stage (stage = 0 .. rk_stages - 1) on every leaf, fused
@@ -253,10 +256,11 @@ int mrb_refine_level(mrb_ctx* ctx, int32_t level, int64_t* n_leaves);
 int mrb_refine_keys(mrb_ctx* ctx, const uint64_t* keys_host, int64_t n, int64_t* n_leaves);
 
 /* nsteps complete steps: dt from Eq. (Cfl), three fused stages each preceded
- * by the halo fill and followed by the averaging, then (when any lmax > 0)
- * halo fill, MR analysis and remesh.  dt_hist_dev (device, nullable)
+ * by the predictions of the halo regions without a same-level neighbour (the
+ * others are read where they are) and followed by the averaging, then (when any
+ * lmax > 0) predictions, MR analysis and remesh.  dt_hist_dev (device, nullable)
  * receives [nsteps][n_instances] time steps.  The stage sequence is replayed
- * from a CUDA graph. */
+ * from a CUDA graph, captured again when the tree has doubled or halved. */
 int mrb_step(mrb_ctx* ctx, int32_t nsteps, double* dt_hist_dev);
 
 /* Conserved totals per instance: sum over leaves of U dx_l^3, [n_instances][5]
