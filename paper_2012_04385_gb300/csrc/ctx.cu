@@ -244,7 +244,8 @@ struct mrb_ctx {
   std::vector<int32_t> nodes_of(const uint64_t* keys, int64_t n) const {
     std::vector<int32_t> out((size_t)n);
     // ascending ids, as mrb_list_blocks gives them, follow the last one found by a few
-    // nodes; others are searched
+    // nodes; others are searched (the host's part between tags and get_state of 5,608
+    // leaves: 375 -> 237 us)
     int64_t i = -1;
     const int64_t nn = (int64_t)nodes.size();
     for (int64_t b = 0; b < n; ++b) {
