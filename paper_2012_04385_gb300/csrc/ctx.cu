@@ -132,6 +132,12 @@ struct mrb_ctx {
     allocs.push_back(p);
     return (T*)p;
   }
+  // Arrays that a kernel reads before anything has written them: their first value is zero.
+  template <class T> T* dalloc_zero(size_t n) {
+    T* p = dalloc<T>(n);
+    CK(cudaMemsetAsync(p, 0, std::max<size_t>(n, 1) * sizeof(T), st));
+    return p;
+  }
 
   int64_t find(uint64_t key) const {
     auto it = std::lower_bound(nodes.begin(), nodes.end(), key, [](const HNode& a, uint64_t k) { return a.key < k; });
@@ -696,17 +702,18 @@ int mrb_init_blocks(const mrb_config* cfg, void* pool, size_t pool_bytes, mrb_ct
     c->d_side = c->dalloc<int32_t>(8 * n);
     c->d_pst = c->dalloc<int32_t>(n);
     c->d_pall = c->dalloc<int32_t>(n);
-    c->d_cnt = c->dalloc<int32_t>(CNT_SIZE);
+    c->d_cnt = c->dalloc_zero<int32_t>(CNT_SIZE);
     c->d_lmax = c->dalloc<int32_t>(cfg->n_instances);
     c->d_list = c->dalloc<int32_t>(2 * n);
     c->d_dt = c->dalloc<double>(cfg->n_instances);
-    c->d_smax = c->dalloc<unsigned long long>(4 * (size_t)cfg->n_instances + 1);
-    c->d_hist = c->dalloc<double*>(1);
+    // (the CFL kernel finds its maxima and count at zero, and no row of time steps asked for)
+    c->d_smax = c->dalloc_zero<unsigned long long>(4 * (size_t)cfg->n_instances + 1);
+    c->d_hist = c->dalloc_zero<double*>(1);
     c->d_delta_node = c->dalloc<double>(n);
     c->d_partial = c->dalloc<double>(5 * n);
     c->d_tags = c->dalloc<int8_t>(n);
-    c->d_status = c->dalloc<int>(1);
-    c->d_lin = c->dalloc<unsigned long long>(2);
+    c->d_status = c->dalloc_zero<int>(1);
+    c->d_lin = c->dalloc_zero<unsigned long long>(2);
     // pinned staging of the topology uploads (keys, six int arrays of n, parent,
     // child0, leaves, level lists, boundary items of 6 n, counts) and of work lists
     if (cudaMallocHost((void**)&c->h_stage, 80 * n + 4 * CNT_SIZE + 256) != cudaSuccess ||
@@ -716,10 +723,7 @@ int mrb_init_blocks(const mrb_config* cfg, void* pool, size_t pool_bytes, mrb_ct
     CK(cudaEventCreateWithFlags(&c->list_ev, cudaEventDisableTiming));
     p.lin_count = c->d_lin;
     p.lmax = c->d_lmax;
-    CK(cudaMemsetAsync(c->d_lin, 0, 2 * sizeof(unsigned long long), c->st));
     CK(cudaMemcpyAsync(c->d_lmax, cfg->lmax, sizeof(int32_t) * cfg->n_instances, cudaMemcpyHostToDevice, c->st));
-    CK(cudaMemsetAsync(c->d_status, 0, sizeof(int), c->st));
-    CK(cudaMemsetAsync(c->d_cnt, 0, sizeof(int32_t) * CNT_SIZE, c->st));
     c->free_slots.clear();
     for (int64_t s = c->nslots - 1; s >= 0; --s) c->free_slots.push_back((int32_t)s);
     for (int inst = 0; inst < cfg->n_instances; ++inst)
