@@ -235,7 +235,9 @@ int mrb_mr_predict_and_tag(mrb_ctx* ctx, int32_t allow_refine, int8_t* tags_dev,
 
 /* Apply tags (device, [n_leaves] int8, leaf order; as from
  * mrb_mr_predict_and_tag or built by the caller): REFINE creates the eight
- * children, each predicted from the parent over its 24^3 stored cells;
+ * children, each predicted from the parent over its 24^3 stored cells (halos
+ * of the parents that do not belong to the present state and tree are filled
+ * first; averages must be current);
  * COARSEN removes a complete sibling group (the parent already holds their
  * average).  Invalid tags (REFINE at lmax, partial COARSEN groups) are
  * ignored.  Rebuilds ids, leaf lists and the 26-neighbour table.

@@ -88,7 +88,10 @@ struct mrb_ctx {
   cudaStream_t cap_st = nullptr;     // private stream for capture (the caller's may be the legacy stream)
   bool graph_dirty = true;
   decltype(h_cnt) cap_cnt;          // the counts that shaped the captured launches
-  bool detail_filled = false;        // stored halos are not complete (fill before the details)
+  // Stored halos of the current buffer against the present state and tree: not kept, the
+  // predicted regions only (as before the details), or all of them (mrb_fill_halos).
+  enum { HALOS_OLD, HALOS_PREDICTED, HALOS_FULL };
+  int halos = HALOS_OLD;
   char* h_stage = nullptr;           // pinned staging of the topology uploads
   int32_t* h_list = nullptr;         // pinned staging of work lists
   cudaEvent_t stage_ev = nullptr, list_ev = nullptr;
@@ -280,6 +283,8 @@ struct mrb_ctx {
     if (mode == FILL_FULL) launch_fill_copies(topo(), P, cur, h_cnt[CNT_NNODES], st);
     for (int l = 1; l <= max_lmax; ++l) launch_predict(topo(), phys, P, cur, l, level_nodes(l), mode, st);
     if (mode == FILL_FULL) launch_fill_bc(topo(), phys, P, cur, st);
+    if (mode == FILL_FULL) halos = HALOS_FULL;
+    else if (mode == FILL_DETAIL && halos == HALOS_OLD) halos = HALOS_PREDICTED;
   }
   // the stage kernels read face neighbours' cells and map boundary cells
   // themselves; the viscous gradients read stored edge cells of the halo
@@ -305,8 +310,10 @@ struct mrb_ctx {
       launch_shadow(topo(), phys, P, cur ^ 1, SH_JUMP, nullptr, 0, 0, st);
     }
     cur ^= 1;
+    halos = HALOS_OLD;
   }
   void project() {
+    if (max_lmax > 0) halos = HALOS_OLD;       // (the internal nodes' cells that halos copy)
     for (int l = max_lmax - 1; l >= 0; --l) launch_project_level(topo(), phys, P, cur, l, st);
   }
   void step_stages() {
@@ -431,8 +438,6 @@ struct mrb_ctx {
 
   int64_t remesh(const int8_t* tags_dev) {
     const int nl = n_leaves();
-    const bool detail_fill = detail_filled;
-    detail_filled = false;
     std::vector<int8_t> tags((size_t)nl);
     if (nl) CK(cudaMemcpyAsync(tags.data(), tags_dev, nl, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
@@ -453,10 +458,10 @@ struct mrb_ctx {
     if ((int64_t)refine.size() * 8 > (int64_t)free_slots.size() + 8 * (int64_t)coarse_parents.size())
       throw Err(MRB_ECAPACITY, "block pool exhausted by refinement");
     if (refine.empty() && coarse_parents.empty()) return nl;
-    if (detail_fill && !refine.empty()) {
-      // the fill before the details computed predicted regions only: complete
-      // the stored halos of the blocks about to be refined, whose children are
-      // predicted over their whole stored range
+    if (!refine.empty() && halos != HALOS_FULL) {
+      // children are predicted over their whole stored range: complete the stored
+      // halos of the blocks about to be refined
+      if (halos == HALOS_OLD) fill_halos(FILL_DETAIL);
       upload_list(refine);
       launch_fill_list(topo(), phys, P, cur, d_list, (int)refine.size(), st);
       list_used();
@@ -495,6 +500,7 @@ struct mrb_ctx {
     }
     std::sort(next.begin(), next.end(), [](const HNode& a, const HNode& b) { return a.key < b.key; });
     nodes.swap(next);
+    halos = HALOS_OLD;
     rebuild();
     if (!newpairs.empty()) {
       std::vector<int32_t> pairs;
@@ -798,6 +804,7 @@ int mrb_set_state(mrb_ctx* c, const uint64_t* keys_host, int64_t n, const double
     if (n < 0 || (n > 0 && (!keys_host || !prim_dev))) throw Err(MRB_EINVAL, "bad arguments");
     std::vector<int32_t> v = c->nodes_of(keys_host, n);
     c->upload_list(v);
+    if (n > 0) c->halos = mrb_ctx::HALOS_OLD;
     launch_set_state(c->topo(), c->phys, c->P, c->cur, c->d_list, (int)n, prim_dev, c->st);
     launch_shadow(c->topo(), c->phys, c->P, c->cur, SH_LIST, c->d_list, (int)n, 1, c->st);
     c->list_used();
@@ -809,6 +816,7 @@ int mrb_set_cons(mrb_ctx* c, const uint64_t* keys_host, int64_t n, const double*
     if (n < 0 || (n > 0 && (!keys_host || !cons_dev))) throw Err(MRB_EINVAL, "bad arguments");
     std::vector<int32_t> v = c->nodes_of(keys_host, n);
     c->upload_list(v);
+    if (n > 0) c->halos = mrb_ctx::HALOS_OLD;
     launch_set_cons(c->topo(), c->phys, c->P, c->cur, c->d_list, (int)n, cons_dev, c->st);
     c->list_used();
   });
@@ -895,7 +903,6 @@ namespace {
 int refine_where(mrb_ctx* c, const std::vector<int8_t>& tags, int64_t* n_leaves) {
   int rc = guarded(c, [&] {
     c->fill_halos();
-    c->detail_filled = false;
     if (!tags.empty()) CK(cudaMemcpyAsync(c->d_tags, tags.data(), tags.size(), cudaMemcpyHostToDevice, c->st));
     int64_t nl = c->remesh(c->d_tags);
     if (n_leaves) *n_leaves = nl;
@@ -944,9 +951,9 @@ int mrb_step(mrb_ctx* c, int32_t nsteps, double* dt_hist_dev) {
         g_kernel_launches += c->graph_kernels[g];
         if (c->phys.rk & 1) c->cur ^= 1;   // every stage flips the stage buffer
       }
+      c->halos = mrb_ctx::HALOS_OLD;
       if (mr) {
         c->fill_halos(FILL_DETAIL);
-        c->detail_filled = true;
         launch_delta_tags(c->topo(), c->phys, c->P, c->cur, c->d_delta_node, 1, c->d_tags, nullptr, c->n_leaves(),
                           c->h_cnt[CNT_NNODES], c->st);
         c->remesh(c->d_tags);

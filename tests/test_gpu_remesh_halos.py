@@ -1,0 +1,96 @@
+"""Refinement by the caller's own tags without a halo fill before it: the same
+tree and states as with one, whatever moved the state or the tree on since the
+halos were last stored."""
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2012_04385_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_2012_04385_gb300 import mrb  # noqa: E402
+
+Z, P, S = I.BC_ZERO_GRADIENT, I.BC_PERIODIC, I.BC_SYMMETRY
+
+
+def _cfg(**kw):
+    # (details stay below this eps: steps keep the tree, of levels 0 and 1)
+    return I.explosion_config(lmax=2, base_blocks=(2, 1, 2), bc=(Z, S, P, P, S, Z), eps=1e9, **kw)
+
+
+def _start(cfg):
+    g = mrb.Context(cfg, 300)
+    keys, geo = g.list_blocks()
+    g.set_state(keys, I.ic_random_smooth(cfg, geo))
+    g.fill_halos()
+    g.remesh((geo[:, 1] == geo[:, 3]).astype(np.int8))
+    keys, geo = g.list_blocks()
+    g.set_state(keys, I.ic_random_smooth(cfg, geo))
+    g.mr_project()
+    g.fill_halos()
+    return g
+
+
+def _tags(geo):
+    return ((geo[:, 0] == 1) & ((geo[:, 1] + geo[:, 2]) % 2 == 0) | (geo[:, 0] == 0) & (geo[:, 1] == 0)).astype(np.int8)
+
+
+def _move(g, what):
+    keys, geo = g.list_blocks()
+    if what == "step":
+        g.step(2)
+    elif what == "stage":
+        g.rk_stage(0, torch.full((1,), 1e-3, dtype=torch.float64, device="cuda"))
+        g.mr_project()
+    elif what == "state":
+        prim = I.ic_random_smooth(g.cfg, geo)
+        prim[:, 0] *= 1.25
+        g.set_state(keys, prim)
+        g.mr_project()
+    else:
+        g.remesh(((geo[:, 0] == 1) & (geo[:, 1] == 1)).astype(np.int8))
+
+
+@pytest.mark.parametrize("what", ["step", "stage", "state", "tree"])
+@pytest.mark.parametrize("kw", [dict(), dict(precision=I.FP32_ACC64), dict(lts=1), dict(precision=I.FP32_ACC64, mu=1e-3)],
+                         ids=["fp64", "fp32", "lts", "viscous"])
+def test_refinement_without_a_fill(kw, what):
+    out = []
+    for fill in (False, True):
+        g = _start(_cfg(**kw))
+        _move(g, what)
+        if fill:
+            g.fill_halos()
+        g.remesh(_tags(g.geometry()))
+        assert g.status() == mrb.MRB_OK
+        nodes = g.keys(leaves_only=False)
+        out.append((nodes, g.get_state(nodes).cpu().numpy()))
+        g.close()
+    assert out[0][0].size > 30 and np.array_equal(out[0][0], out[1][0])
+    assert np.array_equal(out[0][1].view(np.uint64), out[1][1].view(np.uint64))
+
+
+def test_refinement_after_steps_against_oracle():
+    """FP64, bit for bit."""
+    cfg = _cfg()
+    g, o = _start(cfg), oracle.Oracle(cfg)
+    o.set_state(o.keys(), I.ic_random_smooth(cfg, o.geometry()))
+    o.fill_halos()
+    geo = o.geometry()
+    o.remesh((geo[:, 1] == geo[:, 3]).astype(np.int8))
+    o.set_state(o.keys(), I.ic_random_smooth(cfg, o.geometry()))
+    o.project()
+    g.step(2)
+    o.step(2)
+    assert np.array_equal(g.keys(), o.keys())
+    o.fill_halos()
+    o.remesh(_tags(o.geometry()))
+    g.remesh(_tags(g.geometry()))
+    assert np.array_equal(g.keys(), o.keys())
+    assert np.array_equal(g.get_state().cpu().numpy(), o.get_state())
