@@ -171,9 +171,8 @@ int mrb_set_state(mrb_ctx* ctx, const uint64_t* keys_host, int64_t n, const doub
 int mrb_set_cons(mrb_ctx* ctx, const uint64_t* keys_host, int64_t n, const double* cons_dev);
 
 /* Conserved state of the listed blocks into cons_dev: [n][5][16^3] internal
- * cells (with_halo = 0) or [n][5][24^3] stored cells (with_halo = 1; the halos
- * are those of the last mrb_fill_halos, as long as the state has not moved on:
- * stages and steps fill only the predicted regions they read). */
+ * cells (with_halo = 0) or [n][5][24^3] stored cells (with_halo = 1; after a
+ * stage or a step, which keep no stored halos, all halos are filled first). */
 int mrb_get_state(mrb_ctx* ctx, const uint64_t* keys_host, int64_t n, double* cons_dev, int32_t with_halo);
 
 /* FP32 primitive records (rho, u, v, w, p, E) of the internal cells of the

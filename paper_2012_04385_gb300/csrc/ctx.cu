@@ -92,6 +92,9 @@ struct mrb_ctx {
   // predicted regions only (as before the details), or all of them (mrb_fill_halos).
   enum { HALOS_OLD, HALOS_PREDICTED, HALOS_FULL };
   int halos = HALOS_OLD;
+  // No complete fill since the last stage or step: the current buffer's halos may hold that
+  // stage's scratch, and a call that reads them fills what it reads first.
+  bool halos_scratch = true;
   char* h_stage = nullptr;           // pinned staging of the topology uploads
   int32_t* h_list = nullptr;         // pinned staging of work lists
   cudaEvent_t stage_ev = nullptr, list_ev = nullptr;
@@ -283,8 +286,19 @@ struct mrb_ctx {
     if (mode == FILL_FULL) launch_fill_copies(topo(), P, cur, h_cnt[CNT_NNODES], st);
     for (int l = 1; l <= max_lmax; ++l) launch_predict(topo(), phys, P, cur, l, level_nodes(l), mode, st);
     if (mode == FILL_FULL) launch_fill_bc(topo(), phys, P, cur, st);
-    if (mode == FILL_FULL) halos = HALOS_FULL;
-    else if (mode == FILL_DETAIL && halos == HALOS_OLD) halos = HALOS_PREDICTED;
+    if (mode == FILL_FULL) {
+      halos = HALOS_FULL;
+      halos_scratch = false;
+    } else if (mode == FILL_DETAIL && halos == HALOS_OLD) {
+      halos = HALOS_PREDICTED;
+    }
+  }
+  void replace_scratch(int mode) {
+    if (halos_scratch && !(mode == FILL_DETAIL && halos == HALOS_PREDICTED)) fill_halos(mode);
+  }
+  void state_moved() {
+    halos = HALOS_OLD;
+    halos_scratch = true;
   }
   // the stage kernels read face neighbours' cells and map boundary cells
   // themselves; the viscous gradients read stored edge cells of the halo
@@ -310,7 +324,7 @@ struct mrb_ctx {
       launch_shadow(topo(), phys, P, cur ^ 1, SH_JUMP, nullptr, 0, 0, st);
     }
     cur ^= 1;
-    halos = HALOS_OLD;
+    state_moved();
   }
   void project() {
     if (max_lmax > 0) halos = HALOS_OLD;       // (the internal nodes' cells that halos copy)
@@ -826,6 +840,7 @@ int mrb_get_state(mrb_ctx* c, const uint64_t* keys_host, int64_t n, double* cons
   return guarded(c, [&] {
     if (n < 0 || (n > 0 && (!keys_host || !cons_dev))) throw Err(MRB_EINVAL, "bad arguments");
     std::vector<int32_t> v = c->nodes_of(keys_host, n);
+    if (with_halo && n > 0) c->replace_scratch(FILL_FULL);
     c->upload_list(v);
     launch_get_state(c->topo(), c->P, c->cur, c->d_list, (int)n, cons_dev, with_halo ? 1 : 0, c->st);
     c->list_used();
@@ -850,6 +865,7 @@ int mrb_fill_halos(mrb_ctx* c) {
 int mrb_compute_rhs(mrb_ctx* c, double* rhs_dev) {
   return guarded(c, [&] {
     if (!rhs_dev) throw Err(MRB_EINVAL, "null rhs");
+    c->replace_scratch(c->stage_fill());
     if (c->cfg.precision == MRB_FP32_ACC64)
       launch_rhs_rk_f32(c->topo(), c->phys, c->P, c->cur, 0, nullptr, rhs_dev, c->st, c->n_leaves());
     else launch_rhs_rk_f64(c->topo(), c->phys, c->P, c->cur, 0, nullptr, rhs_dev, c->st);
@@ -860,6 +876,7 @@ int mrb_compute_rhs(mrb_ctx* c, double* rhs_dev) {
 int mrb_rk_stage(mrb_ctx* c, int32_t stage, const double* dt_dev) {
   return guarded(c, [&] {
     if (stage < 0 || stage >= c->phys.rk || !dt_dev) throw Err(MRB_EINVAL, "bad stage or dt");
+    c->replace_scratch(c->stage_fill());
     c->stage(stage, dt_dev);
   });
 }
@@ -878,6 +895,7 @@ int mrb_mr_project(mrb_ctx* c) {
 int mrb_mr_predict_and_tag(mrb_ctx* c, int32_t allow_refine, int8_t* tags_dev, double* delta_dev) {
   return guarded(c, [&] {
     if (!tags_dev) throw Err(MRB_EINVAL, "null tags");
+    c->replace_scratch(FILL_DETAIL);
     launch_delta_tags(c->topo(), c->phys, c->P, c->cur, c->d_delta_node, allow_refine ? 1 : 0, tags_dev, delta_dev,
                       c->n_leaves(), c->h_cnt[CNT_NNODES], c->st);
   });
@@ -951,7 +969,7 @@ int mrb_step(mrb_ctx* c, int32_t nsteps, double* dt_hist_dev) {
         g_kernel_launches += c->graph_kernels[g];
         if (c->phys.rk & 1) c->cur ^= 1;   // every stage flips the stage buffer
       }
-      c->halos = mrb_ctx::HALOS_OLD;
+      c->state_moved();
       if (mr) {
         c->fill_halos(FILL_DETAIL);
         launch_delta_tags(c->topo(), c->phys, c->P, c->cur, c->d_delta_node, 1, c->d_tags, nullptr, c->n_leaves(),
@@ -977,8 +995,10 @@ int mrb_face_samples(mrb_ctx* c, float tau_lab, int64_t stride, float* feats_dev
     if (stride < 1 || cap < 0 || (cap > 0 && (!feats_dev || !labels_dev))) throw Err(MRB_EINVAL, "bad arguments");
     const int64_t faces = (int64_t)c->n_leaves() * 3 * 17 * 256;
     const int64_t n = std::min<int64_t>(cap, (faces + stride - 1) / stride);
-    if (n > 0) launch_face_samples(c->topo(), c->phys, c->P, c->cur, tau_lab, stride, feats_dev, labels_dev, where_dev, n,
-                                   c->st);
+    if (n > 0) {
+      c->replace_scratch(FILL_FULL);
+      launch_face_samples(c->topo(), c->phys, c->P, c->cur, tau_lab, stride, feats_dev, labels_dev, where_dev, n, c->st);
+    }
     if (n_out) *n_out = n;
   });
 }
@@ -1038,6 +1058,7 @@ int mrb_sums(mrb_ctx* c, double* sums_dev) {
 int mrb_flux_census(mrb_ctx* c, uint64_t* counts_host) {
   return guarded(c, [&] {
     if (!counts_host) throw Err(MRB_EINVAL, "null counts");
+    c->replace_scratch(FILL_FULL);
     if (!c->d_census) c->d_census = c->dalloc<unsigned long long>(6);
     launch_flux_census(c->topo(), c->phys, c->P, c->cur, c->d_census, c->st);
     CK(cudaMemcpyAsync(counts_host, c->d_census, 6 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->st));

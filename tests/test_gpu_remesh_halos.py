@@ -94,3 +94,38 @@ def test_refinement_after_steps_against_oracle():
     g.remesh(_tags(g.geometry()))
     assert np.array_equal(g.keys(), o.keys())
     assert np.array_equal(g.get_state().cpu().numpy(), o.get_state())
+
+
+READERS = {
+    "state": lambda g: g.get_state(with_halo=True),
+    "rhs": lambda g: g.compute_rhs(),
+    "tags": lambda g: g.mr_predict_and_tag()[1],
+    "census": lambda g: torch.from_numpy(g.flux_census().astype(np.int64)),
+    "samples": lambda g: g.face_samples(stride=7)[0],
+}
+
+
+def _stage(g):
+    g.rk_stage(0, torch.full((1,), 1e-3, dtype=torch.float64, device="cuda"))
+    return g.get_state()
+
+
+@pytest.mark.parametrize("what", ["step", "stage"])
+@pytest.mark.parametrize("kw", [dict(), dict(precision=I.FP32_ACC64), dict(precision=I.FP32_ACC64, mu=1e-3)],
+                         ids=["fp64", "fp32", "viscous"])
+def test_calls_that_read_halos_after_a_stage_or_step(kw, what):
+    """Their results do not depend on a halo fill before them (FP64 stages leave
+    scratch in the stored halos)."""
+    for name, read in list(READERS.items()) + [("next stage", _stage)]:
+        if name == "samples" and "precision" not in kw:
+            continue
+        out = []
+        for fill in (False, True):
+            g = _start(_cfg(**kw))
+            _move(g, what)
+            if fill:
+                g.fill_halos()
+            out.append(read(g).cpu().numpy())
+            assert g.status() == mrb.MRB_OK
+            g.close()
+        assert np.array_equal(out[0].view(np.uint8), out[1].view(np.uint8)), name
