@@ -195,8 +195,8 @@ int mrb_fill_halos(mrb_ctx* ctx);
  * Sec. 2.2: characteristic WENO5-JS, Roe flux with local Lax-Friedrichs
  * fallback per field), with the jump flux correction applied (Sec. 4), into
  * rhs_dev [n_leaves][5][16^3] in leaf order.  Inspection form: the time
- * stepping uses the fused mrb_rk_stage.  Halos must be filled.  (The halo of the
- * other stage buffer is scratch.) */
+ * stepping uses the fused mrb_rk_stage.  Halos must be filled.  (The other stage
+ * buffer, internal cells and halos, is scratch: the state before the current one.) */
 int mrb_compute_rhs(mrb_ctx* ctx, double* rhs_dev);
 
 /* One Runge-Kutta stage (stage = 0 .. rk_stages - 1) on every leaf, fused

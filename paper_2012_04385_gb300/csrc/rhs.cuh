@@ -31,8 +31,9 @@
 // slots used.
 //
 // Scratch.  The differences live in the stage buffer that the stage is about to
-// write: those of x at the cells themselves, those of y and z in its halo,
-// which the next halo fill rewrites.
+// write: those of x at the cells themselves, those of y and z in its halo, which
+// no call reads before a fill rewrites it (the right-hand side alone leaves all
+// three there).
 #pragma once
 
 #include "kernels.cuh"
