@@ -377,14 +377,15 @@ int mrb_get_tune(mrb_ctx* ctx, int32_t* params);
 int mrb_set_tune(mrb_ctx* ctx, const int32_t* params);
 /* Autotuner: times the candidate shapes on the context's current tree (CUDA
  * events on cfg.stream, `reps` repetitions each, after one warm-up) and keeps
- * the fastest: stage waves {1, 2, 4} x item order {0, 1}, then fill CTAs per SM
- * {4, 8, 16} x {2, 4, 8}, then averaging CTAs per SM {4, 8, 16}.  The timed work
+ * the fastest: stage waves {1, 2, 4} x item order {0, 1}, then copy CTAs per SM
+ * {4, 8, 16} on a complete halo fill, prediction CTAs per SM {2, 4, 8} on the fill
+ * that a stage does, averaging CTAs per SM {4, 8, 16}.  The timed work
  * leaves the simulation state unchanged: stage 0 (with the learned selector
  * also stage 1) from the current stage buffer writes only the other buffer and
  * per-step scratch, the halo fill and the averaging recompute what they wrote
  * before.  The selector's face counters (mrb_learned_stats) are reset.
  * times (host, nullable, [6]): default and tuned ms of the stage kernel(s), of
- * one halo fill and of one averaging pass.  Synchronises. */
+ * one complete halo fill and of one averaging pass.  Synchronises. */
 int mrb_autotune(mrb_ctx* ctx, int32_t reps, double* times);
 int mrb_profile_read(mrb_ctx* ctx, double* stage_kernel_ms, int64_t* stage_kernel_launches, int64_t* kernel_launches);
 

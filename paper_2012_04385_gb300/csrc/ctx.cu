@@ -1118,17 +1118,20 @@ int mrb_set_tune(mrb_ctx* c, const int32_t* params) {
 // other stage buffer and the per-step scratch (u^n, face fluxes, decisions,
 // FP32 records of the other buffer); the halo fill of the current buffer;
 // the averaging (the same averages again).  Coordinate search: stage waves
-// and item order, then fill shapes, then averaging shape.
+// and item order, then the copies' shape on a complete fill, the predictions'
+// on the fill of a stage (whose only work they are, viscous runs apart; beside
+// the copies they would hardly show), then the averaging shape.
 int mrb_autotune(mrb_ctx* c, int32_t reps, double* times) {
   return guarded(c, [&] {
     if (reps < 1) throw Err(MRB_EINVAL, "reps < 1");
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
-    const int fmode = c->stage_fill();
+    enum { STAGE, FILL, PROJECT, PREDICT };
+    c->replace_scratch(c->stage_fill());
     launch_cfl(c->topo(), c->phys, c->P, c->cur, c->n_leaves(), c->d_smax, c->d_dt, nullptr, c->d_status, c->st);
     auto run = [&](int what) {
-      if (what == 0) {
+      if (what == STAGE) {
         if (c->cfg.precision == MRB_FP32_ACC64) {
           launch_rhs_rk_f32(c->topo(), c->phys, c->P, c->cur, 0, c->d_dt, nullptr, c->st, c->n_leaves());
           if (c->cfg.recon == MRB_RECON_LEARNED && c->cfg.mlp_weights)
@@ -1136,8 +1139,10 @@ int mrb_autotune(mrb_ctx* c, int32_t reps, double* times) {
         } else {
           launch_rhs_rk_f64(c->topo(), c->phys, c->P, c->cur, 0, c->d_dt, nullptr, c->st);
         }
-      } else if (what == 1) {
-        c->fill_halos(fmode);
+      } else if (what == FILL) {
+        c->fill_halos();
+      } else if (what == PREDICT) {
+        c->fill_halos(c->stage_fill());
       } else {
         c->project();
       }
@@ -1156,27 +1161,35 @@ int mrb_autotune(mrb_ctx* c, int32_t reps, double* times) {
     int32_t best[5] = {c->tune.stage_waves, c->phys.blocked, c->tune.fill_copy, c->tune.fill_pred, c->tune.project};
     const int32_t def[5] = {1, 0, 8, 4, 8};
     double t_def[3], t_best[3];
-    for (int what = 0; what < 3; ++what) t_def[what] = time_of(what, def);
+    for (int what : {STAGE, FILL, PROJECT}) t_def[what] = time_of(what, def);
     std::copy(def, def + 5, best);
-    t_best[0] = t_def[0];
+    t_best[STAGE] = t_def[STAGE];
     for (int w : {1, 2, 4})
       for (int b : {0, 1}) {
         int32_t q[5] = {w, b, best[2], best[3], best[4]};
-        const double tt = time_of(0, q);
-        if (tt < t_best[0]) { t_best[0] = tt; best[0] = w; best[1] = b; }
+        const double tt = time_of(STAGE, q);
+        if (tt < t_best[STAGE]) { t_best[STAGE] = tt; best[0] = w; best[1] = b; }
       }
-    t_best[1] = t_def[1];
-    for (int fc : {4, 8, 16})
+    t_best[FILL] = t_def[FILL];
+    for (int fc : {4, 8, 16}) {
+      int32_t q[5] = {best[0], best[1], fc, best[3], best[4]};
+      const double tt = time_of(FILL, q);
+      if (tt < t_best[FILL]) { t_best[FILL] = tt; best[2] = fc; }
+    }
+    if (c->max_lmax > 0) {                     // (a single level predicts nothing)
+      double t_pred = time_of(PREDICT, best);
       for (int fp : {2, 4, 8}) {
-        int32_t q[5] = {best[0], best[1], fc, fp, best[4]};
-        const double tt = time_of(1, q);
-        if (tt < t_best[1]) { t_best[1] = tt; best[2] = fc; best[3] = fp; }
+        int32_t q[5] = {best[0], best[1], best[2], fp, best[4]};
+        const double tt = time_of(PREDICT, q);
+        if (tt < t_pred) { t_pred = tt; best[3] = fp; }
       }
-    t_best[2] = t_def[2];
+      if (best[3] != def[3]) t_best[FILL] = time_of(FILL, best);
+    }
+    t_best[PROJECT] = t_def[PROJECT];
     for (int pr : {4, 8, 16}) {
       int32_t q[5] = {best[0], best[1], best[2], best[3], pr};
-      const double tt = time_of(2, q);
-      if (tt < t_best[2]) { t_best[2] = tt; best[4] = pr; }
+      const double tt = time_of(PROJECT, q);
+      if (tt < t_best[PROJECT]) { t_best[PROJECT] = tt; best[4] = pr; }
     }
     apply_tune(c, best);
     CK(cudaMemsetAsync(c->d_lin, 0, 2 * sizeof(unsigned long long), c->st));   // the timed launches' selector counts
