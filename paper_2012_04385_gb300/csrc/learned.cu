@@ -465,14 +465,18 @@ extern "C" int mrb_mlp_threshold(const float* logits_dev, const uint8_t* labels_
   KeySelect* S = reinterpret_cast<KeySelect*>(work_dev);
   const int grid = (int)std::min<int64_t>((n + 1023) / 1024, (int64_t)sm_count() * 4);
   if (cudaMemsetAsync(S, 0, sizeof(KeySelect), st) != cudaSuccess) return MRB_ECUDA;
+  // (each launch's own status: an error pending from an earlier call is left alone)
   const int shifts[5] = {25, 18, 12, 6, 0}, widths[5] = {7, 7, 6, 6, 6};
-  for (int d = 0; d < 5; ++d)
-    k_key_select<<<grid, 256, 0, st>>>(logits_dev, labels_dev, n, q, shifts[d], widths[d], S);
-  k_key_next<<<grid, 256, 0, st>>>(logits_dev, labels_dev, n, S);
-  g_kernel_launches += 6;
+  for (int d = 0; d < 6; ++d) {
+    void* select[] = {(void*)&logits_dev, (void*)&labels_dev, (void*)&n, (void*)&q,
+                      (void*)&shifts[d % 5], (void*)&widths[d % 5], (void*)&S};
+    void* next[] = {(void*)&logits_dev, (void*)&labels_dev, (void*)&n, (void*)&S};
+    const void* kernel = d < 5 ? (const void*)k_key_select : (const void*)k_key_next;
+    if (cudaLaunchKernel(kernel, dim3(grid), dim3(256), d < 5 ? select : next, 0, st) != cudaSuccess) return MRB_ECUDA;
+    ++g_kernel_launches;
+  }
   KeySelect h;
-  if (cudaGetLastError() != cudaSuccess ||
-      cudaMemcpyAsync((char*)&h + offsetof(KeySelect, rank), (char*)S + offsetof(KeySelect, rank),
+  if (cudaMemcpyAsync((char*)&h + offsetof(KeySelect, rank), (char*)S + offsetof(KeySelect, rank),
                       sizeof(KeySelect) - offsetof(KeySelect, rank), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess)
     return MRB_ECUDA;

@@ -59,3 +59,20 @@ def test_threshold_equals_the_sorted_order_statistics(kind, n):
             else:
                 scale = max(abs(float(a)), abs(float(d)))
                 assert abs(got - float(want)) <= 4 * 2.0 ** -24 * scale + 1.5e-45, (q, got, want)
+
+
+def test_an_earlier_error_is_left_alone():
+    """An error that another call of the process left pending (a device that does
+    not exist) neither fails the threshold nor is taken by it."""
+    import ctypes
+
+    z = torch.linspace(-1.0, 1.0, 101, device="cuda")
+    y = torch.ones(101, dtype=torch.uint8, device="cuda")
+    work = torch.empty(256, dtype=torch.int64, device="cuda")
+    st = torch.cuda.current_stream().cuda_stream
+    L, out = mrb.lib(), ctypes.c_float()
+    torch.cuda.synchronize()
+    assert L.cudaSetDevice(9999) != 0
+    rc = L.mrb_mlp_threshold(z.data_ptr(), y.data_ptr(), 101, 0.5, work.data_ptr(), ctypes.byref(out), st)
+    left = L.cudaGetLastError()
+    assert rc == mrb.MRB_OK and out.value == z[50].item() and left != 0
