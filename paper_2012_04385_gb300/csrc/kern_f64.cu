@@ -198,33 +198,90 @@ void launch_rhs_rk_f64(const Topo& t, const Phys& p, const Pool& pool, int cur, 
 }
 
 // ---------------------------------------------------------------- fine side of a jump
+// Child of an internal node that covers quarter (ct1, ct2) of its side s.
+__device__ __forceinline__ int side_child(const Topo& t, int node, int s, int ct1, int ct2) {
+  const int d = s / 2, b1 = (d == 0) ? 2 : 1, b2 = (d == 2) ? 2 : 4, bd = (d == 0) ? 1 : (d == 1 ? 2 : 4);
+  return t.child0[node] + ((s & 1) ? bd : 0) + (ct1 ? b1 : 0) + (ct2 ? b2 : 0);
+}
+// Mean of two face cells and the two above them.
+__device__ __forceinline__ double mean4(const double* cf) {
+  const double2 lo = *reinterpret_cast<const double2*>(cf), up = *reinterpret_cast<const double2*>(cf + NB);
+  return 0.25 * ((lo.x + lo.y) + (up.x + up.y));
+}
 // Flux of an internal node's face cell (side s, position aa, bb): the mean of
-// the 2 x 2 covering child face cells, themselves means where the child is
-// refined too.  Formed where a jump reads it; averaging every face of every
-// internal node level by level took a launch per level and 135 us per stage on
-// the shock-bubble, for the few per cent of faces that a jump reads.
-static __device__ __noinline__ double fine_flux(const int32_t* __restrict__ child0, const int32_t* __restrict__ slot,
-                                                const double* __restrict__ faces, int node, int s, int v, int aa, int bb) {
-  const int d = s / 2, hi = s & 1;
+// the 2 x 2 covering child face cells.  Formed where a jump reads it; averaging
+// every face of every internal node level by level took a launch per level and
+// 135 us per stage on the shock-bubble, for the few per cent of faces that a jump
+// reads.
+__device__ __forceinline__ double fine_flux(const Topo& t, const double* faces, int node, int s, int v, int aa, int bb) {
   const int ct1 = aa / 8, ct2 = bb / 8;
-  const int b1 = (d == 0) ? 2 : 1, b2 = (d == 2) ? 2 : 4, bd = (d == 0) ? 1 : (d == 1 ? 2 : 4);
-  const int ch = child0[node] + (hi ? bd : 0) + (ct1 ? b1 : 0) + (ct2 ? b2 : 0);
-  const int fa = 2 * (aa - 8 * ct1), fb = 2 * (bb - 8 * ct2);
-  double f00, f10, f01, f11;
-  if (child0[ch] < 0) {
-    const double* cf = faces + (size_t)slot[ch] * SLOT_F + (s * NV + v) * NFACE + fb * NB + fa;
-    const double2 lo = *reinterpret_cast<const double2*>(cf), up = *reinterpret_cast<const double2*>(cf + NB);
-    f00 = lo.x;
-    f10 = lo.y;
-    f01 = up.x;
-    f11 = up.y;
-  } else {
-    f00 = fine_flux(child0, slot, faces, ch, s, v, fa, fb);
-    f10 = fine_flux(child0, slot, faces, ch, s, v, fa + 1, fb);
-    f01 = fine_flux(child0, slot, faces, ch, s, v, fa, fb + 1);
-    f11 = fine_flux(child0, slot, faces, ch, s, v, fa + 1, fb + 1);
+  const double* cf = faces + (size_t)t.slot[side_child(t, node, s, ct1, ct2)] * SLOT_F + (s * NV + v) * NFACE +
+                     2 * (bb - 8 * ct2) * NB + 2 * (aa - 8 * ct1);
+  return mean4(cf);
+}
+// (children of `node` on its side s are refined)
+__device__ __forceinline__ bool deep_side(const Topo& t, int node, int s) {
+  bool deep = false;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) deep |= t.child0[side_child(t, node, s, q & 1, q >> 1)] >= 0;
+  return deep;
+}
+// Side s of the refined neighbour `top` where leaves two or more levels finer
+// meet the jump (rare: the details of neighbours differ little): the refined
+// children on that side, deepest first, get the means of their own children's
+// fluxes, in their own face buffers, which nothing else uses.  All threads of the
+// CTA; the (up to four) refined children of a node together, as the chain of loads
+// is what a pass lasts.  Only one coarse leaf meets any of these sides.  (One thread
+// per face cell of `top` descending by itself left most threads without work:
+// beside a corner refined six levels deep a right-hand side took 1275 us, now 105;
+// beside a whole side four levels finer 760, now 630.)
+static __device__ __noinline__ void average_side(const Topo& t, double* faces, int top, int s) {
+  int node[MAXL + 1], depth = 0;
+  unsigned todo[MAXL + 1];       // children on the side still to descend into: those with refined children there
+  const int lane = threadIdx.x & 31, g = lane & 15;
+  auto enter = [&](int n) {      // (lanes 4 q .. 4 q + 3 ask the children of child q)
+    const int ch = side_child(t, n, s, (g >> 2) & 1, g >> 3);
+    const bool deep = t.child0[ch] >= 0 && t.child0[side_child(t, ch, s, g & 1, (g >> 1) & 1)] >= 0;
+    const unsigned m = __ballot_sync(0xffffffffu, deep);
+    node[depth] = n;
+    todo[depth] = ((m & 15u) != 0u) | ((m & 0xf0u) ? 2u : 0u) | ((m & 0xf00u) ? 4u : 0u) | ((m & 0xf000u) ? 8u : 0u);
+  };
+  enter(top);
+  while (depth >= 0) {
+    const int n = node[depth];
+    if (todo[depth] != 0u) {
+      const int q = __ffs(todo[depth]) - 1;
+      todo[depth] &= todo[depth] - 1u;
+      ++depth;
+      enter(side_child(t, n, s, q & 1, q >> 1));
+      continue;
+    }
+    // child q by 64 threads, rows of 16 cells 4 i + 0 .. 3 at a time: the lower ones from its
+    // lower children, the upper ones from its upper children
+    const int q = threadIdx.x >> 6, ch = side_child(t, n, s, q & 1, q >> 1);     // (256 threads)
+    if (t.child0[ch] >= 0) {
+      const int a = threadIdx.x & 15, r = (threadIdx.x >> 4) & 3;
+      double* F = faces + (size_t)t.slot[ch] * SLOT_F + s * NV * NFACE + (threadIdx.x & 63);
+      const int in = s * NV * NFACE + 2 * r * NB + 2 * (a & 7);
+      const double* C[2];
+#pragma unroll
+      for (int up = 0; up < 2; ++up) C[up] = faces + (size_t)t.slot[side_child(t, ch, s, a >> 3, up)] * SLOT_F + in;
+#pragma unroll
+      for (int up = 0; up < 2; ++up) {
+        double x[2][NV];
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+#pragma unroll
+          for (int v = 0; v < NV; ++v) x[k][v] = mean4(C[up] + v * NFACE + 8 * k * NB);
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+#pragma unroll
+          for (int v = 0; v < NV; ++v) F[v * NFACE + 64 * (2 * up + k)] = x[k][v];
+      }
+    }
+    __syncthreads();
+    --depth;
   }
-  return 0.25 * ((f00 + f10) + (f01 + f11));
 }
 
 // ---------------------------------------------------------------- local time stepping
@@ -343,7 +400,7 @@ void launch_lts_fmac(const Topo& t, const Phys& p, const Pool& pool, int level, 
 
 // u += (F_c - F_f)/dx on an upper face, (F_f - F_c)/dx on a lower one, with the
 // integrated fluxes of the leaf and of its refined same-level neighbour.
-__global__ void k_lts_reflux(Topo t, Phys p, Pool pool, int cur) {
+__global__ void __launch_bounds__(256, 4) k_lts_reflux(Topo t, Phys p, Pool pool, int cur) {
   const int nitems = t.cnt[CNT_JUMP];
   for (int w = blockIdx.x; w < nitems; w += gridDim.x) {
     const int li = t.jump[w] >> 6, mask = t.jump[w] & 63;
@@ -360,6 +417,7 @@ __global__ void k_lts_reflux(Topo t, Phys p, Pool pool, int cur) {
       if (!((mask >> s) & 1)) continue;
       const int nb = t.nbr[(size_t)node * 27 + r];
       const int so = s ^ 1;
+      if (deep_side(t, nb, so)) average_side(t, pool.fmac, nb, so);
       const int t1 = (d == 0) ? 1 : 0, t2 = (d == 2) ? 1 : 2;
       for (int e = threadIdx.x; e < NFACE; e += blockDim.x) {
         const int aa = e % 16, bb = e / 16;
@@ -370,7 +428,7 @@ __global__ void k_lts_reflux(Topo t, Phys p, Pool pool, int cur) {
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
           const double Fc = Fc_all[(s * NV + v) * NFACE + e];
-          const double Ff = fine_flux(t.child0, t.slot, pool.fmac, nb, so, v, aa, bb);
+          const double Ff = fine_flux(t, pool.fmac, nb, so, v, aa, bb);
           const double dU = div64(hi ? Fc - Ff : Ff - Fc, dx);
           double& ur = U[v * NCELL + sidx(c[0], c[1], c[2])];
           ur = ur + dU;
@@ -391,8 +449,8 @@ void launch_lts_reflux(const Topo& t, const Phys& p, const Pool& pool, int cur, 
 // flux: dL = (F_c - F_f)/dx on an upper face, (F_f - F_c)/dx on a lower one,
 // applied to the stage result as u += b_s (dt dL) (or added to L in the
 // inspection form), sides x-, x+, y-, y+, z-, z+ in order.
-__global__ void k_jump(Topo t, Phys p, Pool pool, int target, int stage, const double* __restrict__ dt,
-                       double* __restrict__ rhs_out) {
+__global__ void __launch_bounds__(256, 4) k_jump(Topo t, Phys p, Pool pool, int target, int stage,
+                                                 const double* __restrict__ dt, double* __restrict__ rhs_out) {
   const int nitems = t.cnt[CNT_JUMP];
   for (int w = blockIdx.x; w < nitems; w += gridDim.x) {
     const int li = t.jump[w] >> 6, mask = t.jump[w] & 63;
@@ -411,6 +469,7 @@ __global__ void k_jump(Topo t, Phys p, Pool pool, int target, int stage, const d
       if (!((mask >> s) & 1)) continue;      // the side's neighbour is not refined
       const int nb = t.nbr[(size_t)node * 27 + r];
       const int so = s ^ 1;
+      if (deep_side(t, nb, so)) average_side(t, pool.face, nb, so);
       const int t1 = (d == 0) ? 1 : 0, t2 = (d == 2) ? 1 : 2;
       for (int e = threadIdx.x; e < NFACE; e += blockDim.x) {
         const int aa = e % 16, bb = e / 16;
@@ -421,7 +480,7 @@ __global__ void k_jump(Topo t, Phys p, Pool pool, int target, int stage, const d
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
           const double Fc = Fc_all[(s * NV + v) * NFACE + e];
-          const double Ff = fine_flux(t.child0, t.slot, pool.face, nb, so, v, aa, bb);
+          const double Ff = fine_flux(t, pool.face, nb, so, v, aa, bb);
           const double dL = div64(hi ? Fc - Ff : Ff - Fc, dx);
           if (rhs_out) {
             double& Lr = rhs_out[((size_t)li * NV + v) * NINT + iidx(c[0], c[1], c[2])];
