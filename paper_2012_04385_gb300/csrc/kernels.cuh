@@ -182,8 +182,12 @@ void launch_rhs_rk_f32(const Topo& t, const Phys& p, const Pool& pool, int cur, 
                        double* rhs_out, cudaStream_t st, int n_nodes, int level = -1);
 // The same on slabs of two planes (n_nodes: the leaves, or the nodes of `level`).
 // Taken while all their slabs are resident at two CTAs per SM: the stage then lasts as
-// long as one item, 15 us instead of 23 on the Sod tube's 8 blocks; on blocks that vary
-// everywhere a step of 36 takes 115 us, one of 39 (slabs of four) 178.
+// long as one item, 15 us instead of 23 on the Sod tube's 8 blocks.  Beyond that the
+// two forms differ by how their last rounds fill.  Microseconds of a single-level step
+// of 38 / 39 / 48 / 56 / 76 / 90 / 114 / 152 leaves that vary everywhere: thin 95 / 140
+// / 141 / 170 / 174 / 213 / 255 / 336, slabs of four 152 / 152 / 154 / 154 / 155 / 233 /
+// 292 / 303; that vary along one direction: thin 65 / 98 / 86 / 110 / 111 / 141 / 159 /
+// 211, slabs of four 96 / 96 / 82 / 97 / 98 / 148 / 180 / 192.
 void launch_rhs_rk_f32_thin(const Topo& t, const Phys& p, const Pool& pool, int cur, int stage, const double* dt,
                             double* rhs_out, cudaStream_t st, int level = -1);
 // FP32 stage kernels of the flux variants (separate translation units):
