@@ -409,6 +409,7 @@ struct mrb_ctx {
     return false;
   }
   void capture_graphs() {
+    graph_dirty = true;                // until both are there
     for (int g = 0; g < 2; ++g) {
       if (graph[g]) cudaGraphExecDestroy(graph[g]);
       graph[g] = nullptr;

@@ -22,7 +22,7 @@ enum : int { ST_OK = 0, ST_NONPHYS = 6 };
 
 // Halo fill modes.  A halo cell facing a same-level node is that node's internal
 // cell, and one beyond a non-periodic boundary is a mapped cell, so the kernels
-// of a step read those where they are (mr.cuh, HaloSrc) and only predicted
+// of a step read those where they are (mr.cuh, region_base and bc_map) and only predicted
 // regions, which exist nowhere else, are ever computed for them:
 //   FILL_FULL       every region of every node in its stored halo (mrb_fill_halos,
 //                   and the stages with viscous terms, which read edges);
