@@ -92,8 +92,9 @@ struct mrb_ctx {
   // predicted regions only (as before the details), or all of them (mrb_fill_halos).
   enum { HALOS_OLD, HALOS_PREDICTED, HALOS_FULL };
   int halos = HALOS_OLD;
-  // No complete fill since the last stage or step: the current buffer's halos may hold that
-  // stage's scratch, and a call that reads them fills what it reads first.
+  // No complete fill since the last stage or step (or since a remesh filled some halos of a
+  // new state): the current buffer's halos may hold that stage's scratch, and a call that
+  // reads them fills what it reads first.
   bool halos_scratch = true;
   char* h_stage = nullptr;           // pinned staging of the topology uploads
   int32_t* h_list = nullptr;         // pinned staging of work lists
@@ -476,7 +477,10 @@ struct mrb_ctx {
     if (!refine.empty() && halos != HALOS_FULL) {
       // children are predicted over their whole stored range: complete the stored
       // halos of the blocks about to be refined
-      if (halos == HALOS_OLD) fill_halos(FILL_DETAIL);
+      if (halos == HALOS_OLD) {
+        fill_halos(FILL_DETAIL);
+        halos_scratch = true;
+      }
       upload_list(refine);
       launch_fill_list(topo(), phys, P, cur, d_list, (int)refine.size(), st);
       list_used();

@@ -129,3 +129,18 @@ def test_calls_that_read_halos_after_a_stage_or_step(kw, what):
             assert g.status() == mrb.MRB_OK
             g.close()
         assert np.array_equal(out[0].view(np.uint8), out[1].view(np.uint8)), name
+
+
+@pytest.mark.parametrize("precision", [I.FP64, I.FP32_ACC64])
+def test_stored_halos_after_a_refinement_without_a_fill(precision):
+    """Halos of one state throughout: those of a complete fill after the remesh."""
+    out = []
+    for fill in (False, True):
+        g = _start(_cfg(precision=precision))
+        _move(g, "state")
+        g.remesh(_tags(g.geometry()))
+        if fill:
+            g.fill_halos()
+        out.append(g.get_state(with_halo=True).cpu().numpy())
+        g.close()
+    assert np.array_equal(out[0].view(np.uint64), out[1].view(np.uint64))
